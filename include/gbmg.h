@@ -74,8 +74,9 @@ typedef struct {
   int nu2;            /* post-smoothing sweeps, default 2 */
   int max_iter;       /* V-cycle limit, default 50 */
   int precision;      /* MG_PREC_F64 (default) or MG_PREC_MIXED */
-  int smoother;       /* MG_SMOOTH_AUTO (default): the fused red + black sweep on FP32 levels
-                         of at least 256^3 cells, half-sweeps elsewhere; _HALF: half-sweeps
+  int smoother;       /* MG_SMOOTH_AUTO (default): whole red + black sweeps on FP32 levels (on
+                         regular box grids from 2^14 cells, 2^18 together in a batch; on others
+                         from 256^3), half-sweeps elsewhere; _HALF: half-sweeps
                          everywhere; _FUSED: the fused sweep on every level but the bottom
                          (the caller's FP64 level 0 then needs phi nghost >= 2, rhs >= 1).
                          All three give the same results. */

@@ -116,6 +116,19 @@ struct UnitB {
     rhs_smem = rhs_smem && t.rhs_smem;
   }
 };
+// Whole sweeps of one level of several solves, phi -> phi2 and back (the same tiling).
+struct SweepB {
+  std::vector<SweepGrid> ab, ba;
+  SweepPlan plan;
+  size_t off_ab = 0, off_ba = 0;
+  void add(const LevelData& D) {
+    ab.push_back(D.sweep_ab);
+    ba.push_back(D.sweep_ba);
+  }
+  void finish() {
+    if (!ab.empty()) plan = plan_sweep(ab, ba);
+  }
+};
 struct JobB {
   std::vector<BottomJob> v;
   int maxN = 0;
@@ -142,6 +155,7 @@ struct LevelLists {
   TagB fill1_half, fill1_all, fill2_phi, fill2_phi2, fill_rhs;
   TagB fill_c;    // the coarse level's phi, one layer, before the trilinear prolongation
   UnitB fab, fba;
+  SweepB sweep;
   JobB bottom_next;      // bottoms at level l + 1
   CoarseB coarse_next;   // coarse cycles from level l + 1
 };
@@ -200,6 +214,11 @@ void build_lists(Ctx& c, StepLists& S, const std::vector<Member*>& run,
   size_t Lmax = 0;
   for (Member* m : run) Lmax = std::max(Lmax, m->H->L.size());
   S.L.assign(Lmax > 0 ? Lmax : 1, LevelLists{});
+  // levels swept whole: the launch covers enough cells of the members' wide levels
+  std::vector<long long> wide(S.L.size(), 0);
+  for (Member* m : run)
+    for (int l = 0; l + 1 < (int)m->H->L.size() && l < m->H->lc; ++l)
+      if (m->H->L[l].wide) wide[l] += m->H->L[l].cells();
   for (Member* m : run) {
     Hierarchy& H = *m->H;
     S.dt = H.dt;
@@ -219,6 +238,8 @@ void build_lists(Ctx& c, StepLists& S, const std::vector<Member*>& run,
         LL.fill2_phi.add(fill_plan(c, *D.phi, &H.bc, 2), D.phi->base);
         LL.fill2_phi2.add(fill_plan(c, *D.phi2, &H.bc, 2), D.phi2->base);
         LL.fill_rhs.add(fill_plan(c, *D.rhs, &H.bc, 1), D.rhs->base);
+      } else if (D.wide && wide[l] >= kSweepMinCellsBatch) {
+        LL.sweep.add(D);
       } else {
         LL.half.add(D.smooth, m->slot);
         if (!D.direct) LL.fill1_half.add(fill_plan(c, *D.phi, &H.bc, 1), D.phi->base);
@@ -241,6 +262,7 @@ void build_lists(Ctx& c, StepLists& S, const std::vector<Member*>& run,
       S.correct0.add(H.correct0, m->slot);
     }
   }
+  for (LevelLists& LL : S.L) LL.sweep.finish();
   for (Member* m : check) {
     S.resid0.add(m->H->resid0, m->slot);
     if (!m->H->direct0) S.fill_phi0.add(fill_plan(c, *m->H->phi0, &m->H->bc, 1), m->H->phi0->base);
@@ -260,6 +282,8 @@ void upload_lists(Ctx& c, StepLists& S, Staging& st, cudaStream_t s) {
     tag(LL.fill1_half); tag(LL.fill1_all); tag(LL.fill2_phi); tag(LL.fill2_phi2); tag(LL.fill_rhs);
     tag(LL.fill_c);
     unit(LL.fab); unit(LL.fba);
+    LL.sweep.off_ab = st.push(LL.sweep.ab);
+    LL.sweep.off_ba = st.push(LL.sweep.ba);
     job(LL.bottom_next);
     cjob(LL.coarse_next);
   }
@@ -293,6 +317,9 @@ void smooth_l(Ctx& c, StepLists& S, LevelLists& LL, int sweeps, const unsigned c
       MG_CK(launch_rbgs_fused_l(S.dt, mk(LL.fba, dev), LL.fba.total, LL.fba.ty, LL.fba.depth,
                                 LL.fba.mp, LL.fba.mpr, LL.fba.rhs_smem, err, s));
     }
+    if (LL.sweep.plan.tiles)
+      for (size_t off : {LL.sweep.off_ab, LL.sweep.off_ba})
+        MG_CK(launch_sweep_f32((const SweepGrid*)(dev + off), (int)LL.sweep.ab.size(), LL.sweep.plan, s));
     if (LL.half.total)
       for (int j = 0; j < 2; ++j)
         for (int color = 0; color < 2; ++color) {

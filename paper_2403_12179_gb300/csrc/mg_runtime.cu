@@ -280,7 +280,7 @@ FaceReads direct_neighbours(const FabObj& f, const int periodic[3], bool outside
   const BoxArray& ba = f.ba->ba;
   const FabLayout& lay = f.lay;
   const size_t nb = ba.boxes.size();
-  if (nb == 0 || lay.g < 1) return out;
+  if (nb == 0) return out;  // (a layout without ghosts works too: only differences are taken)
   // an odd periodic extent makes a boundary cell's periodic neighbour a cell of its own
   // colour, which a half-sweep may be updating at the same time: read filled ghosts there
   for (int d = 0; d < 3; ++d)

@@ -79,6 +79,20 @@ void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
     }, s);
     D.smooth.direct = D.direct;
     D.zero = make_table(c, ba, 0, D.h, 0, [&](int b, DRow& R) { R.v[0] = D.phi->view(b); }, s);
+    if (D.wide) {
+      D.sweep_ab.src = (const float*)D.phi->base;
+      D.sweep_ab.rhs = (const float*)D.rhs->base;
+      D.sweep_ab.dst = (float*)D.phi2->base;
+      D.sweep_ba = D.sweep_ab;
+      D.sweep_ba.src = (const float*)D.phi2->base;
+      D.sweep_ba.dst = (float*)D.phi->base;
+      if (D.cells() >= kSweepMinCells) {
+        std::vector<SweepGrid> ab{D.sweep_ab}, ba{D.sweep_ba};
+        D.sweep_plan = plan_sweep(ab, ba);
+        ab.push_back(ba[0]);
+        D.sweep_dev = c.upload(ab.data(), ab.size() * sizeof(SweepGrid), s);
+      }
+    }
     if (D.fused) {
       D.f_ab = make_fused(c, ba, D.h, *D.phi, *D.rhs, *D.phi2, per, s);
       D.f_ba = make_fused(c, ba, D.h, *D.phi2, *D.rhs, *D.phi, per, s);
@@ -291,11 +305,19 @@ Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, cons
       if (p.smoother == MG_SMOOTH_FUSED && want_fused && !D.fused)
         fail(MG_EINVAL, "fused smoother needs phi nghost >= 2 and rhs nghost >= 1");
     } else {
-      D.phi = internal_fab(c, D.bao, want_fused ? 2 : 1, H->dt);
-      D.rhs = internal_fab(c, D.bao, want_fused ? 1 : 0, H->dt);
-      D.fused = want_fused;
+      // FP32 levels on regular box grids: no ghost cells at all (every stencil reads the
+      // neighbouring boxes), and whole sweeps where a launch covers enough cells
+      if (l + 1 < nl && H->dt == DT_F32 && p.smoother == MG_SMOOTH_AUTO && p.direct_reads &&
+          p.prolong == MG_PROLONG_CONSTANT) {
+        int per[3];
+        bc_code(bc, per);
+        D.wide = sweep_geometry(D.bao->ba, make_layout(D.bao->ba, 1, 0, 4), per, D.h, &D.sweep_ab);
+      }
+      D.fused = want_fused && !D.wide;
+      D.phi = internal_fab(c, D.bao, D.wide ? 0 : D.fused ? 2 : 1, H->dt);
+      D.rhs = internal_fab(c, D.bao, D.fused ? 1 : 0, H->dt);
     }
-    if (D.fused) D.phi2 = internal_fab(c, D.bao, D.phi->lay.g, H->dt);
+    if (D.fused || D.wide) D.phi2 = internal_fab(c, D.bao, D.phi->lay.g, H->dt);
   }
   if (H->mixed) H->r0 = internal_fab(c, phi.ba, 0, DT_F64);
   build_tables(c, *H, s);
@@ -381,6 +403,14 @@ void smooth(Ctx& c, Hierarchy& H, LevelData& D, int sweeps, cudaStream_t s,
             unsigned long long* last_norm = nullptr, bool time_first = false,
             bool skip_first_red = false, bool store_last = false) {
   int k = 0;
+  if (D.sweep_plan.tiles) {
+    // pairs of sweeps: phi -> phi2 -> phi
+    const SweepGrid* g = (const SweepGrid*)D.sweep_dev->p;
+    for (; k + 1 < sweeps; k += 2) {
+      MG_CK(launch_sweep_f32(g, 1, D.sweep_plan, s));
+      MG_CK(launch_sweep_f32(g + 1, 1, D.sweep_plan, s));
+    }
+  }
   if (D.fused) {
     // pairs of fused sweeps: phi -> phi2 -> phi
     for (; k + 1 < sweeps; k += 2) {

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "mg_runtime.hpp"
+#include "mg_sweep.hpp"
 
 namespace gbmg {
 
@@ -13,8 +14,15 @@ struct LevelData {
   OpTable smooth, rr, prolong, zero;
   // the stencil tables read neighbouring boxes directly (no ghost fill before them)
   bool direct = false;
-  // fused sweeps ping-pong between phi and phi2 (same layout)
+  // sweeps ping-pong between phi and phi2 (same layout): fused (mg_fused.cu, ghost cells) or,
+  // on FP32 levels over regular box grids, wide (mg_sweep.cu, neighbouring boxes read directly,
+  // no ghost cells) -- where a launch covers enough cells, else the level's half-sweeps
   bool fused = false;
+  bool wide = false;
+  SweepGrid sweep_ab{}, sweep_ba{};  // phi -> phi2, phi2 -> phi (geometry and pointers)
+  DevBufP sweep_dev;                 // both, tiled for a launch of their own
+  SweepPlan sweep_plan{};            // no tiles: too small for a launch of its own
+  long long cells() const { return bao->ba.dom.npts(); }
   std::shared_ptr<FabObj> phi2;
   FusedTable f_ab, f_ba;
 };
