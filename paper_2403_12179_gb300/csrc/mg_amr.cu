@@ -420,10 +420,11 @@ void enqueue_residual(Ctx& c, AmrPlan& P, cudaStream_t s) {
   unsigned long long* dn = (unsigned long long*)P.dnorm->p;
   fill_fine(c, P, *f0, *f1, s);
   MG_CK(launch_residual(DT_F64, P.fine_resid.rows(), P.fine_resid.nbox, P.fine_resid.nrows,
-                        nullptr, s, P.fine_direct));
+                        nullptr, s, P.fine_direct, -1, P.fine_resid.ext));
   if (!P.coarse_direct) launch_fill(c, *f0, &P.bc, s, 1);
   MG_CK(launch_residual(DT_F64, P.coarse_resid.rows(), P.coarse_resid.nbox,
-                        P.coarse_resid.nrows, nullptr, s, P.coarse_direct));
+                        P.coarse_resid.nrows, nullptr, s, P.coarse_direct, -1,
+                        P.coarse_resid.ext));
   if (P.nrf) {
     launch_k(k_reflux, (P.nrf + 255) / 256, 256, 0, s, (const RefluxCell*)P.rf->p, P.nrf,
                                                   (double*)r0->base, (const double*)f0->base,
@@ -572,7 +573,7 @@ int mg_amr2_solve(mg_ctx_t h, mg_fab_t rhs0, mg_fab_t phi0, mg_fab_t rhs1, mg_fa
             fill_fine(*c, P, *f0, *f1, s);
             MG_CK(launch_rbgs_half(DT_F64, P.fine_smooth.rows(), P.fine_smooth.nbox,
                                    P.fine_smooth.nrows, color, s, P.fine_direct, nullptr,
-                                   P.fine_smooth.width));
+                                   P.fine_smooth.width, false, P.fine_smooth.ext));
           }
         MG_CK(launch_restrict(DT_F64, P.avg_down.rows(), P.avg_down.nbox, P.avg_down.nrows, s));
         enqueue_residual(*c, P, s);

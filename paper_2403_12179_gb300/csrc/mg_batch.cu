@@ -64,9 +64,14 @@ struct SegB {
   long long total = 0;
   size_t off = 0;
   bool direct = false;  // some member's rows carry box-face reads
-  int width = 0;
+  int width = 0, nbox = 0;
+  BoxExtents ext;
   void add(const OpTable& t, int slot) {
     if (!t.nrows) return;
+    const bool first = v.empty();
+    ext.ok = (first || ext.ok) && t.ext.ok && nbox + t.nbox <= kMarchMaxBoxes;
+    ext.even = (first || ext.even) && t.ext.even;
+    for (int d = 0; d < 3; ++d) ext.n[d] = std::max(ext.n[d], t.ext.n[d]);
     direct = direct || t.direct;
     width = std::max(width, t.width);
     Seg s{};
@@ -75,8 +80,10 @@ struct SegB {
     s.row_count = t.nrows;
     s.nbox = t.nbox;
     s.slot = slot;
+    s.box_begin = nbox;
     v.push_back(s);
     total += t.nrows;
+    nbox += t.nbox;
   }
 };
 struct TagB {
@@ -187,6 +194,8 @@ SegList mk(const SegB& b, const unsigned char* dev) {
   SegList L{};
   L.n = (int)b.v.size();
   L.width = b.width;
+  L.nbox = b.nbox;
+  L.ext = b.ext;
   if (L.n == 1) L.one = b.v[0];
   else L.segs = (const Seg*)(dev + b.off);
   return L;

@@ -1078,6 +1078,10 @@ cudaError_t launch_rbgs_half_l(int dt, const SegList& L, long long nrows, int co
   if (nrows <= 0) return cudaSuccess;
   if (norms && (L.n != 1 || !direct)) return cudaErrorInvalidValue;
   if (pre && !norms) return cudaErrorInvalidValue;
+  // FP64 boxes of even width march through their planes (mg_march.cu: 256^3 130 -> 88 us); the
+  // row kernel below is for the others and FP32
+  if (dt == DT_F64 && L.ext.ok && L.ext.even)
+    return launch_half_march(L, norms ? (pre ? 2 : 1) : 0, color, norms, s);
   // a line of w cells holds w / 2 of one colour; two per lane (four on FP32 rows of 64 to
   // 127 cells)
   const bool quad = dt == DT_F32 && !norms && L.width >= 64 && L.width < 128;
@@ -1108,6 +1112,8 @@ cudaError_t launch_rbgs_half_l(int dt, const SegList& L, long long nrows, int co
 cudaError_t launch_residual_l(int dt, const SegList& L, long long nrows, unsigned long long* norms,
                               cudaStream_t s, bool direct, int color) {
   if (nrows <= 0) return cudaSuccess;
+  if (dt == DT_F64 && color < 0 && L.ext.ok)  // (256^3: 238 -> 182 us)
+    return launch_residual_march(L, norms, s);
   Grid g = row_grid(nrows, 16);
   GB_DISPATCH_D(dt, direct, k_residual, g.blocks, kThreads, 0, s, L, nrows, g.per, norms, color);
   count_launches(1);
@@ -1254,8 +1260,8 @@ cudaError_t launch_correct_add_l(const SegList& L, long long nrows, const unsign
 
 cudaError_t launch_rbgs_half(int dt, const DRow* rows, int nbox, long long nrows, int color,
                              cudaStream_t s, bool direct, unsigned long long* norms, int width,
-                             bool pre) {
-  return launch_rbgs_half_l(dt, one_seg(rows, nbox, 0, width), nrows, color, s, direct, norms, pre);
+                             bool pre, const BoxExtents& ext) {
+  return launch_rbgs_half_l(dt, one_seg(rows, nbox, 0, width, ext), nrows, color, s, direct, norms, pre);
 }
 
 cudaError_t launch_restore_colour(int dt, const DRow* rows, int nbox, long long nrows, int color,
@@ -1268,8 +1274,9 @@ cudaError_t launch_restore_colour(int dt, const DRow* rows, int nbox, long long 
 }
 
 cudaError_t launch_residual(int dt, const DRow* rows, int nbox, long long nrows,
-                            unsigned long long* norms, cudaStream_t s, bool direct, int color) {
-  return launch_residual_l(dt, one_seg(rows, nbox), nrows, norms, s, direct, color);
+                            unsigned long long* norms, cudaStream_t s, bool direct, int color,
+                            const BoxExtents& ext) {
+  return launch_residual_l(dt, one_seg(rows, nbox, 0, 0, ext), nrows, norms, s, direct, color);
 }
 
 cudaError_t launch_residual_restrict(int dt, const DRow* rows, int nbox, long long nrows,
@@ -1278,9 +1285,10 @@ cudaError_t launch_residual_restrict(int dt, const DRow* rows, int nbox, long lo
 }
 
 cudaError_t launch_rbgs_half_store(const DRow* rows, int nbox, long long nrows, int color,
-                                   cudaStream_t s, int width) {
+                                   cudaStream_t s, int width, const BoxExtents& ext) {
   if (nrows <= 0) return cudaSuccess;
-  const SegList L = one_seg(rows, nbox, 0, width);
+  const SegList L = one_seg(rows, nbox, 0, width, ext);
+  if (ext.ok && ext.even) return launch_half_march(L, 3, color, nullptr, s);
   const int G = group_lanes(L.width, 4, 8, 16);
   const Grid g = row_grid(nrows, row_blocks_per_sm(L.width), kWarps * (32 / G));
   rbgs_half_norm_g<double, 3>(G, g, s, L, nrows, color, nullptr);

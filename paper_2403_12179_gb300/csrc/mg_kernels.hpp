@@ -106,6 +106,14 @@ __host__ __device__ inline int tag_chunk_rows(int ex, int ncomp, int esize = 8) 
   return ex >= cells ? 1 : cells / ex;
 }
 
+// Largest box extents of a table, for the kernels that march through the planes of a box
+// (mg_march.cu); ok if every box's x extent is at most kMarchMaxX (and there are no more boxes
+// than a grid dimension holds), even if they are all even too.
+constexpr int kMarchMaxX = 256, kMarchMaxBoxes = 65535;
+struct BoxExtents {
+  int n[3] = {0, 0, 0};
+  bool ok = false, even = false;
+};
 // A launch may cover the box tables of several independent solves (batched and served
 // solves): each solve's table is one segment of the launch's row space.  norms and scales
 // of a row live at index slot + DRow::solve.
@@ -115,6 +123,8 @@ struct Seg {
   long long row_count;  // rows of this segment (0: the launch's row count)
   int nbox;
   int slot;
+  int box_begin;        // first box of this segment in the launch
+  int pad_;
 };
 struct SegList {
   const Seg* segs;  // device array, used when n > 1
@@ -122,8 +132,11 @@ struct SegList {
   int n;
   int width;        // host hint: widest box x-extent (cells) in the launch, 0 = unknown; the
                     // launchers size the lane groups of narrow rows from it
+  int nbox;         // boxes of all segments
+  BoxExtents ext;   // over all segments
 };
-inline SegList one_seg(const DRow* rows, int nbox, int slot = 0, int width = 0) {
+inline SegList one_seg(const DRow* rows, int nbox, int slot = 0, int width = 0,
+                       const BoxExtents& ext = {}) {
   SegList L{};
   L.one.rows = rows;
   L.one.row_begin = 0;
@@ -131,6 +144,8 @@ inline SegList one_seg(const DRow* rows, int nbox, int slot = 0, int width = 0) 
   L.one.slot = slot;
   L.n = 1;
   L.width = width;
+  L.nbox = nbox;
+  L.ext = ext;
   return L;
 }
 
@@ -223,7 +238,8 @@ cudaError_t launch_copy_tags(int dt, const DTag* tags, const int2* chunks, int n
 // launch_restore_colour can undo the half-sweep.
 cudaError_t launch_rbgs_half(int dt, const DRow* rows, int nbox, long long nrows, int color,
                              cudaStream_t s, bool direct = false,
-                             unsigned long long* norms = nullptr, int width = 0, bool pre = false);
+                             unsigned long long* norms = nullptr, int width = 0, bool pre = false,
+                             const BoxExtents& ext = {});
 // v[0] = phi, v[2] = saved values (one-colour view): cells of colour `color` take their
 // saved values back.
 cudaError_t launch_restore_colour(int dt, const DRow* rows, int nbox, long long nrows, int color,
@@ -234,7 +250,9 @@ cudaError_t launch_restore_colour(int dt, const DRow* rows, int nbox, long long 
 // every cell; 0 / 1: the cells of that colour only.
 cudaError_t launch_residual(int dt, const DRow* rows, int nbox, long long nrows,
                             unsigned long long* norms, cudaStream_t s, bool direct = false,
-                            int color = -1);
+                            int color = -1, const BoxExtents& ext = {});
+// The same (FP64, every cell) marching through planes (mg_march.cu); norms may be null.
+cudaError_t launch_residual_march(const SegList& L, unsigned long long* norms, cudaStream_t s);
 
 // Rows are coarse x-lines.  v[0] = phi, v[1] = rhs (fine); c[0] = coarse rhs,
 // c[1] = coarse phi (p == null: not zeroed).  stored (FP64, direct): the fine cells of colour
@@ -246,7 +264,11 @@ cudaError_t launch_residual_restrict(int dt, const DRow* rows, int nbox, long lo
 // residual of every cell it updates just after its update (the values a residual pass would
 // compute next).
 cudaError_t launch_rbgs_half_store(const DRow* rows, int nbox, long long nrows, int color,
-                                   cudaStream_t s, int width);
+                                   cudaStream_t s, int width, const BoxExtents& ext = {});
+// The half-sweep (FP64) marching through planes (mg_march.cu); mode 0: plain, 1: norms
+// after the update, 2: norms and values before it, 3: residuals after it.
+cudaError_t launch_half_march(const SegList& L, int mode, int color, unsigned long long* norms,
+                              cudaStream_t s);
 
 // Rows are coarse x-lines.  v[0] = fine field; c[0] = coarse field.
 cudaError_t launch_restrict(int dt, const DRow* rows, int nbox, long long nrows, cudaStream_t s);

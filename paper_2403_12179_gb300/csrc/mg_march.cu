@@ -1,0 +1,432 @@
+// FP64 half-sweep and residual that march through the planes of a box (sm_103a).
+//
+// What bounds these kernels is the FP64 pipe: GB300 issues 1.68 FP64 lanes per clock and SM, so 7
+// FP64 instructions a cell at 100% of it take 111 us for a half-sweep and 222 us for a residual of
+// 256^3 cells, against 56 us and 60 us for their bytes at the copy rate.  Two things take them below
+// that:
+//   * a thread owns a pair of cells in x and marches in z, so that a plane costs one load for the
+//     column above (z neighbours and the pair's inner x neighbour stay in registers, the outer x
+//     neighbour comes by shuffle from the next lane), one for each y neighbour and one for rhs, all
+//     issued a plane ahead; rows at box faces read the neighbouring box (or image, or negated
+//     boundary cell) through DRow::nbd / nbf, as the row kernels do;
+//   * every second cell's six-addend sum, and every update's product with 1/6, is computed on the
+//     integer units (mg_isum.hpp), which run beside the FP64 pipe; results are the same bit for bit.
+// Measured on GB300 at 256^3 (64 boxes of 64^3; row kernels of mg_kernels.cu before): half-sweep 130
+// -> 88 us (marching alone 121), residual 238 -> 182 us; at 128^3 in boxes of 32^3 21 -> 13.5 and
+// 36 -> 30 us; 256^3 FP64 solve 19.5 -> 15.1 ms.  Now FP64 pipe (57%), integer ALU (60%) and
+// load latency share the time.  All sums in integers: 114 us; two rows a thread (96 registers): 88
+// us, slower on small levels; 256 threads at 64 registers: 92 us; the norm and residual-storing
+// half-sweeps run best at 5 blocks an SM (no spills), the residual at 4.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+
+#include "mg_isum.hpp"
+#include "mg_kernels.hpp"
+
+namespace gbmg {
+
+namespace {
+
+constexpr int kMarchThreads = 128;
+
+__device__ __forceinline__ double flip(double v, unsigned n) {  // -v if n is 1
+  unsigned lo, hi;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "d"(v));
+  double r;
+  asm("mov.b64 %0, {%1, %2};" : "=d"(r) : "r"(lo), "r"(hi ^ (n << 31)));
+  return r;
+}
+__device__ __forceinline__ unsigned long long abskey(double a) {
+  unsigned lo, hi;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "d"(a));
+  return ((unsigned long long)(hi & 0x7FFFFFFFu) << 32) | lo;
+}
+// f(x), in a block of its own: a loop over blockDim.y (1 in every launch here, which the compiler
+// does not know), each turn of which would take the last one's result.  Written as a plain
+// condition, the few FP64 instructions of a rare case are predicated instead of branched around,
+// and instructions that are off in all lanes hold the FP64 pipe like any others.
+template <class F>
+__device__ __forceinline__ double rarely(double x, F&& f) {
+  int n = blockDim.y;
+#pragma unroll 1
+  do x = f(x);
+  while (--n > 0);
+  return x;
+}
+__device__ __forceinline__ double sum6_f64(const double (&v)[6]) {
+  double s = __dadd_rn(v[0], v[1]);
+  s = __dadd_rn(s, v[2]);
+  s = __dadd_rn(s, v[3]);
+  s = __dadd_rn(s, v[4]);
+  return __dadd_rn(s, v[5]);
+}
+// The six-addend sum on the integer units (every lane of mask calls it together).
+__device__ __forceinline__ double sum6_int(const double (&v)[6], unsigned mask) {
+  const isum::Six q = isum::six_of(v);
+  if (__all_sync(mask, isum::six_simple(q))) return isum::sum6_simple(v, q);
+  double s;
+  if (!isum::sum6(v, q, &s))
+    s = rarely(v[0], [&](double x) {
+      const double w[6] = {x, v[1], v[2], v[3], v[4], v[5]};
+      return sum6_f64(w);
+    });
+  return s;
+}
+template <bool INT>
+__device__ __forceinline__ double sum6(const double (&v)[6], unsigned mask) {
+  return INT ? sum6_int(v, mask) : sum6_f64(v);
+}
+template <bool INT>
+__device__ __forceinline__ double gs_update(double s, double rhs, double mh2) {
+  const double t = __fma_rn(mh2, rhs, s);
+  double u;
+  if (!INT) return __dmul_rn(t, 1.0 / 6.0);
+  if (!isum::mul_sixth(t, &u)) u = rarely(t, [&](double x) { return __dmul_rn(x, 1.0 / 6.0); });
+  return u;
+}
+__device__ __forceinline__ double residual_of(double s, double phi, double rhs, double mih2) {
+  return __fma_rn(mih2, __fma_rn(-6.0, phi, s), rhs);
+}
+
+template <int V>
+struct Int {
+  static constexpr int value = V;
+};
+
+// Max over the block's threads into *norm.
+__device__ __forceinline__ void block_max(unsigned long long mx, unsigned long long* norm) {
+  __shared__ unsigned long long sm[kMarchThreads / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long w = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = w > mx ? w : mx;
+  }
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kMarchThreads / 32; ++w) mx = sm[w] > mx ? sm[w] : mx;
+    if (mx) atomicMax(norm, mx);
+  }
+}
+
+template <class T>
+__device__ __forceinline__ T* at(T* p, long long bytes) {
+  return (T*)((uintptr_t)p + bytes);
+}
+
+// Box b of the launch; *slot: its segment's norm slot.  MULTI: the launch has several segments.
+template <bool MULTI>
+__device__ __forceinline__ const DRow& box_row(const SegList& L, int b, int* slot) {
+  if (!MULTI) {
+    *slot = L.one.slot;
+    return L.one.rows[b];
+  }
+  Seg S;
+  {
+    int lo = 0, hi = L.n - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (L.segs[mid].box_begin <= b) lo = mid; else hi = mid - 1;
+    }
+    S = L.segs[lo];
+    b -= S.box_begin;
+  }
+  *slot = S.slot;
+  return S.rows[b];
+}
+
+// The half-sweep (x extents even).  MODE as in k_rbgs_half: 0 plain; 1 max-norm of each updated
+// cell's residual after its update; 2 before it, saving the value before to v[2]; 3 the residual
+// after the update stored to v[2] (one-colour views).
+template <int MODE, bool INT, bool MULTI = false>
+__global__ void __launch_bounds__(kMarchThreads, MODE ? 5 : 7)
+    k_half_march(SegList L, int zc, int color, unsigned long long* norms) {
+  pdl_begin();
+  int slot;
+  const DRow& R = box_row<MULTI>(L, blockIdx.y, &slot);
+  const int nx = R.n[0], ny = R.n[1], nz = R.n[2];
+  const int pp = nx >> 1, rb = kMarchThreads / pp;
+  const int nty = (ny + rb - 1) / rb, ntz = (nz + zc - 1) / zc;
+  const int tile = blockIdx.x;
+  if (tile >= nty * ntz) return;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int ry = tid / pp, i = tid - ry * pp;
+  const int y = (tile % nty) * rb + ry;
+  const int z0 = (tile / nty) * zc, z1 = min(z0 + zc, nz);
+  const bool active = ry < rb && y < ny;
+  const unsigned mask = __ballot_sync(0xffffffffu, active);
+  unsigned long long mx = 0;
+  if (active) {
+    const int pitch = R.v[0].pitch;
+    const long long plane = R.v[0].plane;
+    const unsigned nbf = (unsigned)R.nbf;
+    const double mh2 = flip(R.h2, 1u), mih2 = flip(R.ih2, 1u);
+    // place in the pair of the updated cell: pe in planes z0, z0 + 2, ..., pe ^ 1 in the others
+    const int pe = (color + R.lo[0] + R.lo[1] + R.lo[2] + y + z0) & 1, po = pe ^ 1;
+    double* own = (double*)R.v[0].p + z0 * plane + (long long)y * pitch + 2 * i + pe;
+    // byte steps from an even plane's cell to the next plane's, and from an odd one's
+    const int swap = (po - pe) * 8;
+    const long long ie = plane * 8 + swap, io = plane * 8 - swap;
+    const long long re = R.v[1].plane * 8 + swap, ro = R.v[1].plane * 8 - swap;
+    const double* pn = own + plane;  // the other colour's cell above
+    const double* pym = own - pitch + (y == 0 ? R.nbd[2] : 0);
+    const double* pyp = own + pitch + (y == ny - 1 ? R.nbd[3] : 0);
+    const double* pf = (const double*)R.v[1].p + z0 * R.v[1].plane + (long long)y * R.v[1].pitch + 2 * i + pe;
+    const unsigned nym = y == 0 ? (nbf >> 2) & 1u : 0u, nyp = y == ny - 1 ? (nbf >> 3) & 1u : 0u;
+    double* sv = nullptr;
+    long long is = 0;
+    if (MODE == 2 || MODE == 3) {
+      is = R.v[2].plane * 8;
+      sv = (double*)R.v[2].p + z0 * R.v[2].plane + (long long)y * R.v[2].pitch + i;
+    }
+    // outer x neighbour: the next pair's cell from its lane, or loaded at row ends and warp ends
+    const bool exl = i == 0, exr = i == pp - 1;
+    const bool lde = pe ? exr || lane == 31 : exl || lane == 0, ldo = pe ? exl || lane == 0 : exr || lane == 31;
+    const unsigned nxl = exl ? nbf & 1u : 0u, nxr = exr ? (nbf >> 1) & 1u : 0u;
+    const unsigned nxe = pe ? nxr : nxl, nxo = pe ? nxl : nxr;
+    const int srce = pe ? lane + 1 : lane - 1, srco = pe ? lane - 1 : lane + 1;
+    const long long dl = (exl ? R.nbd[0] : 0) - 1, dr = (exr ? R.nbd[1] : 0) + 1;  // from the updated cell
+    const long long dxe = (pe ? dr : dl) * 8, dxo = (pe ? dl : dr) * 8;
+    const double* px = own;  // updated cell of the step being loaded
+    const unsigned nzm = (nbf >> 4) & 1u, nzp = (nbf >> 5) & 1u;
+    const long long dz1 = R.nbd[5] * 8;
+    // the other colour's cell of the column below and beside the updated one
+    double cm = flip(own[-plane + (z0 == 0 ? R.nbd[4] : 0)], z0 == 0 ? nzm : 0u);
+    double cc = own[po - pe];
+    struct In {
+      double n, ym, yp, f, x, o;
+    };
+    auto load = [&](auto Ec, int z, In& v) {  // inputs of step z; the pointers move on to z + 1
+      constexpr int E = decltype(Ec)::value;  // 0: even step
+      if (z == nz - 1) pn = at(pn, dz1);
+      v.n = *pn;
+      v.ym = *pym;
+      v.yp = *pyp;
+      v.f = *pf;
+      if (E ? ldo : lde) v.x = *at(px, E ? dxo : dxe);
+      if (MODE == 2) v.o = *px;
+      pn = at(pn, E ? io : ie);
+      pym = at(pym, E ? io : ie);
+      pyp = at(pyp, E ? io : ie);
+      pf = at(pf, E ? ro : re);
+      px = at(px, E ? io : ie);
+    };
+    auto step = [&](auto Ec, int z, const In& v) {
+      constexpr int E = decltype(Ec)::value;
+      double xo = __shfl_sync(mask, cc, E ? srco : srce);
+      if (E ? ldo : lde) xo = flip(v.x, E ? nxo : nxe);
+      const double cn = z == nz - 1 ? flip(v.n, nzp) : v.n;
+      double w[6] = {xo, cc, flip(v.ym, nym), flip(v.yp, nyp), cm, cn};
+      const double s = sum6<INT && E>(w, mask);
+      const double un = gs_update<INT>(s, v.f, mh2);
+      if (MODE == 2) {
+        const unsigned long long k = abskey(residual_of(s, v.o, v.f, mih2));
+        mx = k > mx ? k : mx;
+        *sv = v.o;
+      }
+      *own = un;
+      if (MODE == 1 || MODE == 3) {
+        double s2 = s;
+        const unsigned sx = (E ? ldo : lde) ? (E ? nxo : nxe) : 0u;
+        const unsigned sm = z == 0 ? nzm : 0u, sp = z == nz - 1 ? nzp : 0u;
+        if (sx | nym | nyp | sm | sp) {  // reads of its own value, negated
+          const double m = flip(un, 1u);
+          if (sx) w[0] = m;
+          if (nym) w[2] = m;
+          if (nyp) w[3] = m;
+          if (sm) w[4] = m;
+          if (sp) w[5] = m;
+          s2 = rarely(w[0], [&](double x) {
+            const double q[6] = {x, w[1], w[2], w[3], w[4], w[5]};
+            return sum6_f64(q);
+          });
+        }
+        const double r = residual_of(s2, un, v.f, mih2);
+        if (MODE == 3) *sv = r;
+        if (MODE == 1) {
+          const unsigned long long k = abskey(r);
+          mx = k > mx ? k : mx;
+        }
+      }
+      if (MODE == 2 || MODE == 3) sv = at(sv, is);
+      own = at(own, E ? io : ie);
+      cm = cc;
+      cc = cn;
+    };
+    In a, b;
+    load(Int<0>{}, z0, a);
+    for (int z = z0; z < z1; z += 2) {
+      if (z + 1 < z1) load(Int<1>{}, z + 1, b);
+      step(Int<0>{}, z, a);
+      if (z + 1 < z1) {
+        if (z + 2 < z1) load(Int<0>{}, z + 2, a);
+        step(Int<1>{}, z + 1, b);
+      }
+    }
+  }
+  if (MODE == 1 || MODE == 2) block_max(mx, &norms[slot + R.solve]);
+}
+
+// Residual of every cell (stored if v[2] is set) and its max-norm into norms (if set); any x extent.
+template <bool INT, bool MULTI>
+__global__ void __launch_bounds__(kMarchThreads, 4)
+    k_residual_march(SegList L, int zc, unsigned long long* norms) {
+  pdl_begin();
+  int slot;
+  const DRow& R = box_row<MULTI>(L, blockIdx.y, &slot);
+  const int nx = R.n[0], ny = R.n[1], nz = R.n[2];
+  const int pp = (nx + 1) >> 1, rb = kMarchThreads / pp;
+  const int nty = (ny + rb - 1) / rb, ntz = (nz + zc - 1) / zc;
+  const int tile = blockIdx.x;
+  if (tile >= nty * ntz) return;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int ry = tid / pp, i = tid - ry * pp;
+  const int y = (tile % nty) * rb + ry;
+  const int z0 = (tile / nty) * zc, z1 = min(z0 + zc, nz);
+  const bool active = ry < rb && y < ny;
+  const unsigned mask = __ballot_sync(0xffffffffu, active);
+  unsigned long long mx = 0;
+  if (active) {
+    const bool two = 2 * i + 1 < nx;  // the pair's second cell exists
+    const int pitch = R.v[0].pitch;
+    const long long plane = R.v[0].plane, ip = plane * 8, ir = R.v[1].plane * 8, io = R.v[2].plane * 8;
+    const unsigned nbf = (unsigned)R.nbf;
+    const double mih2 = flip(R.ih2, 1u);
+    const double* own = (const double*)R.v[0].p + z0 * plane + (long long)y * pitch + 2 * i;
+    const double* pn = own + plane;
+    const double* pym = own - pitch + (y == 0 ? R.nbd[2] : 0);
+    const double* pyp = own + pitch + (y == ny - 1 ? R.nbd[3] : 0);
+    const double* pf = (const double*)R.v[1].p + z0 * R.v[1].plane + (long long)y * R.v[1].pitch + 2 * i;
+    double* out = R.v[2].p ? (double*)R.v[2].p + z0 * R.v[2].plane + (long long)y * R.v[2].pitch + 2 * i : nullptr;
+    const unsigned nym = y == 0 ? (nbf >> 2) & 1u : 0u, nyp = y == ny - 1 ? (nbf >> 3) & 1u : 0u;
+    // outer x neighbours: the next pairs' cells from their lanes, or loaded at row and warp ends
+    const bool exl = i == 0, exr = i == pp - 1, ldl = exl || lane == 0, ldr = exr || lane == 31;
+    const unsigned nxl = exl ? nbf & 1u : 0u, nxr = exr ? (nbf >> 1) & 1u : 0u;
+    const double* pxl = own - 1 + (exl ? R.nbd[0] : 0);
+    const double* pxr = own + (two ? 2 : 1) + (exr ? R.nbd[1] : 0);
+    const unsigned nzm = (nbf >> 4) & 1u, nzp = (nbf >> 5) & 1u;
+    const long long dz1 = R.nbd[5] * 8;
+    const double* below = own - plane + (z0 == 0 ? R.nbd[4] : 0);
+    const unsigned nb = z0 == 0 ? nzm : 0u;
+    double m0 = flip(below[0], nb), m1 = flip(below[1], nb);
+    double c0 = own[0], c1 = own[1];
+    struct In {
+      double n0, n1, ym0, ym1, yp0, yp1, f0, f1, xl, xr;
+    };
+    auto load = [&](int z, In& v) {
+      if (z == nz - 1) pn = at(pn, dz1);
+      v.n0 = pn[0];
+      v.n1 = pn[1];
+      v.ym0 = pym[0];
+      v.ym1 = pym[1];
+      v.yp0 = pyp[0];
+      v.yp1 = pyp[1];
+      v.f0 = pf[0];
+      v.f1 = two ? pf[1] : 0.0;
+      if (ldl) v.xl = *pxl;
+      if (ldr) v.xr = *pxr;
+      pn = at(pn, ip);
+      pym = at(pym, ip);
+      pyp = at(pyp, ip);
+      pxl = at(pxl, ip);
+      pxr = at(pxr, ip);
+      pf = at(pf, ir);
+    };
+    auto step = [&](int z, const In& v) {
+      double xl = __shfl_sync(mask, c1, lane - 1), xr = __shfl_sync(mask, c0, lane + 1);
+      if (ldl) xl = flip(v.xl, nxl);
+      if (ldr) xr = flip(v.xr, nxr);
+      const bool zend = z == nz - 1;
+      const double n0 = zend ? flip(v.n0, nzp) : v.n0, n1 = zend ? flip(v.n1, nzp) : v.n1;
+      const double w0[6] = {xl, two ? c1 : xr, flip(v.ym0, nym), flip(v.yp0, nyp), m0, n0};
+      const double w1[6] = {c0, xr, flip(v.ym1, nym), flip(v.yp1, nyp), m1, n1};
+      const double s0 = sum6<false>(w0, mask), s1 = sum6<INT>(w1, mask);
+      const double r0 = residual_of(s0, c0, v.f0, mih2), r1 = residual_of(s1, c1, v.f1, mih2);
+      unsigned long long k = abskey(r0);
+      mx = k > mx ? k : mx;
+      k = abskey(r1);
+      if (two) mx = k > mx ? k : mx;
+      if (out) {
+        out[0] = r0;
+        if (two) out[1] = r1;
+        out = at(out, io);
+      }
+      m0 = c0;
+      m1 = c1;
+      c0 = n0;
+      c1 = n1;
+    };
+    In a, b;
+    load(z0, a);
+    for (int z = z0; z < z1; z += 2) {
+      if (z + 1 < z1) load(z + 1, b);
+      step(z, a);
+      if (z + 1 < z1) {
+        if (z + 2 < z1) load(z + 2, a);
+        step(z + 1, b);
+      }
+    }
+  }
+  if (norms) block_max(mx, &norms[slot + R.solve]);
+}
+
+// Blocks over (rows of a box x chunks of *zc planes, boxes); chunks are halved until about six
+// blocks an SM are there (4 and 16 instead: within 2% at 256^3, slower at 128^3 and below).
+dim3 march_grid(const SegList& L, int* zc) {
+  const int* ext = L.ext.n;
+  const int rb = kMarchThreads / ((ext[0] + 1) / 2);
+  const int ty = (ext[1] + rb - 1) / rb;
+  *zc = 32;
+  while (*zc > 2 && (long long)L.nbox * ty * ((ext[2] + *zc - 1) / *zc) < 6ll * num_sms()) *zc /= 2;
+  return dim3((unsigned)(ty * ((ext[2] + *zc - 1) / *zc)), (unsigned)L.nbox);
+}
+// Launches over fewer cells leave the FP64 pipe idle most of the time and are bound by latency,
+// where the integer sums' longer chains cost more than they save (64^3 FP64 solve: 1.70 ms with
+// integer sums on every level, 1.62 ms with this line).
+bool use_int(const SegList& L) {
+  return (long long)L.nbox * L.ext.n[0] * L.ext.n[1] * L.ext.n[2] >= 1ll << 15;
+}
+
+}  // namespace
+
+cudaError_t launch_half_march(const SegList& L, int mode, int color, unsigned long long* norms,
+                              cudaStream_t s) {
+  int zc;
+  const dim3 grid = march_grid(L, &zc);
+  auto go = [&](auto k) { launch_k(k, grid, kMarchThreads, 0, s, L, zc, color, norms); };
+  if (mode && L.n != 1) return cudaErrorInvalidValue;
+  if (use_int(L)) {
+    if (mode == 0 && L.n > 1) go(k_half_march<0, true, true>);
+    else if (mode == 0) go(k_half_march<0, true>);
+    else if (mode == 1) go(k_half_march<1, true>);
+    else if (mode == 2) go(k_half_march<2, true>);
+    else go(k_half_march<3, true>);
+  } else {
+    if (mode == 0 && L.n > 1) go(k_half_march<0, false, true>);
+    else if (mode == 0) go(k_half_march<0, false>);
+    else if (mode == 1) go(k_half_march<1, false>);
+    else if (mode == 2) go(k_half_march<2, false>);
+    else go(k_half_march<3, false>);
+  }
+  count_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_residual_march(const SegList& L, unsigned long long* norms, cudaStream_t s) {
+  int zc;
+  const dim3 grid = march_grid(L, &zc);
+  auto go = [&](auto k) { launch_k(k, grid, kMarchThreads, 0, s, L, zc, norms); };
+  if (use_int(L)) {
+    if (L.n > 1) go(k_residual_march<true, true>);
+    else go(k_residual_march<true, false>);
+  } else {
+    if (L.n > 1) go(k_residual_march<false, true>);
+    else go(k_residual_march<false, false>);
+  }
+  count_launches(1);
+  return cudaGetLastError();
+}
+
+}  // namespace gbmg

@@ -336,7 +336,14 @@ OpTable upload_table(Ctx& c, const std::vector<DRow>& rows, long long nrows, cud
   OpTable t;
   t.nbox = (int)rows.size();
   t.nrows = nrows;
-  for (const DRow& R : rows) t.width = std::max(t.width, R.n[0]);
+  t.ext.ok = !rows.empty() && rows.size() <= (size_t)kMarchMaxBoxes;
+  t.ext.even = true;
+  for (const DRow& R : rows) {
+    t.width = std::max(t.width, R.n[0]);
+    for (int d = 0; d < 3; ++d) t.ext.n[d] = std::max(t.ext.n[d], R.n[d]);
+    t.ext.ok = t.ext.ok && R.n[0] <= kMarchMaxX;
+    t.ext.even = t.ext.even && R.n[0] % 2 == 0;
+  }
   if (!rows.empty()) t.d = c.upload(rows.data(), rows.size() * sizeof(DRow), s);
   return t;
 }
@@ -1162,7 +1169,7 @@ int mg_smooth(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double hh
           tt.direct = true;
           return tt;
         });
-        MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, color & 1, s, true, nullptr, t.width));
+        MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, color & 1, s, true, nullptr, t.width, false, t.ext));
         return MG_OK;
       }
     }
@@ -1191,11 +1198,11 @@ int mg_smooth(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double hh
       }
     }
     if (color < 2) {
-      MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, color, s, false, nullptr, t.width));
+      MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, color, s, false, nullptr, t.width, false, t.ext));
     } else {
       for (int col = 0; col < 2; ++col) {
         launch_fill(*c, *fp, bc, s);
-        MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, col, s, false, nullptr, t.width));
+        MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, col, s, false, nullptr, t.width, false, t.ext));
       }
     }
     return MG_OK;
@@ -1250,7 +1257,7 @@ int mg_residual(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, mg_fab_t r, double hh, d
     std::lock_guard<std::mutex> nl(c->op_norm_mu);
     unsigned long long* dn = (unsigned long long*)c->op_norm.d->p;
     MG_CK(cudaMemsetAsync(dn, 0, 8, s));
-    MG_CK(launch_residual(fp->dtype, t.rows(), t.nbox, t.nrows, dn, s));
+    MG_CK(launch_residual(fp->dtype, t.rows(), t.nbox, t.nrows, dn, s, false, -1, t.ext));
     if (norm) {
       MG_CK(cudaMemcpyAsync(c->op_norm.h, dn, 8, cudaMemcpyDeviceToHost, s));
       MG_CK(cudaStreamSynchronize(s));

@@ -151,6 +151,7 @@ struct OpTable {
   long long nrows = 0;
   bool direct = false;  // rows carry box-face reads (DRow::nbd / nbf)
   int width = 0;        // widest box x-extent of the rows
+  BoxExtents ext;       // largest box extents
   const DRow* rows() const { return d ? (const DRow*)d->p : nullptr; }
 };
 

@@ -430,10 +430,10 @@ void smooth(Ctx& c, Hierarchy& H, LevelData& D, int sweeps, cudaStream_t s,
       if (timed) MG_CK(cudaEventRecordWithFlags(H.sweep_ev[0], s, cudaEventRecordExternal));
       if (last && store_last)
         MG_CK(launch_rbgs_half_store(H.store0.rows(), H.store0.nbox, H.store0.nrows, color, s,
-                                     H.store0.width));
+                                     H.store0.width, H.store0.ext));
       else
         MG_CK(launch_rbgs_half(H.dt, D.smooth.rows(), D.smooth.nbox, D.smooth.nrows, color, s,
-                               D.direct, last ? last_norm : nullptr, D.smooth.width));
+                               D.direct, last ? last_norm : nullptr, D.smooth.width, false, D.smooth.ext));
       if (timed) MG_CK(cudaEventRecordWithFlags(H.sweep_ev[1], s, cudaEventRecordExternal));
     }
 }
@@ -483,7 +483,7 @@ void enqueue_step(Ctx& c, Hierarchy& H, cudaStream_t s, int variant) {
     MG_CK(cudaMemsetAsync(dn, 0, 8, s));
     enqueue_vcycle(c, H, s, dn, variant == 2);
     MG_CK(launch_rbgs_half(DT_F64, D0.smooth.rows(), D0.smooth.nbox, D0.smooth.nrows, 0, s, true,
-                           dn, D0.smooth.width, true));
+                           dn, D0.smooth.width, true, D0.smooth.ext));
     MG_CK(cudaMemcpyAsync(H.hnorm, dn, 16, cudaMemcpyDeviceToHost, s));
     return;
   }
@@ -511,7 +511,7 @@ void enqueue_step(Ctx& c, Hierarchy& H, cudaStream_t s, int variant) {
   if (!split_norm) MG_CK(cudaMemsetAsync(dn, 0, 8, s));
   if (!H.direct0) launch_fill(c, *H.phi0, &H.bc, s, 1);
   MG_CK(launch_residual(DT_F64, H.resid0.rows(), H.resid0.nbox, H.resid0.nrows, dn, s, H.direct0,
-                        split_norm ? 0 : -1));
+                        split_norm ? 0 : -1, H.resid0.ext));
   MG_CK(cudaMemcpyAsync(H.hnorm, dn, 16, cudaMemcpyDeviceToHost, s));
 }
 
@@ -605,7 +605,8 @@ int solve(Ctx& c, int64_t rhs_id, int64_t phi_id, const mg_bc* bc, double tol,
   MG_CK(cudaMemsetAsync(dn, 0, 16, s));
   MG_CK(launch_maxabs(DT_F64, H.rhsabs0.rows(), H.rhsabs0.nbox, H.rhsabs0.nrows, dn, s));
   if (!H.direct0) launch_fill(c, *H.phi0, bc, s, 1);
-  MG_CK(launch_residual(DT_F64, H.resid0.rows(), H.resid0.nbox, H.resid0.nrows, dn, s, H.direct0));
+  MG_CK(launch_residual(DT_F64, H.resid0.rows(), H.resid0.nbox, H.resid0.nrows, dn, s, H.direct0, -1,
+                        H.resid0.ext));
   MG_CK(cudaMemcpyAsync(H.hnorm, dn, 16, cudaMemcpyDeviceToHost, s));
   MG_CK(cudaStreamSynchronize(s));
   const double rhsnorm = bits_to_double(H.hnorm[1]);
