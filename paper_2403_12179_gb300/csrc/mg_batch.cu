@@ -136,6 +136,12 @@ struct SweepB {
     if (!ab.empty()) plan = plan_sweep(ab, ba);
   }
 };
+// Residual + restriction of wide levels.
+struct RestrictB {
+  std::vector<RestrictGrid> v;
+  RestrictPlan plan;
+  size_t off = 0;
+};
 struct JobB {
   std::vector<BottomJob> v;
   int maxN = 0;
@@ -163,6 +169,7 @@ struct LevelLists {
   TagB fill_c;    // the coarse level's phi, one layer, before the trilinear prolongation
   UnitB fab, fba;
   SweepB sweep;
+  RestrictB rr_wide;
   JobB bottom_next;      // bottoms at level l + 1
   CoarseB coarse_next;   // coarse cycles from level l + 1
 };
@@ -255,7 +262,8 @@ void build_lists(Ctx& c, StepLists& S, const std::vector<Member*>& run,
       }
       if (!D.direct) LL.fill1_all.add(fill_plan(c, *D.phi, &H.bc, 1), D.phi->base);
       LL.half_all.add(D.smooth, m->slot);
-      LL.rr.add(D.rr, m->slot);
+      if (D.wide_rr) LL.rr_wide.v.push_back(D.rr_grid);
+      else LL.rr.add(D.rr, m->slot);
       if (H.p.prolong == MG_PROLONG_TRILINEAR) {
         LL.prolong3.add(D.prolong, m->slot);
         FabObj& cphi = *H.L[l + 1].phi;
@@ -271,7 +279,10 @@ void build_lists(Ctx& c, StepLists& S, const std::vector<Member*>& run,
       S.correct0.add(H.correct0, m->slot);
     }
   }
-  for (LevelLists& LL : S.L) LL.sweep.finish();
+  for (LevelLists& LL : S.L) {
+    LL.sweep.finish();
+    LL.rr_wide.plan = plan_restrict(LL.rr_wide.v);
+  }
   for (Member* m : check) {
     S.resid0.add(m->H->resid0, m->slot);
     if (!m->H->direct0) S.fill_phi0.add(fill_plan(c, *m->H->phi0, &m->H->bc, 1), m->H->phi0->base);
@@ -293,6 +304,7 @@ void upload_lists(Ctx& c, StepLists& S, Staging& st, cudaStream_t s) {
     unit(LL.fab); unit(LL.fba);
     LL.sweep.off_ab = st.push(LL.sweep.ab);
     LL.sweep.off_ba = st.push(LL.sweep.ba);
+    LL.rr_wide.off = st.push(LL.rr_wide.v);
     job(LL.bottom_next);
     cjob(LL.coarse_next);
   }
@@ -363,11 +375,13 @@ void enqueue_step(Ctx& c, StepLists& S, const unsigned char* dev, unsigned long 
                                 (int)S.coarse0.v.size(), S.coarse0.smem, s));
     for (int l = 0; l < nlev; ++l) {
       LevelLists& LL = S.L[l];
-      if (!LL.rr.total) continue;
+      if (!LL.rr.total && !LL.rr_wide.plan.tiles) continue;
       if (LL.fill_rhs.total) fill_l(c, S.dt, LL.fill_rhs, dev, s);
       smooth_l(c, S, LL, S.nu1, dev, err, s);
       fill_l(c, S.dt, LL.fill1_all, dev, s);
       MG_CK(launch_residual_restrict_l(S.dt, mk(LL.rr, dev), LL.rr.total, s, LL.rr.direct));
+      MG_CK(launch_restrict_f32((const RestrictGrid*)(dev + LL.rr_wide.off), (int)LL.rr_wide.v.size(),
+                                LL.rr_wide.plan, s));
       if (!LL.bottom_next.v.empty())
         MG_CK(launch_bottom(S.dt, (const BottomJob*)(dev + LL.bottom_next.off),
                             (int)LL.bottom_next.v.size(), LL.bottom_next.maxN, s));

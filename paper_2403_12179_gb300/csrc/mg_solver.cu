@@ -56,6 +56,24 @@ DView coarse_view_of(const FabObj& coarse, const Box& fine_box) {
 
 namespace {
 
+// A coarse FP32 field as the wide residual + restriction writes it: pairs of cells (the children of
+// one strip of 4) must lie in one box.
+bool coarse_field(const FabObj& f, CoarseField* out) {
+  Lattice T;
+  if (f.dtype != DT_F32 || !lattice_of(f.ba->ba, f.lay, &T) || (T.E[0] & 1)) return false;
+  CoarseField C{};
+  C.base = (float*)f.base + T.first;
+  for (int d = 0; d < 3; ++d) {
+    C.E[d] = T.E[d];
+    C.nb[d] = T.nb[d];
+  }
+  C.pitch = T.pitch;
+  C.plane = T.plane;
+  C.bstride = T.bstride;
+  *out = C;
+  return true;
+}
+
 // Smallest level (cells) that the automatic smoother choice runs with the fused sweep (FP32).
 // Measured on GB300 (mixed 256^3 / 512^3 solves, 512 batched solves): 256^3 beats 2^18, 2^21,
 // 2^25 and fusing every level.
@@ -97,6 +115,18 @@ void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
       D.f_ab = make_fused(c, ba, D.h, *D.phi, *D.rhs, *D.phi2, per, s);
       D.f_ba = make_fused(c, ba, D.h, *D.phi2, *D.rhs, *D.phi, per, s);
       if (!D.f_ab.ok || !D.f_ba.ok) D.fused = false;
+    }
+    if (D.wide) {
+      const LevelData& C = H.L[l + 1];
+      D.rr_grid.g = D.sweep_ab;
+      D.rr_grid.mih2 = -(float)(1.0 / (D.h * D.h));
+      D.wide_rr = (D.bao->ba.dom.len(2) & 1) == 0 && coarse_field(*C.rhs, &D.rr_grid.crhs) &&
+                  coarse_field(*C.phi, &D.rr_grid.cphi);
+      if (D.wide_rr) {
+        std::vector<RestrictGrid> q{D.rr_grid};
+        D.rr_plan = plan_restrict(q);
+        D.rr_dev = c.upload(q.data(), sizeof(RestrictGrid), s);
+      }
     }
     if (l + 1 < nl) {
       const LevelData& C = H.L[l + 1];
@@ -451,8 +481,11 @@ void enqueue_vcycle(Ctx& c, Hierarchy& H, cudaStream_t s, unsigned long long* no
     smooth(c, H, D, H.p.nu1, s, nullptr, l == 0 && H.graph_timed, l == 0 && skip_first_red,
            stored);
     if (!D.direct) launch_fill(c, *D.phi, &H.bc, s, 1);
-    MG_CK(launch_residual_restrict(H.dt, D.rr.rows(), D.rr.nbox, D.rr.nrows, s, D.direct,
-                                   D.rr.width, stored));
+    if (D.wide_rr)
+      MG_CK(launch_restrict_f32((const RestrictGrid*)D.rr_dev->p, 1, D.rr_plan, s));
+    else
+      MG_CK(launch_residual_restrict(H.dt, D.rr.rows(), D.rr.nbox, D.rr.nrows, s, D.direct,
+                                     D.rr.width, stored));
   }
   if (H.lc < nl) MG_CK(launch_coarse_cycle(H.dt, (const CoarseJob*)H.cjob->p, 1, H.csmem, s));
   else MG_CK(launch_bottom(H.dt, (const BottomJob*)H.job->p, 1, H.N, s));

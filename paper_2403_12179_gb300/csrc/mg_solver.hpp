@@ -21,6 +21,10 @@ struct LevelData {
   bool wide = false;
   SweepGrid sweep_ab{}, sweep_ba{};  // phi -> phi2, phi2 -> phi (geometry and pointers)
   DevBufP sweep_dev;                 // both, tiled for a launch of their own
+  bool wide_rr = false;              // its residual + restriction too (rr_grid)
+  RestrictGrid rr_grid{};
+  DevBufP rr_dev;
+  RestrictPlan rr_plan{};
   SweepPlan sweep_plan{};            // no tiles: too small for a launch of its own
   long long cells() const { return bao->ba.dom.npts(); }
   std::shared_ptr<FabObj> phi2;

@@ -284,6 +284,150 @@ __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
+// Residual + restriction.  A thread owns a strip of 4 cells in two rows (2Y, 2Y + 1), i.e. two
+// coarse cells, and marches through planes; z neighbours stay in registers, the rest is loaded a
+// plane ahead (neighbouring strips and rows mostly from L1, where the threads owning them put
+// them).  Arithmetic and order as k_residual_restrict.  HBM bounds it (phi and rhs read once, 8
+// bytes a cell); measured at 512^3: 959 us by k_residual_restrict reading neighbours directly (128-wide
+// rows, scalar loads, 4 children rows a lane), 196 us here (5.5 TB/s, 81% of the copy rate); 256^3 112
+// -> 38 us.  3, 4 or 5 blocks an SM: within 1%.
+constexpr int kRestrictThreads = 128, kRestrictChunk = 32;
+__global__ void __launch_bounds__(kRestrictThreads, 4)
+    k_restrict_f32(const RestrictGrid* __restrict__ grids, int ng) {
+  pdl_begin();
+  __shared__ long long zoff[kRestrictChunk + 3], coff[2][kRestrictChunk / 2];
+  __shared__ RestrictGrid Gs;
+  if (threadIdx.x == 0) {
+    int lo = 0, hi = ng - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (grids[mid].tile_begin <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
+    }
+    Gs = grids[lo];
+  }
+  __syncthreads();
+  const RestrictGrid& Q = Gs;
+  const SweepGrid& G = Q.g;
+  const int t = blockIdx.x - Q.tile_begin;
+  const int tz = t / Q.tiles_xy, col = (t - tz * Q.tiles_xy) * kRestrictThreads + threadIdx.x;
+  const int N0 = G.N[0], N1 = G.N[1], N2 = G.N[2], strips = N0 >> 2;
+  const bool px = G.periodic & 1, py = G.periodic & 2, pz = G.periodic & 4;
+  const int z0 = tz * Q.ZC, z1 = min(z0 + Q.ZC, N2);
+  for (int q = threadIdx.x; q < z1 - z0 + 2; q += kRestrictThreads) {  // planes z0 - 1 ... z1
+    int p = z0 - 1 + q;
+    if (pz) p = p < 0 ? p + N2 : p >= N2 ? p - N2 : p;
+    else p = min(max(p, 0), N2 - 1);  // the mirrored plane
+    const int bz = p / G.E[2];
+    zoff[q] = ((long long)bz * G.nb[0] * G.nb[1] * G.bstride + (long long)(p - bz * G.E[2]) * G.plane) * 4;
+  }
+  for (int q = threadIdx.x; q < z1 - z0; q += kRestrictThreads) {  // coarse planes, rhs and phi
+    const CoarseField& C = q & 1 ? Q.cphi : Q.crhs;
+    const int Z = (z0 + q) >> 1, bz = Z / C.E[2];
+    coff[q & 1][q >> 1] = ((long long)bz * C.nb[0] * C.nb[1] * C.bstride + (long long)(Z - bz * C.E[2]) * C.plane) * 4;
+  }
+  __syncthreads();
+  if (col >= strips * (N1 >> 1)) return;
+  const int m = col / strips, gx = (col - m * strips) * 4, gy = 2 * m;
+  // place of cell (x, y) in plane 0 of the lattice, bytes
+  auto place = [&](int x, int y) {
+    const int bx = x / G.E[0], by = y / G.E[1];
+    return ((long long)(by * G.nb[0] + bx) * G.bstride + (long long)(y - by * G.E[1]) * G.pitch + (x - bx * G.E[0])) * 4;
+  };
+  const long long pA = place(gx, gy), pB = place(gx, gy + 1);
+  // outside a Dirichlet face: the cell's own value, negated
+  const bool ylo = gy == 0, yhi = gy + 2 == N1, xlo = gx == 0, xhi = gx + 4 == N0;
+  const long long pym = ylo ? (py ? place(gx, N1 - 1) : pA) : place(gx, gy - 1);
+  const long long pyp = yhi ? (py ? place(gx, 0) : pB) : place(gx, gy + 2);
+  const int xl = xlo ? (px ? N0 - 1 : 0) : gx - 1, xr = xhi ? (px ? 0 : N0 - 1) : gx + 4;
+  const long long plA = place(xl, gy), plB = place(xl, gy + 1), prA = place(xr, gy), prB = place(xr, gy + 1);
+  const uint32_t nym = ylo && !py ? 0x80000000u : 0u, nyp = yhi && !py ? 0x80000000u : 0u;
+  const uint32_t nxl = xlo && !px ? 0x80000000u : 0u, nxr = xhi && !px ? 0x80000000u : 0u;
+  const char* src = (const char*)G.src;
+  const char* rhs = (const char*)G.rhs;
+  const float mih2 = Q.mih2;
+  const int X = gx >> 1, Y = m;
+  auto cplace = [&](const CoarseField& C) {
+    const int bx = X / C.E[0], by = Y / C.E[1];  // (a strip's two coarse cells share a box)
+    return (char*)C.base + ((long long)(by * C.nb[0] + bx) * C.bstride + (long long)(Y - by * C.E[1]) * C.pitch + (X - bx * C.E[0])) * 4;
+  };
+  char* cr = cplace(Q.crhs);
+  char* cp = Q.cphi.base ? cplace(Q.cphi) : nullptr;
+  struct In {
+    float4 nA, nB, ym, yp, fA, fB;
+    float lA, lB, rA, rB;
+  };
+  auto ld4 = [](const char* q) { return __ldg(reinterpret_cast<const float4*>(q)); };
+  auto ld1 = [](const char* q) { return __ldg(reinterpret_cast<const float*>(q)); };
+  auto load = [&](int z, In& v) {  // inputs of plane z: its surroundings, and the plane above
+    const char* s = src + zoff[z - z0 + 1];
+    const char* u = src + zoff[z - z0 + 2];
+    const char* f = rhs + zoff[z - z0 + 1];
+    v.nA = ld4(u + pA);
+    v.nB = ld4(u + pB);
+    v.ym = ld4(s + pym);
+    v.yp = ld4(s + pyp);
+    v.fA = ld4(f + pA);
+    v.fB = ld4(f + pB);
+    v.lA = ld1(s + plA);
+    v.lB = ld1(s + plB);
+    v.rA = ld1(s + prA);
+    v.rB = ld1(s + prB);
+  };
+  const uint32_t nz0 = !pz && z0 == 0 ? 0x80000000u : 0u;
+  float4 mA = flip4(ld4(src + zoff[0] + pA), nz0), mB = flip4(ld4(src + zoff[0] + pB), nz0);
+  float4 cA = ld4(src + zoff[1] + pA), cB = ld4(src + zoff[1] + pB);
+  float acc0 = 0.f, acc1 = 0.f;
+  auto res = [&](float xm, float xp, float ym, float yp, float zm, float zp, float c, float f) {
+    float s = __fadd_rn(xm, xp);
+    s = __fadd_rn(s, ym);
+    s = __fadd_rn(s, yp);
+    s = __fadd_rn(s, zm);
+    s = __fadd_rn(s, zp);
+    return __fmaf_rn(mih2, __fmaf_rn(-6.f, c, s), f);
+  };
+  auto step = [&](auto Kc, int z, const In& v) {
+    constexpr int K = decltype(Kc)::value;  // plane of the pair
+    const uint32_t nz = !pz && z == N2 - 1 ? 0x80000000u : 0u;
+    const float4 nA = flip4(v.nA, nz), nB = flip4(v.nB, nz), ym = flip4(v.ym, nym), yp = flip4(v.yp, nyp);
+    const float lA = flip1(v.lA, nxl), lB = flip1(v.lB, nxl), rA = flip1(v.rA, nxr), rB = flip1(v.rB, nxr);
+    const float a0 = res(lA, cA.y, ym.x, cB.x, mA.x, nA.x, cA.x, v.fA.x);
+    const float a1 = res(cA.x, cA.z, ym.y, cB.y, mA.y, nA.y, cA.y, v.fA.y);
+    const float a2 = res(cA.y, cA.w, ym.z, cB.z, mA.z, nA.z, cA.z, v.fA.z);
+    const float a3 = res(cA.z, rA, ym.w, cB.w, mA.w, nA.w, cA.w, v.fA.w);
+    const float b0 = res(lB, cB.y, cA.x, yp.x, mB.x, nB.x, cB.x, v.fB.x);
+    const float b1 = res(cB.x, cB.z, cA.y, yp.y, mB.y, nB.y, cB.y, v.fB.y);
+    const float b2 = res(cB.y, cB.w, cA.z, yp.z, mB.z, nB.z, cB.z, v.fB.z);
+    const float b3 = res(cB.z, rB, cA.w, yp.w, mB.w, nB.w, cB.w, v.fB.w);
+    acc0 = K ? __fadd_rn(acc0, a0) : a0;
+    acc1 = K ? __fadd_rn(acc1, a2) : a2;
+    acc0 = __fadd_rn(__fadd_rn(__fadd_rn(acc0, a1), b0), b1);
+    acc1 = __fadd_rn(__fadd_rn(__fadd_rn(acc1, a3), b2), b3);
+    if (K) {
+      const int q = (z - z0) >> 1;
+      float* c = reinterpret_cast<float*>(cr + coff[0][q]);
+      c[0] = __fmul_rn(acc0, 0.125f);
+      c[1] = __fmul_rn(acc1, 0.125f);
+      if (cp) {
+        float* e = reinterpret_cast<float*>(cp + coff[1][q]);
+        e[0] = 0.f;
+        e[1] = 0.f;
+      }
+    }
+    mA = cA;
+    mB = cB;
+    cA = nA;
+    cB = nB;
+  };
+  In a, b;
+  load(z0, a);
+  for (int z = z0; z < z1; z += 2) {
+    load(z + 1, b);
+    step(Int<0>{}, z, a);
+    if (z + 2 < z1) load(z + 2, a);
+    step(Int<1>{}, z + 1, b);
+  }
+}
+
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 // Threads of a tile, rounded to warps.
@@ -293,24 +437,21 @@ int tile_threads(int S, int TY, int hx, int hy) { return (((S + 2 * hx) * (TY / 
 
 const long long kSweepMinCells = 1ll << 14, kSweepMinCellsBatch = 1ll << 18;
 
-bool sweep_geometry(const BoxArray& ba, const FabLayout& lay, const int periodic[3], double h,
-                    SweepGrid* out) {
-  if (ba.boxes.empty() || lay.g != 0 || lay.ncomp != 1 || lay.esize != 4) return false;
-  SweepGrid G{};
+bool lattice_of(const BoxArray& ba, const FabLayout& lay, Lattice* out) {
+  if (ba.boxes.empty()) return false;
+  Lattice G{};
   for (int d = 0; d < 3; ++d) {
     G.N[d] = ba.dom.len(d);
     G.E[d] = ba.boxes[0].len(d);
-    if (G.N[d] % G.E[d] != 0 || (periodic[d] && (G.N[d] & 1))) return false;
+    if (G.N[d] % G.E[d] != 0) return false;
     G.nb[d] = G.N[d] / G.E[d];
-    G.periodic |= periodic[d] ? 1 << d : 0;
   }
-  if (G.E[0] % 4 != 0 || (G.N[1] & 1) || lay.pitch[0] % 4 != 0) return false;
   const size_t nb = ba.boxes.size();
   if ((long long)nb != (long long)G.nb[0] * G.nb[1] * G.nb[2] || lay.plane[0] > (1ll << 30)) return false;
   G.pitch = lay.pitch[0];
   G.plane = (int)lay.plane[0];
-  G.bstride = nb > 1 ? lay.off[1] - lay.off[0] : lay.plane[0] * G.E[2];
-  if (lay.off[0] != 0 || G.bstride % 4 != 0) return false;
+  G.first = lay.off[0] + lay.g * (lay.plane[0] + lay.pitch[0] + 1);
+  G.bstride = nb > 1 ? lay.off[1] - lay.off[0] : lay.cstride[0];
   size_t b = 0;
   for (int z = 0; z < G.nb[2]; ++z)
     for (int y = 0; y < G.nb[1]; ++y)
@@ -318,9 +459,30 @@ bool sweep_geometry(const BoxArray& ba, const FabLayout& lay, const int periodic
         const int at[3] = {x, y, z};
         for (int d = 0; d < 3; ++d)
           if (ba.boxes[b].lo[d] != ba.dom.lo[d] + at[d] * G.E[d] || ba.boxes[b].len(d) != G.E[d]) return false;
-        if (lay.off[b] != (long long)b * G.bstride || lay.pitch[b] != G.pitch || lay.plane[b] != G.plane)
+        if (lay.off[b] != lay.off[0] + (long long)b * G.bstride || lay.pitch[b] != G.pitch ||
+            lay.plane[b] != G.plane)
           return false;
       }
+  *out = G;
+  return true;
+}
+
+bool sweep_geometry(const BoxArray& ba, const FabLayout& lay, const int periodic[3], double h,
+                    SweepGrid* out) {
+  Lattice T;
+  if (lay.g != 0 || lay.ncomp != 1 || lay.esize != 4 || !lattice_of(ba, lay, &T)) return false;
+  if (T.E[0] % 4 != 0 || (T.N[1] & 1) || T.pitch % 4 != 0 || T.first != 0 || T.bstride % 4 != 0) return false;
+  SweepGrid G{};
+  for (int d = 0; d < 3; ++d) {
+    if (periodic[d] && (T.N[d] & 1)) return false;
+    G.N[d] = T.N[d];
+    G.E[d] = T.E[d];
+    G.nb[d] = T.nb[d];
+    G.periodic |= periodic[d] ? 1 << d : 0;
+  }
+  G.pitch = T.pitch;
+  G.plane = T.plane;
+  G.bstride = T.bstride;
   G.par0 = (ba.dom.lo[0] + ba.dom.lo[1] + ba.dom.lo[2]) & 1;
   G.mh2 = -(float)(h * h);
   *out = G;
@@ -433,6 +595,30 @@ SweepPlan plan_sweep(std::vector<SweepGrid>& grids, std::vector<SweepGrid>& back
     B.dst = dst;
   }
   return plan;
+}
+
+RestrictPlan plan_restrict(std::vector<RestrictGrid>& grids) {
+  long long cols = 0;
+  for (RestrictGrid& Q : grids) {
+    Q.tiles_xy = ceil_div((Q.g.N[0] / 4) * (Q.g.N[1] / 2), kRestrictThreads);
+    cols += (long long)Q.tiles_xy * Q.g.N[2];
+  }
+  int zc = kRestrictChunk;
+  while (zc > 2 && cols / zc < 8ll * num_sms()) zc /= 2;
+  RestrictPlan p;
+  for (RestrictGrid& Q : grids) {
+    Q.ZC = zc;
+    Q.tile_begin = p.tiles;
+    p.tiles += Q.tiles_xy * ceil_div(Q.g.N[2], zc);
+  }
+  return p;
+}
+
+cudaError_t launch_restrict_f32(const RestrictGrid* grids, int ngrids, const RestrictPlan& p, cudaStream_t s) {
+  if (p.tiles <= 0) return cudaSuccess;
+  launch_k(k_restrict_f32, (unsigned)p.tiles, kRestrictThreads, 0, s, grids, ngrids);
+  count_launches(1);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_sweep_f32(const SweepGrid* grids, int ngrids, const SweepPlan& p, cudaStream_t s) {

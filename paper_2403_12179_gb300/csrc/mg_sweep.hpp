@@ -32,6 +32,36 @@ struct SweepGrid {
   int pad_;
 };
 
+// Boxes of one size on a lattice anchored at the domain's low corner, stored in lattice order (x
+// fastest) at a constant stride; offsets in elements of the fab.
+struct Lattice {
+  int N[3], E[3], nb[3];
+  int pitch, plane;
+  long long bstride, first;  // from one box to the next; the first box's first valid cell
+};
+bool lattice_of(const BoxArray& ba, const FabLayout& lay, Lattice* out);
+
+// Residual + restriction of such a level (mg_sweep.cu): crhs = mean of the 8 children's
+// residuals, cphi = 0.  The coarse fields lie on a lattice of their own.
+struct CoarseField {
+  float* base;  // first valid cell
+  int E[3], nb[3];
+  int pitch, plane;
+  long long bstride;
+};
+struct RestrictGrid {
+  SweepGrid g;  // src = phi, rhs; geometry
+  float mih2;   // -1 / h^2
+  int ZC;       // fine planes of a tile (even)
+  int tiles_xy, tile_begin;
+  CoarseField crhs, cphi;
+};
+struct RestrictPlan {
+  int tiles = 0;
+};
+RestrictPlan plan_restrict(std::vector<RestrictGrid>& grids);
+cudaError_t launch_restrict_f32(const RestrictGrid* grids, int ngrids, const RestrictPlan& p, cudaStream_t s);
+
 // Fills the geometry of a level (not the pointers and the tiling); false if the level cannot
 // be swept this way: boxes of one size on a lattice in lattice order, x extents in whole strips
 // of 4 cells, even y extent, even periodic extents, FP32 without ghosts.

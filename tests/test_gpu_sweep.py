@@ -1,5 +1,5 @@
-"""The whole red + black sweep of FP32 levels on regular box grids (csrc/mg_sweep.cu) against the
-half-sweeps it stands for: the mixed-precision iterates after two outer iterations are equal bit
+"""The whole red + black sweep and the residual + restriction of FP32 levels on regular box grids
+(csrc/mg_sweep.cu) against the half-sweeps and the row kernel they stand for: the mixed-precision iterates after two outer iterations are equal bit
 for bit, alone (levels of at least 2^14 cells are swept whole) and in batches (levels of at least
 2^18 cells together).  The shapes put tile edges everywhere: domains narrower and lower than a
 tile, one strip more than a tile, row counts that are no multiple of a tile's, single boxes and
