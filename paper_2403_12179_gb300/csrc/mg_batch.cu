@@ -170,14 +170,14 @@ struct LevelLists {
   UnitB fab, fba;
   SweepB sweep;
   RestrictB rr_wide;
-  JobB bottom_next;      // bottoms at level l + 1
-  CoarseB coarse_next;   // coarse cycles from level l + 1
 };
 
 struct StepLists {
   std::vector<LevelLists> L;
-  JobB bottom0;
-  CoarseB coarse0;
+  // bottom solves and coarse cycles of all members, whatever their level: one launch each after
+  // the last residual + restriction (the members that end at an earlier level wait for it)
+  JobB bottom;
+  CoarseB coarse;
   SegB resid0, rhsabs0, scale0, correct0;
   TagB fill_phi0;
   int dt = DT_F64;
@@ -243,8 +243,8 @@ void build_lists(Ctx& c, StepLists& S, const std::vector<Member*>& run,
     S.nu2 = H.p.nu2;
     S.inner = H.mixed ? H.p.inner : 1;
     const int nl = (int)H.L.size();
-    if (nl == 1) S.bottom0.add(H);
-    if (H.lc == 0 && nl > 1) S.coarse0.add(H);
+    if (H.lc < nl) S.coarse.add(H);
+    else S.bottom.add(H);
     for (int l = 0; l + 1 < nl && l < H.lc; ++l) {
       LevelData& D = H.L[l];
       LevelLists& LL = S.L[l];
@@ -271,8 +271,6 @@ void build_lists(Ctx& c, StepLists& S, const std::vector<Member*>& run,
       } else {
         LL.prolong.add(D.prolong, m->slot);
       }
-      if (l + 1 == H.lc) LL.coarse_next.add(H);
-      else if (l + 2 == nl) LL.bottom_next.add(H);
     }
     if (H.mixed) {
       S.scale0.add(H.scale0, m->slot);
@@ -305,11 +303,9 @@ void upload_lists(Ctx& c, StepLists& S, Staging& st, cudaStream_t s) {
     LL.sweep.off_ab = st.push(LL.sweep.ab);
     LL.sweep.off_ba = st.push(LL.sweep.ba);
     LL.rr_wide.off = st.push(LL.rr_wide.v);
-    job(LL.bottom_next);
-    cjob(LL.coarse_next);
   }
-  job(S.bottom0);
-  cjob(S.coarse0);
+  job(S.bottom);
+  cjob(S.coarse);
   seg(S.resid0); seg(S.rhsabs0); seg(S.scale0); seg(S.correct0);
   tag(S.fill_phi0);
   size_t need = std::max<size_t>(st.host.size(), 256);
@@ -367,12 +363,6 @@ void enqueue_step(Ctx& c, StepLists& S, const unsigned char* dev, unsigned long 
   }
   // the V-cycle (mixed form: S.inner FP32 cycles, the later ones from the correction so far)
   for (int rep = 0; rep < S.inner; ++rep) {
-    if (!S.bottom0.v.empty())
-      MG_CK(launch_bottom(S.dt, (const BottomJob*)(dev + S.bottom0.off), (int)S.bottom0.v.size(),
-                          S.bottom0.maxN, s));
-    if (!S.coarse0.v.empty())
-      MG_CK(launch_coarse_cycle(S.dt, (const CoarseJob*)(dev + S.coarse0.off),
-                                (int)S.coarse0.v.size(), S.coarse0.smem, s));
     for (int l = 0; l < nlev; ++l) {
       LevelLists& LL = S.L[l];
       if (!LL.rr.total && !LL.rr_wide.plan.tiles) continue;
@@ -382,13 +372,13 @@ void enqueue_step(Ctx& c, StepLists& S, const unsigned char* dev, unsigned long 
       MG_CK(launch_residual_restrict_l(S.dt, mk(LL.rr, dev), LL.rr.total, s, LL.rr.direct));
       MG_CK(launch_restrict_f32((const RestrictGrid*)(dev + LL.rr_wide.off), (int)LL.rr_wide.v.size(),
                                 LL.rr_wide.plan, s));
-      if (!LL.bottom_next.v.empty())
-        MG_CK(launch_bottom(S.dt, (const BottomJob*)(dev + LL.bottom_next.off),
-                            (int)LL.bottom_next.v.size(), LL.bottom_next.maxN, s));
-      if (!LL.coarse_next.v.empty())
-        MG_CK(launch_coarse_cycle(S.dt, (const CoarseJob*)(dev + LL.coarse_next.off),
-                                  (int)LL.coarse_next.v.size(), LL.coarse_next.smem, s));
     }
+    if (!S.bottom.v.empty())
+      MG_CK(launch_bottom(S.dt, (const BottomJob*)(dev + S.bottom.off), (int)S.bottom.v.size(),
+                          S.bottom.maxN, s));
+    if (!S.coarse.v.empty())
+      MG_CK(launch_coarse_cycle(S.dt, (const CoarseJob*)(dev + S.coarse.off), (int)S.coarse.v.size(),
+                                S.coarse.smem, s));
     for (int l = nlev - 1; l >= 0; --l) {
       LevelLists& LL = S.L[l];
       if (!LL.prolong.total && !LL.prolong3.total) continue;

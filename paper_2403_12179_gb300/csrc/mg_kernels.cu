@@ -781,21 +781,36 @@ __global__ void k_set_flat(T* p, long long n, T value) {
     p[i] = value;
 }
 
-// Exact bottom solve: one block per job, rhs gathered to shared memory in FP64.
+// Exact bottom solve: one warp-sized block per 32 rows of a job, rhs gathered to shared memory in
+// FP64.  The FP64 pipe of an SM bounds it (2 N operations a row at 1.68 lanes a clock: 210 rows in one
+// block took 39 us), so the rows are spread over SMs, and 64 matrix loads go ahead of the chain of
+// additions.
+constexpr int kBottomRows = 32;
 template <class T>
-__global__ void k_bottom(const BottomJob* __restrict__ jobs) {
+__global__ void __launch_bounds__(kBottomRows) k_bottom(const BottomJob* __restrict__ jobs, int chunks) {
   pdl_begin();
   extern __shared__ double sb[];
-  const BottomJob J = jobs[blockIdx.x];
+  const BottomJob J = jobs[blockIdx.x / chunks];
+  const int i = (blockIdx.x % chunks) * kBottomRows + threadIdx.x;
+  if (i - (int)threadIdx.x >= J.N) return;
   const T* rhs = (const T*)J.rhs;
   T* phi = (T*)J.phi;
-  for (int j = threadIdx.x; j < J.N; j += blockDim.x) sb[j] = (double)rhs[J.off_rhs[j]];
-  __syncthreads();
-  for (int i = threadIdx.x; i < J.N; i += blockDim.x) {
-    double s = 0.0;
-    for (int j = 0; j < J.N; ++j) s = __dadd_rn(s, __dmul_rn(J.Mt[(long long)j * J.N + i], sb[j]));
-    phi[J.off_phi[i]] = (T)s;
+  for (int j = threadIdx.x; j < J.N; j += kBottomRows) sb[j] = (double)rhs[J.off_rhs[j]];
+  __syncwarp();
+  if (i >= J.N) return;
+  double s = 0.0;
+  constexpr int kAhead = 64;
+  const double* m = J.Mt + i;
+  for (int j0 = 0; j0 < J.N; j0 += kAhead) {
+    double v[kAhead];
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j)
+      if (j0 + j < J.N) v[j] = m[(long long)(j0 + j) * J.N];
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j)
+      if (j0 + j < J.N) s = __dadd_rn(s, __dmul_rn(v[j], sb[j0 + j]));
   }
+  phi[J.off_phi[i]] = (T)s;
 }
 
 template <class T>
@@ -1316,10 +1331,11 @@ cudaError_t launch_prolong_trilinear(int dt, const DRow* rows, int nbox, long lo
 
 cudaError_t launch_bottom(int dt, const BottomJob* jobs, int njobs, int maxN, cudaStream_t s) {
   if (njobs <= 0) return cudaSuccess;
-  int threads = maxN < 32 ? 32 : (maxN > 1024 ? 1024 : (maxN + 31) / 32 * 32);
-  size_t smem = (size_t)maxN * sizeof(double);
-  if (dt == DT_F64) launch_k(k_bottom<double>, njobs, threads, smem, s, jobs);
-  else launch_k(k_bottom<float>, njobs, threads, smem, s, jobs);
+  const int chunks = (maxN + kBottomRows - 1) / kBottomRows;
+  const size_t smem = (size_t)maxN * sizeof(double);
+  const unsigned blocks = (unsigned)(njobs * chunks);
+  if (dt == DT_F64) launch_k(k_bottom<double>, blocks, kBottomRows, smem, s, jobs, chunks);
+  else launch_k(k_bottom<float>, blocks, kBottomRows, smem, s, jobs, chunks);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -73,8 +73,8 @@ struct BottomJob {
 };
 
 // The coarse end of a V-cycle (levels lc .. bottom) in one CTA: every level held densely in
-// shared memory (phi with one ghost layer, then rhs, x fastest), offsets in elements of the
-// level's type.  Level lc's cell i (dense, x fastest) lives at phi[off_phi[i]] and
+// shared memory (phi, then rhs, x fastest; then level lc's residuals at off_res), offsets in
+// elements of the level's type.  Level lc's cell i (dense, x fastest) lives at phi[off_phi[i]] and
 // rhs[off_rhs[i]] in its fabs: phi and rhs are gathered from there and phi scattered back.
 constexpr int kMaxCoarseLevels = 8;
 struct CoarseLevel {
@@ -91,6 +91,7 @@ struct CoarseJob {
   const double* Mt;  // bottom (pseudo-)inverse, transposed, over the last level's cells
   int nlev, nu1, nu2, N;
   int periodic[3];
+  int off_res;
   CoarseLevel lev[kMaxCoarseLevels];
 };
 

@@ -254,10 +254,11 @@ void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
       V.h2 = D.h * D.h;
       V.ih2 = 1.0 / (D.h * D.h);
       V.off_phi = off;
-      off += (V.n[0] + 2) * (V.n[1] + 2) * (V.n[2] + 2);
+      off += V.n[0] * V.n[1] * V.n[2];
       V.off_rhs = off;
       off += V.n[0] * V.n[1] * V.n[2];
     }
+    C.off_res = off;
     H.csmem = smem;
     MG_CK(coarse_opt_in(H.dt, smem));
     H.cjob = c.upload(&C, sizeof C, s);
