@@ -783,8 +783,8 @@ __global__ void k_set_flat(T* p, long long n, T value) {
 
 // Exact bottom solve: one warp-sized block per 32 rows of a job, rhs gathered to shared memory in
 // FP64.  The FP64 pipe of an SM bounds it (2 N operations a row at 1.68 lanes a clock: 210 rows in one
-// block took 39 us), so the rows are spread over SMs, and 64 matrix loads go ahead of the chain of
-// additions.
+// block took 39 us, 32 spread over SMs; ncu, cold), with 16 matrix loads ahead of the chain of
+// additions (64 ahead, 160 registers: 43 us).
 constexpr int kBottomRows = 32;
 template <class T>
 __global__ void __launch_bounds__(kBottomRows) k_bottom(const BottomJob* __restrict__ jobs, int chunks) {
@@ -799,17 +799,8 @@ __global__ void __launch_bounds__(kBottomRows) k_bottom(const BottomJob* __restr
   __syncwarp();
   if (i >= J.N) return;
   double s = 0.0;
-  constexpr int kAhead = 64;
-  const double* m = J.Mt + i;
-  for (int j0 = 0; j0 < J.N; j0 += kAhead) {
-    double v[kAhead];
-#pragma unroll
-    for (int j = 0; j < kAhead; ++j)
-      if (j0 + j < J.N) v[j] = m[(long long)(j0 + j) * J.N];
-#pragma unroll
-    for (int j = 0; j < kAhead; ++j)
-      if (j0 + j < J.N) s = __dadd_rn(s, __dmul_rn(v[j], sb[j0 + j]));
-  }
+#pragma unroll 16
+  for (int j = 0; j < J.N; ++j) s = __dadd_rn(s, __dmul_rn(J.Mt[(long long)j * J.N + i], sb[j]));
   phi[J.off_phi[i]] = (T)s;
 }
 

@@ -75,3 +75,27 @@ def test_batched_sweeps_equal_single_solves():
             np.testing.assert_array_equal(got.view(np.int64), _dense(ctx, phi, n).view(np.int64))
     finally:
         mg.mg_finalize(ctx)
+
+
+@pytest.mark.parametrize("n,ragged,even", [((48, 40, 56), (32, 24, 32), (8, 8, 8)), ((96, 48, 32), (40, 48, 24), (32, 16, 16))])
+@pytest.mark.parametrize("per", [(0, 0, 0), (1, 1, 1), (0, 1, 0)])
+@pytest.mark.parametrize("precision", [mg.MG_PREC_F64, mg.MG_PREC_MIXED])
+def test_ragged_boxes_equal_even_ones(n, ragged, even, per, precision):
+    """Boxes of several sizes (whose internal levels are laid out as one box) against boxes of one size,
+    alone and in a batch: the same iterates bit for bit, with and without direct reads."""
+    ctx = mg.mg_init(0)
+    try:
+        got = []
+        for box, direct, batch in ((ragged, 1, False), (ragged, 1, True), (ragged, 0, False), (even, 1, False)):
+            rhs, phi, bc = _problem(ctx, n, box, per, 23)
+            opt = mg.make_options(precision=precision, fixed_vcycles=2, direct_reads=direct)
+            if batch:
+                mg.mg_solve_batch(ctx, [rhs], [phi], [bc], 1e-10, opt)
+            else:
+                mg.mg_solve(ctx, rhs, phi, bc, 1e-10, opt)
+            got.append(_dense(ctx, phi, n))
+        assert np.abs(got[0]).max() > 0
+        for g in got[1:]:
+            np.testing.assert_array_equal(got[0].view(np.int64), g.view(np.int64))
+    finally:
+        mg.mg_finalize(ctx)
