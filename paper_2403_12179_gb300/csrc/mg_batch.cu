@@ -128,9 +128,11 @@ struct SweepB {
   std::vector<SweepGrid> ab, ba;
   SweepPlan plan;
   size_t off_ab = 0, off_ba = 0;
+  bool coarse = true;  // every member's sweep can add the prolongation
   void add(const LevelData& D) {
     ab.push_back(D.sweep_ab);
     ba.push_back(D.sweep_ba);
+    coarse = coarse && D.sweep_ab.coarse.base;
   }
   void finish() {
     if (!ab.empty()) plan = plan_sweep(ab, ba);
@@ -182,6 +184,7 @@ struct StepLists {
   TagB fill_phi0;
   int dt = DT_F64;
   bool mixed = false;
+  bool zero0 = false;  // every member's level 0 starts from zero in its sweeps
   int nu1 = 2, nu2 = 2, inner = 1;  // (the members of one step share them)
 };
 
@@ -235,8 +238,16 @@ void build_lists(Ctx& c, StepLists& S, const std::vector<Member*>& run,
   for (Member* m : run)
     for (int l = 0; l + 1 < (int)m->H->L.size() && l < m->H->lc; ++l)
       if (m->H->L[l].wide) wide[l] += m->H->L[l].cells();
+  auto swept = [&](const Hierarchy& H, int l) {
+    return l + 1 < (int)H.L.size() && l < H.lc && H.L[l].wide && wide[l] >= kSweepMinCellsBatch;
+  };
+  for (Member* m : run)  // (a level's sweeps add the prolongation only if all of them can)
+    for (int l = 0; l < (int)m->H->L.size(); ++l)
+      if (swept(*m->H, l)) S.L[l].sweep.coarse = S.L[l].sweep.coarse && m->H->L[l].sweep_ab.coarse.base;
+  S.zero0 = !run.empty();
   for (Member* m : run) {
     Hierarchy& H = *m->H;
+    S.zero0 = S.zero0 && swept(H, 0) && H.p.nu1 >= 2;
     S.dt = H.dt;
     S.mixed = H.mixed;
     S.nu1 = H.p.nu1;
@@ -254,7 +265,7 @@ void build_lists(Ctx& c, StepLists& S, const std::vector<Member*>& run,
         LL.fill2_phi.add(fill_plan(c, *D.phi, &H.bc, 2), D.phi->base);
         LL.fill2_phi2.add(fill_plan(c, *D.phi2, &H.bc, 2), D.phi2->base);
         LL.fill_rhs.add(fill_plan(c, *D.rhs, &H.bc, 1), D.rhs->base);
-      } else if (D.wide && wide[l] >= kSweepMinCellsBatch) {
+      } else if (swept(H, l)) {
         LL.sweep.add(D);
       } else {
         LL.half.add(D.smooth, m->slot);
@@ -262,13 +273,18 @@ void build_lists(Ctx& c, StepLists& S, const std::vector<Member*>& run,
       }
       if (!D.direct) LL.fill1_all.add(fill_plan(c, *D.phi, &H.bc, 1), D.phi->base);
       LL.half_all.add(D.smooth, m->slot);
-      if (D.wide_rr) LL.rr_wide.v.push_back(D.rr_grid);
-      else LL.rr.add(D.rr, m->slot);
+      if (D.wide_rr) {
+        LL.rr_wide.v.push_back(D.rr_grid);
+        // (a coarser level that starts its sweeps from zero needs no zeros)
+        if (swept(H, l + 1) && H.p.nu1 >= 2) LL.rr_wide.v.back().cphi.base = nullptr;
+      } else {
+        LL.rr.add(D.rr, m->slot);
+      }
       if (H.p.prolong == MG_PROLONG_TRILINEAR) {
         LL.prolong3.add(D.prolong, m->slot);
         FabObj& cphi = *H.L[l + 1].phi;
         LL.fill_c.add(fill_plan(c, cphi, &H.bc, 1), cphi.base);
-      } else {
+      } else if (!(swept(H, l) && LL.sweep.coarse && H.p.nu2 >= 2)) {
         LL.prolong.add(D.prolong, m->slot);
       }
     }
@@ -322,7 +338,7 @@ void fill_l(Ctx& c, int dt, const TagB& b, const unsigned char* dev, cudaStream_
   if (b.total) MG_CK(launch_copy_tags_l(dt, mk(b, dev), b.total, 1, s));
 }
 
-void smooth_l(Ctx& c, StepLists& S, LevelLists& LL, int sweeps, const unsigned char* dev,
+void smooth_l(Ctx& c, StepLists& S, LevelLists& LL, int sweeps, int start, const unsigned char* dev,
               int* err, cudaStream_t s) {
   int k = 0;
   for (; k + 1 < sweeps; k += 2) {
@@ -334,9 +350,12 @@ void smooth_l(Ctx& c, StepLists& S, LevelLists& LL, int sweeps, const unsigned c
       MG_CK(launch_rbgs_fused_l(S.dt, mk(LL.fba, dev), LL.fba.total, LL.fba.ty, LL.fba.depth,
                                 LL.fba.mp, LL.fba.mpr, LL.fba.rhs_smem, err, s));
     }
-    if (LL.sweep.plan.tiles)
-      for (size_t off : {LL.sweep.off_ab, LL.sweep.off_ba})
-        MG_CK(launch_sweep_f32((const SweepGrid*)(dev + off), (int)LL.sweep.ab.size(), LL.sweep.plan, s));
+    if (LL.sweep.plan.tiles) {
+      const int n = (int)LL.sweep.ab.size();
+      MG_CK(launch_sweep_f32((const SweepGrid*)(dev + LL.sweep.off_ab), n, LL.sweep.plan,
+                             k == 0 ? start : SWEEP_SOURCE, s));
+      MG_CK(launch_sweep_f32((const SweepGrid*)(dev + LL.sweep.off_ba), n, LL.sweep.plan, SWEEP_SOURCE, s));
+    }
     if (LL.half.total)
       for (int j = 0; j < 2; ++j)
         for (int color = 0; color < 2; ++color) {
@@ -359,7 +378,7 @@ void enqueue_step(Ctx& c, StepLists& S, const unsigned char* dev, unsigned long 
   int* err = (int*)c.d_err->p;
   const int nlev = (int)S.L.size();
   if (S.mixed && S.scale0.total) {
-    MG_CK(launch_scale_residual_f32_l(mk(S.scale0, dev), S.scale0.total, norms, s));
+    MG_CK(launch_scale_residual_f32_l(mk(S.scale0, dev), S.scale0.total, norms, s, !S.zero0));
   }
   // the V-cycle (mixed form: S.inner FP32 cycles, the later ones from the correction so far)
   for (int rep = 0; rep < S.inner; ++rep) {
@@ -367,7 +386,7 @@ void enqueue_step(Ctx& c, StepLists& S, const unsigned char* dev, unsigned long 
       LevelLists& LL = S.L[l];
       if (!LL.rr.total && !LL.rr_wide.plan.tiles) continue;
       if (LL.fill_rhs.total) fill_l(c, S.dt, LL.fill_rhs, dev, s);
-      smooth_l(c, S, LL, S.nu1, dev, err, s);
+      smooth_l(c, S, LL, S.nu1, l > 0 || (rep == 0 && S.zero0) ? SWEEP_ZERO : SWEEP_SOURCE, dev, err, s);
       fill_l(c, S.dt, LL.fill1_all, dev, s);
       MG_CK(launch_residual_restrict_l(S.dt, mk(LL.rr, dev), LL.rr.total, s, LL.rr.direct));
       MG_CK(launch_restrict_f32((const RestrictGrid*)(dev + LL.rr_wide.off), (int)LL.rr_wide.v.size(),
@@ -381,13 +400,13 @@ void enqueue_step(Ctx& c, StepLists& S, const unsigned char* dev, unsigned long 
                                 S.coarse.smem, s));
     for (int l = nlev - 1; l >= 0; --l) {
       LevelLists& LL = S.L[l];
-      if (!LL.prolong.total && !LL.prolong3.total) continue;
+      if (!LL.prolong.total && !LL.prolong3.total && !LL.sweep.plan.tiles) continue;
       if (LL.prolong.total) MG_CK(launch_prolong_add_l(S.dt, mk(LL.prolong, dev), LL.prolong.total, s));
       if (LL.prolong3.total) {
         fill_l(c, S.dt, LL.fill_c, dev, s);
         MG_CK(launch_prolong_trilinear_l(S.dt, mk(LL.prolong3, dev), LL.prolong3.total, s));
       }
-      smooth_l(c, S, LL, S.nu2, dev, err, s);
+      smooth_l(c, S, LL, S.nu2, LL.sweep.coarse ? SWEEP_PROLONG : SWEEP_SOURCE, dev, err, s);
     }
   }
   if (S.mixed && S.correct0.total)

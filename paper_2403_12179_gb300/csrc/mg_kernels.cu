@@ -872,7 +872,8 @@ constexpr int kScaleCells = 4;
 template <int G>
 __global__ void __launch_bounds__(kThreads) k_scale_residual_f32(SegList L, long long nrows,
                                                                  long long per,
-                                                                 const unsigned long long* norms) {
+                                                                 const unsigned long long* norms,
+                                                                 bool zero) {
   pdl_begin();
   const int sub = threadIdx.x & (G - 1);
   for_rows<32 / G>(L, nrows, per, [&](const DRow& R, long long lr, int slot) {
@@ -896,7 +897,7 @@ __global__ void __launch_bounds__(kThreads) k_scale_residual_f32(SegList L, long
         float f;
         if (!bits::scale_to_f32(v[k], e, &f)) f = __double2float_rn(__dmul_rn(v[k], down));
         r32[x + G * k] = f;
-        e32[x + G * k] = 0.0f;
+        if (zero) e32[x + G * k] = 0.0f;
       }
     }
   });
@@ -1239,13 +1240,13 @@ cudaError_t launch_maxabs_l(int dt, const SegList& L, long long nrows, unsigned 
 }
 
 cudaError_t launch_scale_residual_f32_l(const SegList& L, long long nrows,
-                                        const unsigned long long* norms, cudaStream_t s) {
+                                        const unsigned long long* norms, cudaStream_t s, bool zero) {
   if (nrows <= 0) return cudaSuccess;
   const int G = group_lanes(L.width, kScaleCells, 8, 32);
   const Grid g = row_grid(nrows, row_blocks_per_sm(L.width), kWarps * (32 / G));
-  if (G == 32) launch_k(k_scale_residual_f32<32>, g.blocks, kThreads, 0, s, L, nrows, g.per, norms);
-  else if (G == 16) launch_k(k_scale_residual_f32<16>, g.blocks, kThreads, 0, s, L, nrows, g.per, norms);
-  else launch_k(k_scale_residual_f32<8>, g.blocks, kThreads, 0, s, L, nrows, g.per, norms);
+  if (G == 32) launch_k(k_scale_residual_f32<32>, g.blocks, kThreads, 0, s, L, nrows, g.per, norms, zero);
+  else if (G == 16) launch_k(k_scale_residual_f32<16>, g.blocks, kThreads, 0, s, L, nrows, g.per, norms, zero);
+  else launch_k(k_scale_residual_f32<8>, g.blocks, kThreads, 0, s, L, nrows, g.per, norms, zero);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1376,8 +1377,9 @@ cudaError_t launch_maxabs(int dt, const DRow* rows, int nbox, long long nrows,
 }
 
 cudaError_t launch_scale_residual_f32(const DRow* rows, int nbox, long long nrows,
-                                      const unsigned long long* norms, cudaStream_t s, int width) {
-  return launch_scale_residual_f32_l(one_seg(rows, nbox, 0, width), nrows, norms, s);
+                                      const unsigned long long* norms, cudaStream_t s, int width,
+                                      bool zero) {
+  return launch_scale_residual_f32_l(one_seg(rows, nbox, 0, width), nrows, norms, s, zero);
 }
 
 cudaError_t launch_correct_add(const DRow* rows, int nbox, long long nrows,

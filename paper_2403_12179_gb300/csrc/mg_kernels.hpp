@@ -324,10 +324,10 @@ cudaError_t launch_maxabs(int dt, const DRow* rows, int nbox, long long nrows,
 
 // Mixed precision.  v[0] = r (FP64 residual stored by the norm check), c[0] = r32 out,
 // c[1] = e32 out (FP32 views with the same box geometry): r32 = float(r * 2^-e) with
-// 2^e <= norms[solve] < 2^(e+1), e32 = 0.
+// 2^e <= norms[solve] < 2^(e+1), e32 = 0 (zero false: e32 is left alone).
 cudaError_t launch_scale_residual_f32(const DRow* rows, int nbox, long long nrows,
                                       const unsigned long long* norms, cudaStream_t s,
-                                      int width = 0);
+                                      int width = 0, bool zero = true);
 // v[0] = phi (FP64), c[0] = e (FP32 view, same geometry): phi = phi + 2^e * double(e32) with
 // the 2^e of the scale above.
 cudaError_t launch_correct_add(const DRow* rows, int nbox, long long nrows,
@@ -354,7 +354,8 @@ cudaError_t launch_fp64_probe(int iters, long long* lane_ops, cudaStream_t s);
 cudaError_t launch_maxabs_l(int dt, const SegList& L, long long nrows, unsigned long long* norms,
                             cudaStream_t s);
 cudaError_t launch_scale_residual_f32_l(const SegList& L, long long nrows,
-                                        const unsigned long long* norms, cudaStream_t s);
+                                        const unsigned long long* norms, cudaStream_t s,
+                                        bool zero = true);
 cudaError_t launch_correct_add_l(const SegList& L, long long nrows, const unsigned long long* norms,
                                  cudaStream_t s);
 cudaError_t launch_rbgs_fused_l(int dt, const UnitList& L, long long nunits, int ty, int depth,

@@ -115,12 +115,15 @@ void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
       D.sweep_ab.src = (const float*)D.phi->base;
       D.sweep_ab.rhs = (const float*)D.rhs->base;
       D.sweep_ab.dst = (float*)D.phi2->base;
+      const bool coarse = coarse_field(*H.L[l + 1].phi, &D.sweep_ab.coarse);
       D.sweep_ba = D.sweep_ab;
       D.sweep_ba.src = (const float*)D.phi2->base;
       D.sweep_ba.dst = (float*)D.phi->base;
       if (D.cells() >= kSweepMinCells) {
         std::vector<SweepGrid> ab{D.sweep_ab}, ba{D.sweep_ba};
         D.sweep_plan = plan_sweep(ab, ba);
+        D.zero_start = H.p.nu1 >= 2;
+        D.add_start = H.p.nu2 >= 2 && coarse;
         ab.push_back(ba[0]);
         D.sweep_dev = c.upload(ab.data(), ab.size() * sizeof(SweepGrid), s);
       }
@@ -136,11 +139,6 @@ void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
       D.rr_grid.mih2 = -(float)(1.0 / (D.h * D.h));
       D.wide_rr = (D.bao->ba.dom.len(2) & 1) == 0 && coarse_field(*C.rhs, &D.rr_grid.crhs) &&
                   coarse_field(*C.phi, &D.rr_grid.cphi);
-      if (D.wide_rr) {
-        std::vector<RestrictGrid> q{D.rr_grid};
-        D.rr_plan = plan_restrict(q);
-        D.rr_dev = c.upload(q.data(), sizeof(RestrictGrid), s);
-      }
     }
     if (l + 1 < nl) {
       const LevelData& C = H.L[l + 1];
@@ -278,6 +276,15 @@ void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
     H.cjob = c.upload(&C, sizeof C, s);
     H.lc = l;
     break;
+  }
+  for (int l = 0; l + 1 < nl; ++l) {
+    LevelData& D = H.L[l];
+    if (!D.wide_rr) continue;
+    std::vector<RestrictGrid> q{D.rr_grid};
+    // (a coarser level that starts its sweeps from zero needs no zeros)
+    if (H.L[l + 1].zero_start && l + 1 < H.lc) q[0].cphi.base = nullptr;
+    D.rr_plan = plan_restrict(q);
+    D.rr_dev = c.upload(q.data(), sizeof(RestrictGrid), s);
   }
   // fill plans must exist before any graph capture
   for (auto& D : H.L) {
@@ -451,16 +458,17 @@ namespace {
 // the cells it updates there (the caller adds the red cells).  store_last: the final (black)
 // half-sweep also stores the residuals of the cells it updates (level 0: H.store0), for the
 // residual + restriction that follows.
+// start: what the first whole sweep starts from (wide levels with launches of their own).
 void smooth(Ctx& c, Hierarchy& H, LevelData& D, int sweeps, cudaStream_t s,
             unsigned long long* last_norm = nullptr, bool time_first = false,
-            bool skip_first_red = false, bool store_last = false) {
+            bool skip_first_red = false, bool store_last = false, int start = SWEEP_SOURCE) {
   int k = 0;
   if (D.sweep_plan.tiles) {
     // pairs of sweeps: phi -> phi2 -> phi
     const SweepGrid* g = (const SweepGrid*)D.sweep_dev->p;
     for (; k + 1 < sweeps; k += 2) {
-      MG_CK(launch_sweep_f32(g, 1, D.sweep_plan, s));
-      MG_CK(launch_sweep_f32(g + 1, 1, D.sweep_plan, s));
+      MG_CK(launch_sweep_f32(g, 1, D.sweep_plan, k == 0 ? start : SWEEP_SOURCE, s));
+      MG_CK(launch_sweep_f32(g + 1, 1, D.sweep_plan, SWEEP_SOURCE, s));
     }
   }
   if (D.fused) {
@@ -490,8 +498,9 @@ void smooth(Ctx& c, Hierarchy& H, LevelData& D, int sweeps, cudaStream_t s,
     }
 }
 
+// zero0: level 0 starts from zero (the first FP32 cycle of a mixed outer iteration).
 void enqueue_vcycle(Ctx& c, Hierarchy& H, cudaStream_t s, unsigned long long* norm0 = nullptr,
-                    bool skip_first_red = false) {
+                    bool skip_first_red = false, bool zero0 = false) {
   const int nl = (int)H.L.size();
   const int top = H.lc < nl ? H.lc : nl - 1;  // levels below `top` run stage by stage
   for (int l = 0; l < top; ++l) {
@@ -501,7 +510,7 @@ void enqueue_vcycle(Ctx& c, Hierarchy& H, cudaStream_t s, unsigned long long* no
     // residuals come from the last pre-smoothing half-sweep
     const bool stored = l == 0 && H.stored0;
     smooth(c, H, D, H.p.nu1, s, nullptr, l == 0 && H.graph_timed, l == 0 && skip_first_red,
-           stored);
+           stored, D.zero_start && (l > 0 || zero0) ? SWEEP_ZERO : SWEEP_SOURCE);
     if (!D.direct) launch_fill(c, *D.phi, &H.bc, s, 1);
     if (D.wide_rr)
       MG_CK(launch_restrict_f32((const RestrictGrid*)D.rr_dev->p, 1, D.rr_plan, s));
@@ -517,11 +526,12 @@ void enqueue_vcycle(Ctx& c, Hierarchy& H, cudaStream_t s, unsigned long long* no
       launch_fill(c, *H.L[l + 1].phi, &H.bc, s, 1);  // the coarse neighbours it reads
       MG_CK(launch_prolong_trilinear(H.dt, D.prolong.rows(), D.prolong.nbox, D.prolong.nrows, s,
                                      D.prolong.width));
-    } else {
+    } else if (!D.add_start) {
       MG_CK(launch_prolong_add(H.dt, D.prolong.rows(), D.prolong.nbox, D.prolong.nrows, s,
                                D.prolong.width));
     }
-    smooth(c, H, D, H.p.nu2, s, l == 0 ? norm0 : nullptr);
+    smooth(c, H, D, H.p.nu2, s, l == 0 ? norm0 : nullptr, false, false, false,
+           D.add_start ? SWEEP_PROLONG : SWEEP_SOURCE);
   }
 }
 
@@ -544,7 +554,7 @@ void enqueue_step(Ctx& c, Hierarchy& H, cudaStream_t s, int variant) {
   }
   if (H.mixed)  // the FP32 right-hand side from the residual of the last norm check; e = 0
     MG_CK(launch_scale_residual_f32(H.scale0.rows(), H.scale0.nbox, H.scale0.nrows, dn, s,
-                                    H.scale0.width));
+                                    H.scale0.width, !(H.L[0].zero_start && H.lc > 0)));
   // FP64 with half-sweeps on the finest level: the cycle's last (black) half-sweep there
   // takes the residual norm of the cells it updates, and only the red cells need a residual
   // pass; the values are those of a full residual pass
@@ -557,7 +567,7 @@ void enqueue_step(Ctx& c, Hierarchy& H, cudaStream_t s, int variant) {
       if (per[d] && (H.L[0].bao->ba.dom.len(d) & 1)) split_norm = false;
   }
   if (split_norm) MG_CK(cudaMemsetAsync(dn, 0, 8, s));
-  enqueue_vcycle(c, H, s, split_norm ? dn : nullptr);
+  enqueue_vcycle(c, H, s, split_norm ? dn : nullptr, false, H.mixed);
   if (H.mixed)  // the further FP32 cycles of the outer iteration, from the correction so far
     for (int k = 1; k < H.p.inner; ++k) enqueue_vcycle(c, H, s, nullptr);
   if (H.mixed)

@@ -26,6 +26,9 @@ struct LevelData {
   DevBufP rr_dev;
   RestrictPlan rr_plan{};
   SweepPlan sweep_plan{};            // no tiles: too small for a launch of its own
+  // the first pre-smoothing sweep starts from zero without reading phi (nobody zeroes it), the first
+  // post-smoothing sweep adds the prolongation (no kernel of its own): launches of their own sweep
+  bool zero_start = false, add_start = false;
   long long cells() const { return bao->ba.dom.npts(); }
   std::shared_ptr<FabObj> phi2;
   FusedTable f_ab, f_ba;

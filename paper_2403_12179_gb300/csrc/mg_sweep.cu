@@ -22,7 +22,9 @@
 //     (no barrier for it).
 // Measured on GB300 (CUDA events, 12 bytes a cell): 512^3 in boxes of 128^3 316 us (5.1 TB/s, 75%
 // of the copy rate; the TMA sweep of mg_fused.cu took 389 us plus two fills of two layers), 60
-// periodic 96^3 levels in boxes of 32^3 121 us (two half-sweeps 324 us).  One row a thread took
+// periodic 96^3 levels in boxes of 32^3 121 us (two half-sweeps 324 us); inside the 512^3 mixed solve
+// 265 us (ncu; 90% of the copy rate), 172 us starting from zero (phi not read), 334 us adding the
+// prolongation (whose own kernel took 214).  One row a thread took
 // 352 us at 512^3 (62% of the shared-memory wavefronts, 54% more instructions a cell in
 // barriers and addresses); selecting colours at run time instead of by the unrolled plane
 // parity took 441 us (100 instructions a cell against 38).
@@ -78,25 +80,39 @@ __device__ __forceinline__ float4 flip4(float4 v, uint32_t m) {
 __device__ __forceinline__ float2 even2(const float4& v) { return make_float2(v.x, v.z); }
 __device__ __forceinline__ float2 odd2(const float4& v) { return make_float2(v.y, v.w); }
 
+// The grid of this block's tile to shared memory, a word a thread.
+template <class G>
+__device__ __forceinline__ void load_grid(G* to, const G* __restrict__ grids, int ng) {
+  int lo = 0, hi = ng - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (grids[mid].tile_begin <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
+  }
+  static_assert(sizeof(G) % 8 == 0, "");
+  for (int i = threadIdx.x; i < (int)(sizeof(G) / 8); i += blockDim.x)
+    reinterpret_cast<long long*>(to)[i] = reinterpret_cast<const long long*>(grids + lo)[i];
+}
+
 template <int V>
 struct Int {
   static constexpr int value = V;
 };
 
+__device__ __forceinline__ void cpa4(uint32_t d, const void* s) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(s) : "memory");
+}
+__device__ __forceinline__ float4 add_pairs(const float4& v, const float2& c) {  // c: one value a pair
+  return make_float4(__fadd_rn(v.x, c.x), __fadd_rn(v.y, c.x), __fadd_rn(v.z, c.y), __fadd_rn(v.w, c.y));
+}
+
+template <int START>
 __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
     k_sweep_f32(const SweepGrid* __restrict__ grids, int ng) {
   pdl_begin();
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ long long zoff[kMaxPlanes];
+  __shared__ long long zoff[kMaxPlanes], czoff[START == SWEEP_PROLONG ? kMaxPlanes : 1];
   __shared__ SweepGrid Gs;
-  if (threadIdx.x == 0) {
-    int lo = 0, hi = ng - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (grids[mid].tile_begin <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
-    }
-    Gs = grids[lo];
-  }
+  load_grid(&Gs, grids, ng);
   __syncthreads();
   const SweepGrid& G = Gs;
   const int t = blockIdx.x - G.tile_begin;
@@ -156,6 +172,11 @@ __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
     }
     const int bz = p / G.E[2];
     zoff[q] = ((long long)bz * G.nb[0] * G.nb[1] * G.bstride + (long long)(p - bz * G.E[2]) * G.plane) * 4;
+    if (START == SWEEP_PROLONG) {
+      const CoarseField& C = G.coarse;
+      const int Z = p >> 1, cz = Z / C.E[2];
+      czoff[q] = ((long long)cz * C.nb[0] * C.nb[1] * C.bstride + (long long)(Z - cz * C.E[2]) * C.plane) * 4;
+    }
   }
   __syncthreads();
   const int bx = gx / G.E[0], by = gy / G.E[1], byB = gyB / G.E[1];
@@ -166,6 +187,15 @@ __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
   const char* src = (const char*)G.src + tcol;
   const char* rhs = (const char*)G.rhs + tcol;
   char* dst = (char*)G.dst + tcol;
+  // the strip's two parents (rows A and B share them), and their slots in the ring
+  const char* crs = nullptr;
+  const uint32_t cring = ring + 4 * kDepth * rst - tid * 8, cst = kst;
+  if (START == SWEEP_PROLONG) {
+    const CoarseField& C = G.coarse;
+    const int X = gx >> 1, Y = gy >> 1, cx = X / C.E[0], cy = Y / C.E[1];
+    crs = (const char*)C.base + ((long long)(cy * C.nb[0] + cx) * C.bstride +
+                                 (long long)(Y - cy * C.E[1]) * C.pitch + (X - cx * C.E[0])) * 4;
+  }
   const float mh2 = G.mh2;
   constexpr float inv6 = 1.0f / 6.0f;
   const int s_first = z0 - 1, nit = z1 - z0 + 2;  // stages: red of planes z0 - 1 ... z1
@@ -179,16 +209,27 @@ __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
   Row RA, RB;
   {
     const uint32_t n0 = neg ^ plane_neg(s_first - 1), n1 = neg ^ plane_neg(s_first);
-    const float4 A0 = flip4(*reinterpret_cast<const float4*>(src + zoff[0]), n0);
-    const float4 A1 = flip4(*reinterpret_cast<const float4*>(src + zoff[1]), n1);
-    const float4 B0 = flip4(*reinterpret_cast<const float4*>(src + dB + zoff[0]), n0);
-    const float4 B1 = flip4(*reinterpret_cast<const float4*>(src + dB + zoff[1]), n1);
+    auto first = [&](long long dy, int q) {  // phi of plane z0 - 2 + q
+      if (START == SWEEP_ZERO) return make_float4(0.f, 0.f, 0.f, 0.f);
+      const float4 v = *reinterpret_cast<const float4*>(src + dy + zoff[q]);
+      if (START == SWEEP_SOURCE) return v;
+      const float* c = reinterpret_cast<const float*>(crs + czoff[q]);
+      return add_pairs(v, make_float2(c[0], c[1]));
+    };
+    const float4 A0 = flip4(first(0, 0), n0), A1 = flip4(first(0, 1), n1);
+    const float4 B0 = flip4(first(dB, 0), n0), B1 = flip4(first(dB, 1), n1);
 #pragma unroll
     for (int d = 0; d < kDepth; ++d) {
-      cpa16(ring + (4 * d) * rst, src + zoff[2 + d]);
-      cpa16(ring + (4 * d + 1) * rst, src + dB + zoff[2 + d]);
+      if (START != SWEEP_ZERO) {
+        cpa16(ring + (4 * d) * rst, src + zoff[2 + d]);
+        cpa16(ring + (4 * d + 1) * rst, src + dB + zoff[2 + d]);
+      }
       cpa16(ring + (4 * d + 2) * rst, rhs + zoff[1 + d]);
       cpa16(ring + (4 * d + 3) * rst, rhs + dB + zoff[1 + d]);
+      if (START == SWEEP_PROLONG) {
+        cpa4(cring + d * cst, crs + czoff[2 + d]);
+        cpa4(cring + d * cst + 4, crs + czoff[2 + d] + 4);
+      }
       cpa_commit();
     }
     // row A at plane s_first has parity P0 (red at odd places if 1), row B the other
@@ -205,7 +246,7 @@ __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
     sts2(me + 2 * kst, zero);
     sts2(me + 3 * kst, zero);
   }
-  uint32_t slot = ring;
+  uint32_t slot = ring, cslot = cring;
   const uint32_t slot_end = ring + 4 * kDepth * rst;
   __syncthreads();
   auto stage = [&](auto Pc, auto Kc, int k) {
@@ -213,14 +254,33 @@ __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
     const int s = s_first + k;
     asm volatile("cp.async.wait_group %0;" ::"n"(kDepth - 1) : "memory");
     const uint32_t n1 = neg ^ plane_neg(s + 1);
-    const float4 pA = flip4(lds4(slot), n1), pB = flip4(lds4(slot + rst), n1);  // phi of s + 1
-    const float4 fA = lds4(slot + 2 * rst), fB = lds4(slot + 3 * rst);          // rhs of s
+    float4 pA = make_float4(0.f, 0.f, 0.f, 0.f), pB = pA;  // phi of s + 1
+    if (START != SWEEP_ZERO) {
+      pA = lds4(slot);
+      pB = lds4(slot + rst);
+    }
+    if (START == SWEEP_PROLONG) {
+      const float2 c = lds2(cslot);
+      pA = add_pairs(pA, c);
+      pB = add_pairs(pB, c);
+    }
+    pA = flip4(pA, n1);
+    pB = flip4(pB, n1);
+    const float4 fA = lds4(slot + 2 * rst), fB = lds4(slot + 3 * rst);  // rhs of s
     {
-      const long long o = zoff[k + 2 + kDepth], o1 = zoff[k + 1 + kDepth];
-      cpa16(slot, src + o);
-      cpa16(slot + rst, src + dB + o);
+      const int q = k + 2 + kDepth;
+      const long long o = zoff[q], o1 = zoff[q - 1];
+      if (START != SWEEP_ZERO) {
+        cpa16(slot, src + o);
+        cpa16(slot + rst, src + dB + o);
+      }
       cpa16(slot + 2 * rst, rhs + o1);
       cpa16(slot + 3 * rst, rhs + dB + o1);
+      if (START == SWEEP_PROLONG) {
+        cpa4(cslot, crs + czoff[q]);
+        cpa4(cslot + 4, crs + czoff[q] + 4);
+        cslot = cslot == cring + (kDepth - 1) * cst ? cring : cslot + cst;
+      }
       cpa_commit();
     }
     slot = slot + 4 * rst == slot_end ? ring : slot + 4 * rst;
@@ -297,14 +357,7 @@ __global__ void __launch_bounds__(kRestrictThreads, 4)
   pdl_begin();
   __shared__ long long zoff[kRestrictChunk + 3], coff[2][kRestrictChunk / 2];
   __shared__ RestrictGrid Gs;
-  if (threadIdx.x == 0) {
-    int lo = 0, hi = ng - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (grids[mid].tile_begin <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
-    }
-    Gs = grids[lo];
-  }
+  load_grid(&Gs, grids, ng);
   __syncthreads();
   const RestrictGrid& Q = Gs;
   const SweepGrid& G = Q.g;
@@ -621,14 +674,18 @@ cudaError_t launch_restrict_f32(const RestrictGrid* grids, int ngrids, const Res
   return cudaGetLastError();
 }
 
-cudaError_t launch_sweep_f32(const SweepGrid* grids, int ngrids, const SweepPlan& p, cudaStream_t s) {
+cudaError_t launch_sweep_f32(const SweepGrid* grids, int ngrids, const SweepPlan& p, int start,
+                             cudaStream_t s) {
   if (p.tiles <= 0) return cudaSuccess;
+  const auto k = start == SWEEP_ZERO      ? k_sweep_f32<SWEEP_ZERO>
+                 : start == SWEEP_PROLONG ? k_sweep_f32<SWEEP_PROLONG>
+                                          : k_sweep_f32<SWEEP_SOURCE>;
   // published pairs: 2 stages x 2 colours x 2 rows of 8 bytes; ring: kDepth planes of 2 rows of
-  // phi and rhs, 16 bytes each
-  const size_t smem = (size_t)p.threads * (64 + 64 * kDepth);
-  cudaError_t e = opt_in_smem((const void*)k_sweep_f32, smem);
+  // phi and rhs, 16 bytes each, and of the two parents
+  const size_t smem = (size_t)p.threads * (64 + (64 + (start == SWEEP_PROLONG ? 8 : 0)) * kDepth);
+  cudaError_t e = opt_in_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
-  launch_k(k_sweep_f32, (unsigned)p.tiles, p.threads, smem, s, grids, ngrids);
+  launch_k(k, (unsigned)p.tiles, p.threads, smem, s, grids, ngrids);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -11,6 +11,18 @@
 
 namespace gbmg {
 
+// A field of the next coarser level, on a lattice of its own.
+struct CoarseField {
+  float* base;  // first valid cell
+  int E[3], nb[3];
+  int pitch, plane;
+  long long bstride;
+};
+
+// What a sweep starts from: its source, zero (the source is not read), or the source plus the
+// piecewise-constant prolongation of the coarser level's field.
+enum { SWEEP_SOURCE = 0, SWEEP_ZERO = 1, SWEEP_PROLONG = 2 };
+
 // One level of one solve in a sweep launch.  All boxes have extents E on a lattice anchored at
 // the domain's low corner, stored in lattice order (x fastest) every bstride elements, without
 // ghost cells; src, rhs and dst share that layout.  The domain's low corner is local (0,0,0).
@@ -24,6 +36,7 @@ struct SweepGrid {
   int periodic;       // bit d: dimension d is periodic
   int par0;           // colour parity of the domain's low corner
   float mh2;          // -h^2
+  CoarseField coarse; // the coarser level's field (SWEEP_PROLONG); base null: none
   // tiling, set by plan_sweep: S strips of 4 cells x TY rows x ZC planes per block, hx / hy
   // strips and rows read around it, nt tiles per dimension, first tile of this grid
   int S, TY, ZC, hx, hy;
@@ -43,12 +56,6 @@ bool lattice_of(const BoxArray& ba, const FabLayout& lay, Lattice* out);
 
 // Residual + restriction of such a level (mg_sweep.cu): crhs = mean of the 8 children's
 // residuals, cphi = 0.  The coarse fields lie on a lattice of their own.
-struct CoarseField {
-  float* base;  // first valid cell
-  int E[3], nb[3];
-  int pitch, plane;
-  long long bstride;
-};
 struct RestrictGrid {
   SweepGrid g;  // src = phi, rhs; geometry
   float mih2;   // -1 / h^2
@@ -83,6 +90,7 @@ SweepPlan plan_sweep(std::vector<SweepGrid>& grids, std::vector<SweepGrid>& back
 // 18.9 / 19.2 ms (a step's lists are tiled anew).
 extern const long long kSweepMinCells, kSweepMinCellsBatch;
 
-cudaError_t launch_sweep_f32(const SweepGrid* grids, int ngrids, const SweepPlan& p, cudaStream_t s);
+cudaError_t launch_sweep_f32(const SweepGrid* grids, int ngrids, const SweepPlan& p, int start,
+                             cudaStream_t s);
 
 }  // namespace gbmg

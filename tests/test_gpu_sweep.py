@@ -45,7 +45,7 @@ def _opt(smoother, nu1=2, nu2=2):
 
 
 @pytest.mark.parametrize("n,box,per", SHAPES)
-@pytest.mark.parametrize("nu", [(2, 2), (3, 1)])
+@pytest.mark.parametrize("nu", [(2, 2), (3, 1), (1, 2), (4, 0)])
 def test_sweep_equals_half_sweeps(n, box, per, nu):
     ctx = mg.mg_init(0)
     try:
@@ -60,18 +60,19 @@ def test_sweep_equals_half_sweeps(n, box, per, nu):
         mg.mg_finalize(ctx)
 
 
-def test_batched_sweeps_equal_single_solves():
+@pytest.mark.parametrize("nu", [(2, 2), (1, 3)])
+def test_batched_sweeps_equal_single_solves(nu):
     """Different shapes in one launch (one tiling, one block size for all), each as alone with
     half-sweeps."""
     ctx = mg.mg_init(0)
     try:
         P = [_problem(ctx, n, box, per, 11 + i) for i, (n, box, per) in enumerate(SHAPES)]
         mg.mg_solve_batch(ctx, [p[0] for p in P], [p[1] for p in P], [p[2] for p in P], 1e-10,
-                          _opt(mg.MG_SMOOTH_AUTO))
+                          _opt(mg.MG_SMOOTH_AUTO, *nu))
         for i, (n, box, per) in enumerate(SHAPES):
             got = _dense(ctx, P[i][1], n)
             rhs, phi, bc = _problem(ctx, n, box, per, 11 + i)
-            mg.mg_solve(ctx, rhs, phi, bc, 1e-10, _opt(mg.MG_SMOOTH_HALF))
+            mg.mg_solve(ctx, rhs, phi, bc, 1e-10, _opt(mg.MG_SMOOTH_HALF, *nu))
             np.testing.assert_array_equal(got.view(np.int64), _dense(ctx, phi, n).view(np.int64))
     finally:
         mg.mg_finalize(ctx)
