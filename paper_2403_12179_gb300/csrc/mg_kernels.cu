@@ -1145,6 +1145,7 @@ void prolong_add_g(int G, const Grid& g, cudaStream_t s, const SegList& L, long 
 cudaError_t launch_residual_restrict_l(int dt, const SegList& L, long long nrows, cudaStream_t s,
                                        bool direct, bool stored) {
   if (nrows <= 0) return cudaSuccess;
+  if (dt == DT_F64 && L.ext.ok && L.ext.even) return launch_restrict_march(L, stored, s);
   // rows are coarse lines of width / 2 cells, one per lane
   const int G = group_lanes(L.width, 2, 8, 32);
   const Grid g = row_grid(nrows, row_blocks_per_sm(L.width), kWarps * (32 / G));
@@ -1287,8 +1288,9 @@ cudaError_t launch_residual(int dt, const DRow* rows, int nbox, long long nrows,
 }
 
 cudaError_t launch_residual_restrict(int dt, const DRow* rows, int nbox, long long nrows,
-                                     cudaStream_t s, bool direct, int width, bool stored) {
-  return launch_residual_restrict_l(dt, one_seg(rows, nbox, 0, width), nrows, s, direct, stored);
+                                     cudaStream_t s, bool direct, int width, bool stored,
+                                     const BoxExtents& ext) {
+  return launch_residual_restrict_l(dt, one_seg(rows, nbox, 0, width, ext), nrows, s, direct, stored);
 }
 
 cudaError_t launch_rbgs_half_store(const DRow* rows, int nbox, long long nrows, int color,

@@ -260,12 +260,14 @@ cudaError_t launch_residual_march(const SegList& L, unsigned long long* norms, c
 // 1 take the residual in v[2] (one-colour view) that launch_rbgs_half_store left there.
 cudaError_t launch_residual_restrict(int dt, const DRow* rows, int nbox, long long nrows,
                                      cudaStream_t s, bool direct = false, int width = 0,
-                                     bool stored = false);
+                                     bool stored = false, const BoxExtents& ext = {});
 // FP64 half-sweep (direct reads, one table) that also stores, in v[2] (one-colour view), the
 // residual of every cell it updates just after its update (the values a residual pass would
 // compute next).
 cudaError_t launch_rbgs_half_store(const DRow* rows, int nbox, long long nrows, int color,
                                    cudaStream_t s, int width, const BoxExtents& ext = {});
+// Residual + restriction (FP64; extents and corners of the boxes even) marching through planes.
+cudaError_t launch_restrict_march(const SegList& L, bool stored, cudaStream_t s);
 // The half-sweep (FP64) marching through planes (mg_march.cu); mode 0: plain, 1: norms
 // after the update, 2: norms and values before it, 3: residuals after it.
 cudaError_t launch_half_march(const SegList& L, int mode, int color, unsigned long long* norms,

@@ -322,12 +322,195 @@ __global__ void __launch_bounds__(kMarchThreads, 4)
   if (norms) block_max(mx, &norms[slot + R.solve]);
 }
 
+// Residual + restriction (even extents and box corners): a thread owns a coarse column, i.e. a pair of
+// cells in rows 2Y (A) and 2Y + 1 (B), and marches through planes; crhs = (sum of the 8 children's
+// residuals, x fastest) / 8, cphi = 0 (if c[1] is set).  STORED: the black children's residuals are
+// read from v[2] (one-colour view), only the red ones computed.  Row B's sums run on the integer
+// units.  FP64-pipe bound like the kernels above: 256^3 level of the FP64 solve (STORED) 186 -> 133 us
+// against a lane per coarse cell, 128^3 level 45 -> 37 us, 16^3 level 10.5 -> 7.1 us (ncu, cold); the
+// 256^3 solve 15.1 -> 14.0 ms.
+template <bool STORED, bool INT, bool MULTI>
+__global__ void __launch_bounds__(kMarchThreads, 4) k_restrict_march(SegList L, int zc) {
+  pdl_begin();
+  int slot;
+  const DRow& R = box_row<MULTI>(L, blockIdx.y, &slot);
+  const int pp = R.n[0] >> 1, ny = R.n[1], nz = R.n[2], nc1 = ny >> 1, rb = kMarchThreads / pp;
+  const int nty = (nc1 + rb - 1) / rb, ntz = (nz + zc - 1) / zc;
+  const int tile = blockIdx.x;
+  if (tile >= nty * ntz) return;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int ry = tid / pp, i = tid - ry * pp, Y = (tile % nty) * rb + ry, y = 2 * Y;
+  const int z0 = (tile / nty) * zc, z1 = min(z0 + zc, nz);  // (zc even)
+  const bool active = ry < rb && Y < nc1;
+  const unsigned mask = __ballot_sync(0xffffffffu, active);
+  if (!active) return;
+  const int pitch = R.v[0].pitch;
+  const long long ip = R.v[0].plane * 8, ir = R.v[1].plane * 8, dB = (long long)pitch * 8,
+                  dfB = (long long)R.v[1].pitch * 8;
+  const unsigned nbf = (unsigned)R.nbf;
+  const double mih2 = flip(R.ih2, 1u);
+  const double* own = (const double*)R.v[0].p + z0 * R.v[0].plane + (long long)y * pitch + 2 * i;
+  const double* pf = (const double*)R.v[1].p + z0 * R.v[1].plane + (long long)y * R.v[1].pitch + 2 * i;
+  const double* pym = own - pitch + (y == 0 ? R.nbd[2] : 0);
+  const double* pyp = own + 2 * pitch + (y == ny - 2 ? R.nbd[3] : 0);
+  const unsigned nym = y == 0 ? (nbf >> 2) & 1u : 0u, nyp = y == ny - 2 ? (nbf >> 3) & 1u : 0u;
+  const double* st = nullptr;
+  long long is = 0, dsB = 0;
+  if (STORED) {
+    is = R.v[2].plane * 8;
+    dsB = R.v[2].pitch * 8;
+    st = (const double*)R.v[2].p + z0 * R.v[2].plane + (long long)y * R.v[2].pitch + i;
+  }
+  double* cr = (double*)R.c[0].p + (z0 >> 1) * R.c[0].plane + (long long)Y * R.c[0].pitch + i;
+  double* cp = R.c[1].p ? (double*)R.c[1].p + (z0 >> 1) * R.c[1].plane + (long long)Y * R.c[1].pitch + i : nullptr;
+  const bool exl = i == 0, exr = i == pp - 1, ldl = exl || lane == 0, ldr = exr || lane == 31;
+  const unsigned nxl = exl ? nbf & 1u : 0u, nxr = exr ? (nbf >> 1) & 1u : 0u;
+  const double* pxl = own - 1 + (exl ? R.nbd[0] : 0);
+  const double* pxr = own + 2 + (exr ? R.nbd[1] : 0);
+  const unsigned nzm = (nbf >> 4) & 1u, nzp = (nbf >> 5) & 1u;
+  const long long dz1 = R.nbd[5] * 8;
+  const double* below = own - R.v[0].plane + (z0 == 0 ? R.nbd[4] : 0);
+  const unsigned nb = z0 == 0 ? nzm : 0u;
+  double acc = 0.0;
+  if constexpr (STORED) {
+    // box corners are even: the red cell of row A sits at place 0 of the pair in even planes, at 1 in odd
+    // ones, row B's at the other place; mX / cX: the black cells below and beside them
+    double mA = flip(below[0], nb), mB = flip(at(below, dB)[1], nb);
+    double cA = own[1], cB = at(own, dB)[0];
+    struct In {
+      double nA, nB, ym, yp, fA, fB, oA, oB, sA, sB, xA, xB;
+    };
+    auto load = [&](auto Kc, int z, In& v) {
+      constexpr int K = decltype(Kc)::value;
+      const long long o = (long long)(z - z0) * ip;
+      const double* up = at(own, o + ip + (z == nz - 1 ? dz1 : 0));
+      const double* c = at(own, o);
+      const double* f = at(pf, (long long)(z - z0) * ir);
+      const double* t = at(st, (long long)(z - z0) * is);
+      v.nA = up[K];
+      v.nB = at(up, dB)[K ^ 1];
+      v.ym = at(pym, o)[K];
+      v.yp = at(pyp, o)[K ^ 1];
+      v.fA = f[K];
+      v.fB = at(f, dfB)[K ^ 1];
+      v.oA = c[K];
+      v.oB = at(c, dB)[K ^ 1];
+      v.sA = *t;
+      v.sB = *at(t, dsB);
+      if (K ? ldr : ldl) v.xA = *at(K ? pxr : pxl, o);
+      if (K ? ldl : ldr) v.xB = *at(K ? pxl : pxr, o + dB);
+    };
+    auto step = [&](auto Kc, int z, const In& v) {
+      constexpr int K = decltype(Kc)::value;
+      double xA = __shfl_sync(mask, cA, K ? lane + 1 : lane - 1), xB = __shfl_sync(mask, cB, K ? lane - 1 : lane + 1);
+      if (K ? ldr : ldl) xA = flip(v.xA, K ? nxr : nxl);
+      if (K ? ldl : ldr) xB = flip(v.xB, K ? nxl : nxr);
+      const unsigned e = z == nz - 1 ? nzp : 0u;
+      const double nA = flip(v.nA, e), nB = flip(v.nB, e);
+      const double wA[6] = {xA, cA, flip(v.ym, nym), cB, mA, nA}, wB[6] = {xB, cB, cA, flip(v.yp, nyp), mB, nB};
+      const double rA = residual_of(sum6<false>(wA, mask), v.oA, v.fA, mih2);
+      const double rB = residual_of(sum6<INT>(wB, mask), v.oB, v.fB, mih2);
+      acc = K ? __dadd_rn(acc, v.sA) : __dadd_rn(rA, v.sA);
+      if (K) acc = __dadd_rn(acc, rA);
+      acc = __dadd_rn(acc, K ? rB : v.sB);
+      acc = __dadd_rn(acc, K ? v.sB : rB);
+      mA = cA;
+      cA = nA;
+      mB = cB;
+      cB = nB;
+    };
+    In a, b;
+    load(Int<0>{}, z0, a);
+    for (int z = z0; z < z1; z += 2) {
+      load(Int<1>{}, z + 1, b);
+      step(Int<0>{}, z, a);
+      if (z + 2 < z1) load(Int<0>{}, z + 2, a);
+      step(Int<1>{}, z + 1, b);
+      *cr = __dmul_rn(acc, 0.125);
+      cr += R.c[0].plane;
+      if (cp) {
+        *cp = 0.0;
+        cp += R.c[1].plane;
+      }
+    }
+  } else {
+    double mA0 = flip(below[0], nb), mA1 = flip(below[1], nb);
+    double mB0 = flip(at(below, dB)[0], nb), mB1 = flip(at(below, dB)[1], nb);
+    double cA0 = own[0], cA1 = own[1], cB0 = at(own, dB)[0], cB1 = at(own, dB)[1];
+    struct In {
+      double nA0, nA1, nB0, nB1, ym0, ym1, yp0, yp1, fA0, fA1, fB0, fB1, lA, lB, rA, rB;
+    };
+    auto load = [&](int z, In& v) {
+      const long long o = (long long)(z - z0) * ip;
+      const double* up = at(own, o + ip + (z == nz - 1 ? dz1 : 0));
+      const double* f = at(pf, (long long)(z - z0) * ir);
+      v.nA0 = up[0];
+      v.nA1 = up[1];
+      v.nB0 = at(up, dB)[0];
+      v.nB1 = at(up, dB)[1];
+      v.ym0 = at(pym, o)[0];
+      v.ym1 = at(pym, o)[1];
+      v.yp0 = at(pyp, o)[0];
+      v.yp1 = at(pyp, o)[1];
+      v.fA0 = f[0];
+      v.fA1 = f[1];
+      v.fB0 = at(f, dfB)[0];
+      v.fB1 = at(f, dfB)[1];
+      if (ldl) {
+        v.lA = *at(pxl, o);
+        v.lB = *at(pxl, o + dB);
+      }
+      if (ldr) {
+        v.rA = *at(pxr, o);
+        v.rB = *at(pxr, o + dB);
+      }
+    };
+    auto step = [&](int z, const In& v) {
+      double lA = __shfl_sync(mask, cA1, lane - 1), lB = __shfl_sync(mask, cB1, lane - 1);
+      double rA = __shfl_sync(mask, cA0, lane + 1), rB = __shfl_sync(mask, cB0, lane + 1);
+      if (ldl) {
+        lA = flip(v.lA, nxl);
+        lB = flip(v.lB, nxl);
+      }
+      if (ldr) {
+        rA = flip(v.rA, nxr);
+        rB = flip(v.rB, nxr);
+      }
+      const unsigned e = z == nz - 1 ? nzp : 0u;
+      const double nA0 = flip(v.nA0, e), nA1 = flip(v.nA1, e), nB0 = flip(v.nB0, e), nB1 = flip(v.nB1, e);
+      const double a0[6] = {lA, cA1, flip(v.ym0, nym), cB0, mA0, nA0}, a1[6] = {cA0, rA, flip(v.ym1, nym), cB1, mA1, nA1};
+      const double b0[6] = {lB, cB1, cA0, flip(v.yp0, nyp), mB0, nB0}, b1[6] = {cB0, rB, cA1, flip(v.yp1, nyp), mB1, nB1};
+      const double r0 = residual_of(sum6<false>(a0, mask), cA0, v.fA0, mih2);
+      acc = z & 1 ? __dadd_rn(acc, r0) : r0;
+      acc = __dadd_rn(acc, residual_of(sum6<false>(a1, mask), cA1, v.fA1, mih2));
+      acc = __dadd_rn(acc, residual_of(sum6<INT>(b0, mask), cB0, v.fB0, mih2));
+      acc = __dadd_rn(acc, residual_of(sum6<INT>(b1, mask), cB1, v.fB1, mih2));
+      mA0 = cA0, mA1 = cA1, mB0 = cB0, mB1 = cB1;
+      cA0 = nA0, cA1 = nA1, cB0 = nB0, cB1 = nB1;
+    };
+    In a, b;
+    load(z0, a);
+    for (int z = z0; z < z1; z += 2) {
+      load(z + 1, b);
+      step(z, a);
+      if (z + 2 < z1) load(z + 2, a);
+      step(z + 1, b);
+      *cr = __dmul_rn(acc, 0.125);
+      cr += R.c[0].plane;
+      if (cp) {
+        *cp = 0.0;
+        cp += R.c[1].plane;
+      }
+    }
+  }
+}
+
 // Blocks over (rows of a box x chunks of *zc planes, boxes); chunks are halved until about six
 // blocks an SM are there (4 and 16 instead: within 2% at 256^3, slower at 128^3 and below).
-dim3 march_grid(const SegList& L, int* zc) {
+dim3 march_grid(const SegList& L, int* zc, int rows = 1) {  // rows of a thread
   const int* ext = L.ext.n;
   const int rb = kMarchThreads / ((ext[0] + 1) / 2);
-  const int ty = (ext[1] + rb - 1) / rb;
+  const int ty = ((ext[1] + rows - 1) / rows + rb - 1) / rb;
   *zc = 32;
   while (*zc > 2 && (long long)L.nbox * ty * ((ext[2] + *zc - 1) / *zc) < 6ll * num_sms()) *zc /= 2;
   return dim3((unsigned)(ty * ((ext[2] + *zc - 1) / *zc)), (unsigned)L.nbox);
@@ -374,6 +557,26 @@ cudaError_t launch_residual_march(const SegList& L, unsigned long long* norms, c
   } else {
     if (L.n > 1) go(k_residual_march<false, true>);
     else go(k_residual_march<false, false>);
+  }
+  count_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_restrict_march(const SegList& L, bool stored, cudaStream_t s) {
+  int zc;
+  const dim3 grid = march_grid(L, &zc, 2);
+  auto go = [&](auto k) { launch_k(k, grid, kMarchThreads, 0, s, L, zc); };
+  const bool ints = use_int(L);
+  if (stored && L.n != 1) return cudaErrorInvalidValue;
+  if (stored) {
+    if (ints) go(k_restrict_march<true, true, false>);
+    else go(k_restrict_march<true, false, false>);
+  } else if (L.n > 1) {
+    if (ints) go(k_restrict_march<false, true, true>);
+    else go(k_restrict_march<false, false, true>);
+  } else {
+    if (ints) go(k_restrict_march<false, true, false>);
+    else go(k_restrict_march<false, false, false>);
   }
   count_launches(1);
   return cudaGetLastError();

@@ -1296,7 +1296,7 @@ int mg_residual_restrict(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, mg_fab_t crhs, 
         if (fz) R.c[1] = coarse_view(*fz, map[b], F.boxes[b]);
       }, c->stream);
     });
-    MG_CK(launch_residual_restrict(fp->dtype, t.rows(), t.nbox, t.nrows, s, false, t.width));
+    MG_CK(launch_residual_restrict(fp->dtype, t.rows(), t.nbox, t.nrows, s, false, t.width, false, t.ext));
     return MG_OK;
   });
 }

@@ -516,7 +516,7 @@ void enqueue_vcycle(Ctx& c, Hierarchy& H, cudaStream_t s, unsigned long long* no
       MG_CK(launch_restrict_f32((const RestrictGrid*)D.rr_dev->p, 1, D.rr_plan, s));
     else
       MG_CK(launch_residual_restrict(H.dt, D.rr.rows(), D.rr.nbox, D.rr.nrows, s, D.direct,
-                                     D.rr.width, stored));
+                                     D.rr.width, stored, D.rr.ext));
   }
   if (H.lc < nl) MG_CK(launch_coarse_cycle(H.dt, (const CoarseJob*)H.cjob->p, 1, H.csmem, s));
   else MG_CK(launch_bottom(H.dt, (const BottomJob*)H.job->p, 1, H.N, s));
