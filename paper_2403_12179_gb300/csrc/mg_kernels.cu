@@ -804,14 +804,29 @@ __global__ void __launch_bounds__(kBottomRows) k_bottom(const BottomJob* __restr
   phi[J.off_phi[i]] = (T)s;
 }
 
-template <class T>
+// Rows from one place to another: G lanes per x-line, kCopyCells cells of a lane per step, loads first.
+constexpr int kCopyCells = 4;
+template <class T, int G>
+__device__ __forceinline__ void copy_line(T* __restrict__ d, const T* __restrict__ s, int n, int lane) {
+  for (int x = lane; x < n; x += kCopyCells * G) {
+    T v[kCopyCells];
+#pragma unroll
+    for (int k = 0; k < kCopyCells; ++k)
+      if (x + G * k < n) v[k] = s[x + G * k];
+#pragma unroll
+    for (int k = 0; k < kCopyCells; ++k)
+      if (x + G * k < n) d[x + G * k] = v[k];
+  }
+}
+
+template <class T, int G>
 __global__ void __launch_bounds__(kThreads) k_dense_copy(SegList L, long long nrows, long long per,
                                                          T* dense, int3 dlo, int3 dn, int ncomp,
                                                          int to_dense) {
   pdl_begin();
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & (G - 1);
   const long long dplane = (long long)dn.x * dn.y, dcomp = dplane * dn.z;
-  for_rows(L, nrows, per, [&](const DRow& R, long long lr, int) {
+  for_rows<32 / G>(L, nrows, per, [&](const DRow& R, long long lr, int) {
     const int n0 = R.n[0], n1 = R.n[1];
     const int y = (int)lr % n1, z = (int)lr / n1;
     T* f = line<T>(R.v[0], y, z);
@@ -820,12 +835,20 @@ __global__ void __launch_bounds__(kThreads) k_dense_copy(SegList L, long long nr
     for (int c = 0; c < ncomp; ++c) {
       T* fc = f + c * R.v[0].cstride;
       T* dc = d + c * dcomp;
-      if (to_dense) {
-        for (int x = lane; x < n0; x += 32) dc[x] = fc[x];
-      } else {
-        for (int x = lane; x < n0; x += 32) fc[x] = dc[x];
-      }
+      if (to_dense) copy_line<T, G>(dc, fc, n0, lane);
+      else copy_line<T, G>(fc, dc, n0, lane);
     }
+  });
+}
+
+// v[0] = v[1] on valid cells.
+template <class T, int G>
+__global__ void __launch_bounds__(kThreads) k_copy_valid(SegList L, long long nrows, long long per) {
+  pdl_begin();
+  const int lane = threadIdx.x & (G - 1);
+  for_rows<32 / G>(L, nrows, per, [&](const DRow& R, long long lr, int) {
+    const int y = (int)lr % R.n[1], z = (int)lr / R.n[1];
+    copy_line<T, G>(line<T>(R.v[0], y, z), line<T>(R.v[1], y, z), R.n[0], lane);
   });
 }
 
@@ -1360,15 +1383,35 @@ cudaError_t launch_set_flat(int dt, void* p, long long n, double value, cudaStre
 
 cudaError_t launch_dense_copy(int dt, const DRow* rows, int nbox, long long nrows, void* dense,
                               const int dom_lo[3], const int dom_n[3], int ncomp, int to_dense,
-                              cudaStream_t s) {
+                              cudaStream_t s, int width) {
   if (nrows <= 0) return cudaSuccess;
-  Grid g = row_grid(nrows, 16);
+  const int G = group_lanes(width, kCopyCells, 8, 32);
+  const Grid g = row_grid(nrows, row_blocks_per_sm(width), kWarps * (32 / G));
+  const SegList L = one_seg(rows, nbox, 0, width);
   int3 lo = make_int3(dom_lo[0], dom_lo[1], dom_lo[2]);
   int3 n = make_int3(dom_n[0], dom_n[1], dom_n[2]);
-  if (dt == DT_F64)
-    launch_k(k_dense_copy<double>, g.blocks, kThreads, 0, s, one_seg(rows, nbox), nrows, g.per, (double*)dense, lo, n, ncomp, to_dense);
-  else
-    launch_k(k_dense_copy<float>, g.blocks, kThreads, 0, s, one_seg(rows, nbox), nrows, g.per, (float*)dense, lo, n, ncomp, to_dense);
+  auto go = [&](auto k, auto* p) { launch_k(k, g.blocks, kThreads, 0, s, L, nrows, g.per, p, lo, n, ncomp, to_dense); };
+  if (dt == DT_F64) {
+    if (G == 32) go(k_dense_copy<double, 32>, (double*)dense);
+    else if (G == 16) go(k_dense_copy<double, 16>, (double*)dense);
+    else go(k_dense_copy<double, 8>, (double*)dense);
+  } else {
+    if (G == 32) go(k_dense_copy<float, 32>, (float*)dense);
+    else if (G == 16) go(k_dense_copy<float, 16>, (float*)dense);
+    else go(k_dense_copy<float, 8>, (float*)dense);
+  }
+  count_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_copy_valid_f32(const DRow* rows, int nbox, long long nrows, cudaStream_t s, int width) {
+  if (nrows <= 0) return cudaSuccess;
+  const int G = group_lanes(width, kCopyCells, 8, 32);
+  const Grid g = row_grid(nrows, row_blocks_per_sm(width), kWarps * (32 / G));
+  const SegList L = one_seg(rows, nbox, 0, width);
+  if (G == 32) launch_k(k_copy_valid<float, 32>, g.blocks, kThreads, 0, s, L, nrows, g.per);
+  else if (G == 16) launch_k(k_copy_valid<float, 16>, g.blocks, kThreads, 0, s, L, nrows, g.per);
+  else launch_k(k_copy_valid<float, 8>, g.blocks, kThreads, 0, s, L, nrows, g.per);
   count_launches(1);
   return cudaGetLastError();
 }

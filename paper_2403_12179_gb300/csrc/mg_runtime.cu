@@ -396,7 +396,7 @@ void dense_upload(Ctx& c, FabObj& f, const void* host, cudaStream_t s) {
   DevBufP stage = c.alloc(bytes, s);
   MG_CK(cudaMemcpyAsync(stage->p, host, bytes, cudaMemcpyHostToDevice, s));
   MG_CK(launch_dense_copy(f.dtype, (const DRow*)f.valid_rows->p, (int)f.ba->ba.boxes.size(),
-                          f.nrows, stage->p, D.lo, n, f.lay.ncomp, 0, s));
+                          f.nrows, stage->p, D.lo, n, f.lay.ncomp, 0, s, f.width()));
   stage->reset(s);
 }
 
@@ -407,7 +407,7 @@ void dense_download(Ctx& c, FabObj& f, void* host, cudaStream_t s) {
   const size_t bytes = (size_t)D.npts() * f.lay.ncomp * f.esize();
   DevBufP stage = c.alloc(bytes, s);
   MG_CK(launch_dense_copy(f.dtype, (const DRow*)f.valid_rows->p, (int)f.ba->ba.boxes.size(),
-                          f.nrows, stage->p, D.lo, n, f.lay.ncomp, 1, s));
+                          f.nrows, stage->p, D.lo, n, f.lay.ncomp, 1, s, f.width()));
   MG_CK(cudaMemcpyAsync(host, stage->p, bytes, cudaMemcpyDeviceToHost, s));
   stage->reset(s);
 }
@@ -438,6 +438,16 @@ void drop_cached_ops_of(Ctx& c, int64_t fab_id) {
     if (uses) {
       if (!synced) { cudaDeviceSynchronize(); synced = true; }
       it = c.fused_cache.erase(it);
+    } else {
+      ++it;
+    }
+  }
+  for (auto it = c.sweep_cache.begin(); it != c.sweep_cache.end();) {
+    bool uses = false;
+    for (int64_t id : it->second->owner_fabs) uses |= id == fab_id;
+    if (uses) {
+      if (!synced) { cudaDeviceSynchronize(); synced = true; }
+      it = c.sweep_cache.erase(it);
     } else {
       ++it;
     }
@@ -606,6 +616,49 @@ std::shared_ptr<FabObj> partner_of(Ctx& c, FabObj& f) {
   return p;
 }
 
+const SweepTable& sweep_table(Ctx& c, int64_t phi_id, FabObj& phi, int64_t rhs_id, FabObj& rhs,
+                              const mg_bc* bc, double h) {
+  int per[3];
+  const int code = bc_code(bc, per);
+  char key[160];
+  std::snprintf(key, sizeof key, "%lld:%lld:%d:%.17g", (long long)phi_id, (long long)rhs_id, code, h);
+  auto it = c.sweep_cache.find(key);
+  if (it != c.sweep_cache.end()) return *it->second;
+  auto t = std::make_shared<SweepTable>();
+  t->owner_fabs = {phi_id, rhs_id};
+  SweepGrid G;
+  const FabLayout plain = make_layout(phi.ba->ba, 1, 0, 4);
+  if (phi.dtype == DT_F32 && sweep_fabs_geometry(phi.ba->ba, phi.lay, rhs.lay, plain, per, h, &G)) {
+    if (!phi.plain) {
+      auto p = std::make_shared<FabObj>();
+      p->ba = phi.ba;
+      p->dtype = DT_F32;
+      p->lay = plain;
+      p->bytes = (size_t)plain.total * 4;
+      p->own = c.alloc(p->bytes, c.stream);
+      p->base = p->own->p;
+      phi.plain = p;
+    }
+    Lattice P, R;
+    lattice_of(phi.ba->ba, phi.lay, &P);
+    lattice_of(phi.ba->ba, rhs.lay, &R);
+    G.src = (const float*)phi.base + P.first;
+    G.rhs = (const float*)rhs.base + R.first;
+    G.dst = (float*)phi.plain->base;
+    std::vector<SweepGrid> v{G}, w{G};
+    t->plan = plan_sweep(v, w);
+    t->grid = c.upload(v.data(), sizeof(SweepGrid), c.stream);
+    t->back = make_table(c, phi.ba->ba, 0, h, 0, [&](int b, DRow& row) {
+      row.v[0] = phi.view(b);
+      row.v[1] = phi.plain->view(b);
+    }, c.stream);
+    t->ok = true;
+    MG_CK(cudaStreamSynchronize(c.stream));
+  }
+  c.sweep_cache[key] = t;
+  return *t;
+}
+
 void check_device_error(Ctx& c) {
   int e = 0;
   MG_CK(cudaMemcpy(&e, c.d_err->p, sizeof e, cudaMemcpyDeviceToHost));
@@ -669,6 +722,8 @@ void same_shape(const FabObj& a, const FabObj& b, const char* what) {
 
 double default_h(const FabObj& f, double h) { return h > 0 ? h : 1.0 / f.ba->ba.dom.len(0); }
 
+// (Checked and built once per pair of fabs, with the cached table: the search is over all pairs of
+// boxes, 50 us a call with 216 of them.)
 // The coarse fab must be on level 1 of the fine fab's hierarchy (domain halved, boxes the
 // coarsened fine boxes or one box covering the coarse domain).  Returns, for every fine
 // box, the coarse box holding its parent cells.
@@ -774,6 +829,7 @@ int mg_finalize(mg_ctx_t h) {
     destroy_hierarchies(*c);
     c->op_cache.clear();
     c->fused_cache.clear();
+    c->sweep_cache.clear();
     c->fabs.clear();
     c->tag_cache.clear();
     c->bas.clear();
@@ -1056,7 +1112,8 @@ int mg_fab_copy_from_dense(mg_ctx_t h, mg_fab_t fab, const void* src, int src_on
       dsrc = stage->p;
     }
     MG_CK(launch_dense_copy(f->dtype, (const DRow*)f->valid_rows->p, (int)f->ba->ba.boxes.size(),
-                            f->nrows, const_cast<void*>(dsrc), D.lo, n, f->lay.ncomp, 0, s));
+                            f->nrows, const_cast<void*>(dsrc), D.lo, n, f->lay.ncomp, 0, s,
+                            f->width()));
     if (stage) stage->reset(s);
     return MG_OK;
   });
@@ -1079,7 +1136,7 @@ int mg_fab_copy_to_dense(mg_ctx_t h, mg_fab_t fab, void* dst, int dst_on_host, v
       ddst = stage->p;
     }
     MG_CK(launch_dense_copy(f->dtype, (const DRow*)f->valid_rows->p, (int)f->ba->ba.boxes.size(),
-                            f->nrows, ddst, D.lo, n, f->lay.ncomp, 1, s));
+                            f->nrows, ddst, D.lo, n, f->lay.ncomp, 1, s, f->width()));
     if (dst_on_host) {
       MG_CK(cudaMemcpyAsync(dst, stage->p, bytes, cudaMemcpyDeviceToHost, s));
       stage->reset(s);
@@ -1182,7 +1239,44 @@ int mg_smooth(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double hh
         R.v[1] = fr->view(b);
       }, c->stream);
     });
-    if (color == 2 && fused_eligible(*fp, *fr)) {
+    const bool fusable = color == 2 && fused_eligible(*fp, *fr);
+    if (fusable && fp->dtype == DT_F32) {
+      // boxes on a lattice: a sweep that reads the neighbouring boxes, into a scratch array, and back
+      // (256^3, boxes of 64^3: 121 us a call, sweep 74, copy back 28, rhs fill 18, against 135 for two
+      // fills, the TMA sweep and a copy of the whole fab, and no autotuning on the first call: 92 ms)
+      const SweepTable& st = sweep_table(*c, phi, *fp, rhs, *fr, bc, hv);
+      if (st.ok) {
+        launch_fill(*c, *fr, bc, s);
+        MG_CK(launch_sweep_f32_fabs((const SweepGrid*)st.grid->p, st.plan, fp->lay.g, s));
+        MG_CK(launch_copy_valid_f32(st.back.rows(), st.back.nbox, st.back.nrows, s, st.back.width));
+        return MG_OK;
+      }
+    }
+    // the red half-sweep may read neighbouring boxes instead of ghost cells (and, in FP64 with the
+    // layout of the fused sweep, which leaves phi's ghosts stale, the black one too)
+    const OpTable* td = nullptr;
+    if (color == 2 && (fp->dtype == DT_F64 || !fusable)) {
+      int per[3];
+      const int code = bc_code(bc, per);
+      const OpTable& q = op_table(*c, ("smooth_any" + std::to_string(code)).c_str(), {phi, rhs}, hv, [&] {
+        FaceReads faces = direct_neighbours(*fp, per);
+        OpTable tt = make_table(*c, fp->ba->ba, 0, hv, 0, [&](int b, DRow& R) {
+          R.v[0] = fp->view(b);
+          R.v[1] = fr->view(b);
+          faces.apply(b, R);
+        }, c->stream);
+        tt.direct = faces.ok();
+        return tt;
+      });
+      if (q.direct) td = &q;
+    }
+    if (fusable && td) {
+      launch_fill(*c, *fr, bc, s);
+      for (int col = 0; col < 2; ++col)
+        MG_CK(launch_rbgs_half(fp->dtype, td->rows(), td->nbox, td->nrows, col, s, true, nullptr, td->width, false, td->ext));
+      return MG_OK;
+    }
+    if (fusable) {
       // one fused sweep into the scratch partner, then copied back (ghosts included; they
       // are refilled before the next read)
       auto tmp = partner_of(*c, *fp);
@@ -1201,6 +1295,10 @@ int mg_smooth(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double hh
       MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, color, s, false, nullptr, t.width, false, t.ext));
     } else {
       for (int col = 0; col < 2; ++col) {
+        if (col == 0 && td) {
+          MG_CK(launch_rbgs_half(fp->dtype, td->rows(), td->nbox, td->nrows, 0, s, true, nullptr, td->width, false, td->ext));
+          continue;
+        }
         launch_fill(*c, *fp, bc, s);
         MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, col, s, false, nullptr, t.width, false, t.ext));
       }
@@ -1284,11 +1382,11 @@ int mg_residual_restrict(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, mg_fab_t crhs, 
     if (fc->dtype != fp->dtype) fail(MG_EINVAL, "coarse and fine types differ");
     if (!aligned(fp->ba->ba)) fail(MG_EINVAL, "fine boxes must have even bounds");
     if (fp->lay.g < 1) fail(MG_EINVAL, "phi needs at least one ghost cell");
-    std::vector<int> map = coarse_map(*fp, *fc);
     cudaStream_t s = S(stream);
     double hv = default_h(*fp, hh);
     const BoxArray& F = fp->ba->ba;
     const OpTable& t = op_table(*c, "resrestrict", {phi, rhs, crhs, cphi}, hv, [&] {
+      const std::vector<int> map = coarse_map(*fp, *fc);
       return make_table(*c, F, 1, hv, 0, [&](int b, DRow& R) {
         R.v[0] = fp->view(b);
         R.v[1] = fr->view(b);
@@ -1309,10 +1407,10 @@ int mg_restrict(mg_ctx_t h, mg_fab_t fine, mg_fab_t coarse, void* stream) {
     auto fc = c->get_fab(coarse);
     if (fc->dtype != ff->dtype) fail(MG_EINVAL, "coarse and fine types differ");
     if (!aligned(ff->ba->ba)) fail(MG_EINVAL, "fine boxes must have even bounds");
-    std::vector<int> map = coarse_map(*ff, *fc);
     cudaStream_t s = S(stream);
     const BoxArray& F = ff->ba->ba;
     const OpTable& t = op_table(*c, "restrict", {fine, coarse}, 1.0, [&] {
+      const std::vector<int> map = coarse_map(*ff, *fc);
       return make_table(*c, F, 1, 1.0, 0, [&](int b, DRow& R) {
         R.v[0] = ff->view(b);
         R.c[0] = coarse_view(*fc, map[b], F.boxes[b]);
@@ -1330,10 +1428,10 @@ int mg_prolong_add(mg_ctx_t h, mg_fab_t coarse, mg_fab_t fine, void* stream) {
     auto ff = c->get_fab(fine);
     auto fc = c->get_fab(coarse);
     if (fc->dtype != ff->dtype) fail(MG_EINVAL, "coarse and fine types differ");
-    std::vector<int> map = coarse_map(*ff, *fc);
     cudaStream_t s = S(stream);
     const BoxArray& F = ff->ba->ba;
     const OpTable& t = op_table(*c, "prolong", {coarse, fine}, 1.0, [&] {
+      const std::vector<int> map = coarse_map(*ff, *fc);
       return make_table(*c, F, 0, 1.0, 0, [&](int b, DRow& R) {
         R.v[0] = ff->view(b);
         R.c[0] = coarse_view(*fc, map[b], F.boxes[b]);
@@ -1352,10 +1450,10 @@ int mg_prolong_add_trilinear(mg_ctx_t h, mg_fab_t coarse, mg_fab_t fine, void* s
     auto fc = c->get_fab(coarse);
     if (fc->dtype != ff->dtype) fail(MG_EINVAL, "coarse and fine types differ");
     if (fc->lay.g < 1) fail(MG_EINVAL, "trilinear prolongation reads one coarse ghost layer");
-    std::vector<int> map = coarse_map(*ff, *fc);
     cudaStream_t s = S(stream);
     const BoxArray& F = ff->ba->ba;
     const OpTable& t = op_table(*c, "prolong", {coarse, fine}, 1.0, [&] {
+      const std::vector<int> map = coarse_map(*ff, *fc);
       return make_table(*c, F, 0, 1.0, 0, [&](int b, DRow& R) {
         R.v[0] = ff->view(b);
         R.c[0] = coarse_view(*fc, map[b], F.boxes[b]);

@@ -20,6 +20,7 @@
 #include "../../include/gbmg.h"
 #include "mg_host.hpp"
 #include "mg_kernels.hpp"
+#include "mg_sweep.hpp"
 
 namespace gbmg {
 
@@ -119,6 +120,12 @@ struct FabObj {
   DevBufP valid_rows;  // DRow table, v[0] = this fab (fine x-lines)
   long long nrows = 0;
   std::shared_ptr<FabObj> partner;  // same-layout scratch for out-of-place sweeps
+  std::shared_ptr<FabObj> plain;    // the same boxes without ghosts, for the same purpose
+  int width() const {               // widest box
+    int w = 0;
+    for (const Box& b : ba->ba.boxes) w = w > b.len(0) ? w : b.len(0);
+    return w;
+  }
   DView view(int b) const;
   int esize() const { return dtype == DT_F64 ? 8 : 4; }
 };
@@ -197,6 +204,7 @@ struct Ctx {
   };
   std::map<std::string, CachedOp> op_cache;
   std::map<std::string, std::shared_ptr<struct FusedTable>> fused_cache;
+  std::map<std::string, std::shared_ptr<struct SweepTable>> sweep_cache;
   // ghost-fill patterns shared by all fabs of one layout
   std::mutex tag_mu;
   std::map<std::string, std::shared_ptr<TagSet>> tag_cache;
@@ -310,6 +318,17 @@ void launch_fused(Ctx& c, const FusedTable& t, int dt, cudaStream_t s);
 const FusedTable& fused_table(Ctx& c, int64_t src_id, FabObj& src, int64_t rhs_id, FabObj& rhs,
                               int64_t dst_id, FabObj& dst, const mg_bc* bc, double h);
 std::shared_ptr<FabObj> partner_of(Ctx& c, FabObj& f);
+// Cached whole sweep of a caller's FP32 fabs (mg_sweep.cu) into phi's plain partner, and the copy
+// back; ok == false where the boxes do not allow it.
+struct SweepTable {
+  bool ok = false;
+  DevBufP grid;
+  SweepPlan plan;
+  OpTable back;
+  std::vector<int64_t> owner_fabs;
+};
+const SweepTable& sweep_table(Ctx& c, int64_t phi_id, FabObj& phi, int64_t rhs_id, FabObj& rhs,
+                              const mg_bc* bc, double h);
 void check_device_error(Ctx& c);
 
 // Copy-tag conversion to device layout (offsets relative to the fab base).

@@ -105,12 +105,40 @@ __device__ __forceinline__ float4 add_pairs(const float4& v, const float2& c) { 
   return make_float4(__fadd_rn(v.x, c.x), __fadd_rn(v.y, c.x), __fadd_rn(v.z, c.y), __fadd_rn(v.w, c.y));
 }
 
-template <int START>
+__device__ __forceinline__ void cpa8(uint32_t d, const void* s) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(s) : "memory");
+}
+// A strip of 16 bytes whose source is aligned to AL.
+template <int AL>
+__device__ __forceinline__ void cpa_strip(uint32_t d, const char* s) {
+  if (AL == 16) {
+    cpa16(d, s);
+  } else if (AL == 8) {
+    cpa8(d, s);
+    cpa8(d + 8, s + 8);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 16; i += 4) cpa4(d + i, s + i);
+  }
+}
+template <int AL>
+__device__ __forceinline__ float4 ld_strip(const char* s) {
+  if (AL == 16) return *reinterpret_cast<const float4*>(s);
+  const float* f = reinterpret_cast<const float*>(s);
+  return make_float4(f[0], f[1], f[2], f[3]);
+}
+
+// PAL, RAL: alignment of the strips of phi and rhs; below 16 the three fields have layouts of their own.
+template <int START, int PAL = 16, int RAL = 16>
 __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
     k_sweep_f32(const SweepGrid* __restrict__ grids, int ng) {
   pdl_begin();
   extern __shared__ __align__(16) unsigned char smem[];
+  constexpr bool kOne = PAL == 16 && RAL == 16;  // one layout
   __shared__ long long zoff[kMaxPlanes], czoff[START == SWEEP_PROLONG ? kMaxPlanes : 1];
+  __shared__ long long rzoff_[kOne ? 1 : kMaxPlanes], dzoff_[kOne ? 1 : kMaxPlanes];
+  const long long* const rzoff = kOne ? zoff : rzoff_;
+  const long long* const dzoff = kOne ? zoff : dzoff_;
   __shared__ SweepGrid Gs;
   load_grid(&Gs, grids, ng);
   __syncthreads();
@@ -172,6 +200,11 @@ __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
     }
     const int bz = p / G.E[2];
     zoff[q] = ((long long)bz * G.nb[0] * G.nb[1] * G.bstride + (long long)(p - bz * G.E[2]) * G.plane) * 4;
+    if (!kOne) {
+      const long long col = (long long)bz * G.nb[0] * G.nb[1], pl = p - bz * G.E[2];
+      rzoff_[q] = (col * G.rstride + pl * G.rplane) * 4;
+      dzoff_[q] = (col * G.dstride + pl * G.dplane) * 4;
+    }
     if (START == SWEEP_PROLONG) {
       const CoarseField& C = G.coarse;
       const int Z = p >> 1, cz = Z / C.E[2];
@@ -180,13 +213,18 @@ __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
   }
   __syncthreads();
   const int bx = gx / G.E[0], by = gy / G.E[1], byB = gyB / G.E[1];
-  const long long tcol = ((long long)(by * G.nb[0] + bx) * G.bstride +
-                          (long long)(gy - by * G.E[1]) * G.pitch + (gx - bx * G.E[0])) * 4;
-  const long long dB = ((long long)(byB - by) * G.nb[0] * G.bstride +  // row A to row B
-                        (long long)((gyB - byB * G.E[1]) - (gy - by * G.E[1])) * G.pitch) * 4;
+  // place of the thread's strip in row A, and from there to row B, in a field's plane 0
+  auto place = [&](long long stride, int pitch) {
+    return ((long long)(by * G.nb[0] + bx) * stride + (long long)(gy - by * G.E[1]) * pitch + (gx - bx * G.E[0])) * 4;
+  };
+  auto to_b = [&](long long stride, int pitch) {
+    return ((long long)(byB - by) * G.nb[0] * stride + (long long)((gyB - byB * G.E[1]) - (gy - by * G.E[1])) * pitch) * 4;
+  };
+  const long long tcol = place(G.bstride, G.pitch), dB = to_b(G.bstride, G.pitch);
   const char* src = (const char*)G.src + tcol;
-  const char* rhs = (const char*)G.rhs + tcol;
-  char* dst = (char*)G.dst + tcol;
+  const char* rhs = (const char*)G.rhs + (kOne ? tcol : place(G.rstride, G.rpitch));
+  char* dst = (char*)G.dst + (kOne ? tcol : place(G.dstride, G.dpitch));
+  const long long rdB = kOne ? dB : to_b(G.rstride, G.rpitch), ddB = kOne ? dB : to_b(G.dstride, G.dpitch);
   // the strip's two parents (rows A and B share them), and their slots in the ring
   const char* crs = nullptr;
   const uint32_t cring = ring + 4 * kDepth * rst - tid * 8, cst = kst;
@@ -211,7 +249,7 @@ __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
     const uint32_t n0 = neg ^ plane_neg(s_first - 1), n1 = neg ^ plane_neg(s_first);
     auto first = [&](long long dy, int q) {  // phi of plane z0 - 2 + q
       if (START == SWEEP_ZERO) return make_float4(0.f, 0.f, 0.f, 0.f);
-      const float4 v = *reinterpret_cast<const float4*>(src + dy + zoff[q]);
+      const float4 v = ld_strip<PAL>(src + dy + zoff[q]);
       if (START == SWEEP_SOURCE) return v;
       const float* c = reinterpret_cast<const float*>(crs + czoff[q]);
       return add_pairs(v, make_float2(c[0], c[1]));
@@ -221,11 +259,11 @@ __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
 #pragma unroll
     for (int d = 0; d < kDepth; ++d) {
       if (START != SWEEP_ZERO) {
-        cpa16(ring + (4 * d) * rst, src + zoff[2 + d]);
-        cpa16(ring + (4 * d + 1) * rst, src + dB + zoff[2 + d]);
+        cpa_strip<PAL>(ring + (4 * d) * rst, src + zoff[2 + d]);
+        cpa_strip<PAL>(ring + (4 * d + 1) * rst, src + dB + zoff[2 + d]);
       }
-      cpa16(ring + (4 * d + 2) * rst, rhs + zoff[1 + d]);
-      cpa16(ring + (4 * d + 3) * rst, rhs + dB + zoff[1 + d]);
+      cpa_strip<RAL>(ring + (4 * d + 2) * rst, rhs + rzoff[1 + d]);
+      cpa_strip<RAL>(ring + (4 * d + 3) * rst, rhs + rdB + rzoff[1 + d]);
       if (START == SWEEP_PROLONG) {
         cpa4(cring + d * cst, crs + czoff[2 + d]);
         cpa4(cring + d * cst + 4, crs + czoff[2 + d] + 4);
@@ -269,13 +307,13 @@ __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
     const float4 fA = lds4(slot + 2 * rst), fB = lds4(slot + 3 * rst);  // rhs of s
     {
       const int q = k + 2 + kDepth;
-      const long long o = zoff[q], o1 = zoff[q - 1];
+      const long long o = zoff[q], o1 = rzoff[q - 1];
       if (START != SWEEP_ZERO) {
-        cpa16(slot, src + o);
-        cpa16(slot + rst, src + dB + o);
+        cpa_strip<PAL>(slot, src + o);
+        cpa_strip<PAL>(slot + rst, src + dB + o);
       }
-      cpa16(slot + 2 * rst, rhs + o1);
-      cpa16(slot + 3 * rst, rhs + dB + o1);
+      cpa_strip<RAL>(slot + 2 * rst, rhs + o1);
+      cpa_strip<RAL>(slot + 3 * rst, rhs + rdB + o1);
       if (START == SWEEP_PROLONG) {
         cpa4(cslot, crs + czoff[q]);
         cpa4(cslot + 4, crs + czoff[q] + 4);
@@ -317,9 +355,9 @@ __global__ void __launch_bounds__(kMaxThreads, kBlocksPerSM)
     update((cur * 4 + 2) * kst, RA.bm, RB.bm, RA.r1b, RB.r1b, RA.r1a, rA, RB.r1a, rB, RA.rb1, RB.rb1, bA, bB);
     if (own && k >= 2) {  // plane s - 1 is final; its row A has parity P ^ 1
       const float2 xA = RA.r1b, xB = RB.r1b;
-      char* d = dst + zoff[k];
+      char* d = dst + dzoff[k];
       *reinterpret_cast<float4*>(d) = P ? make_float4(xA.x, bA.x, xA.y, bA.y) : make_float4(bA.x, xA.x, bA.y, xA.y);
-      *reinterpret_cast<float4*>(d + dB) = P ? make_float4(bB.x, xB.x, bB.y, xB.y) : make_float4(xB.x, bB.x, xB.y, bB.y);
+      *reinterpret_cast<float4*>(d + ddB) = P ? make_float4(bB.x, xB.x, bB.y, xB.y) : make_float4(xB.x, bB.x, xB.y, bB.y);
     }
     sts2(me + (nxt * 4) * kst, bnA);
     sts2(me + (nxt * 4 + 1) * kst, bnB);
@@ -542,6 +580,24 @@ bool sweep_geometry(const BoxArray& ba, const FabLayout& lay, const int periodic
   return true;
 }
 
+bool sweep_fabs_geometry(const BoxArray& ba, const FabLayout& phi, const FabLayout& rhs,
+                         const FabLayout& dst, const int periodic[3], double h, SweepGrid* out) {
+  Lattice P, R;
+  if (phi.ncomp != 1 || rhs.ncomp != 1 || phi.esize != 4 || rhs.esize != 4) return false;
+  if (!sweep_geometry(ba, dst, periodic, h, out) || !lattice_of(ba, phi, &P) || !lattice_of(ba, rhs, &R))
+    return false;
+  out->dpitch = out->pitch;
+  out->dplane = out->plane;
+  out->dstride = out->bstride;
+  out->pitch = P.pitch;
+  out->plane = P.plane;
+  out->bstride = P.bstride;
+  out->rpitch = R.pitch;
+  out->rplane = R.plane;
+  out->rstride = R.bstride;
+  return true;
+}
+
 // The tiling trades redundant work at a tile's rim against a full chip.  For each limit on a
 // block's threads every grid takes the strips x rows with the least redundancy, and for each
 // chunk length the launch is costed as waves of resident blocks: a plane takes a block set
@@ -686,6 +742,17 @@ cudaError_t launch_sweep_f32(const SweepGrid* grids, int ngrids, const SweepPlan
   cudaError_t e = opt_in_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   launch_k(k, (unsigned)p.tiles, p.threads, smem, s, grids, ngrids);
+  count_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sweep_f32_fabs(const SweepGrid* grid, const SweepPlan& p, int phi_ghosts, cudaStream_t s) {
+  // (rows start on 16 bytes, so the first valid cell is as aligned as the ghost cells before it)
+  const auto k = phi_ghosts % 2 == 0 ? k_sweep_f32<SWEEP_SOURCE, 8, 4> : k_sweep_f32<SWEEP_SOURCE, 4, 4>;
+  const size_t smem = (size_t)p.threads * (64 + 64 * kDepth);
+  cudaError_t e = opt_in_smem((const void*)k, smem);
+  if (e != cudaSuccess) return e;
+  launch_k(k, (unsigned)p.tiles, p.threads, smem, s, grid, 1);
   count_launches(1);
   return cudaGetLastError();
 }

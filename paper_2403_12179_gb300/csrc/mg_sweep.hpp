@@ -37,6 +37,10 @@ struct SweepGrid {
   int par0;           // colour parity of the domain's low corner
   float mh2;          // -h^2
   CoarseField coarse; // the coarser level's field (SWEEP_PROLONG); base null: none
+  // sweeps of fabs with ghost cells (launch_sweep_f32_fabs): the layouts of rhs and dst, which above
+  // have the source's
+  int rpitch, rplane, dpitch, dplane;
+  long long rstride, dstride;
   // tiling, set by plan_sweep: S strips of 4 cells x TY rows x ZC planes per block, hx / hy
   // strips and rows read around it, nt tiles per dimension, first tile of this grid
   int S, TY, ZC, hx, hy;
@@ -92,5 +96,11 @@ extern const long long kSweepMinCells, kSweepMinCellsBatch;
 
 cudaError_t launch_sweep_f32(const SweepGrid* grids, int ngrids, const SweepPlan& p, int start,
                              cudaStream_t s);
+
+// The same sweep on a caller's FP32 fabs with ghost cells (not read): phi and rhs on lattices of any
+// alignment, dst of phi's boxes without ghosts.
+bool sweep_fabs_geometry(const BoxArray& ba, const FabLayout& phi, const FabLayout& rhs,
+                         const FabLayout& dst, const int periodic[3], double h, SweepGrid* out);
+cudaError_t launch_sweep_f32_fabs(const SweepGrid* grid, const SweepPlan& p, int phi_ghosts, cudaStream_t s);
 
 }  // namespace gbmg
