@@ -75,18 +75,17 @@ GB_HD double pow2(int k) {
 // (float)(r * 2^-e) with an exact product.  Applies when r is a normal double and the result is
 // a normal float or rounds up to infinity; false otherwise (zero, subnormal, infinite or NaN r,
 // or a result in the float subnormal range).
+// In 32-bit words (a dozen operations; the 64-bit form took twice that): the 29 dropped bits, plus
+// half a unit less one, plus the lowest kept bit, carry into the kept ones exactly when the value
+// rounds up (to nearest, ties to even).  |e| < 2^20.
 GB_HD bool scale_to_f32(double r, int e, float* out) {
   const uint64_t b = d2u(r);
-  const int Er = (int)((b >> 52) & 0x7FF);
-  if (Er == 0 || Er == 0x7FF) return false;
-  const long long F = (long long)Er - 1023 - e + 127;  // biased binary32 exponent
-  if (F < 1 || F > 254) return false;
-  const uint64_t m = b & 0xFFFFFFFFFFFFFull;          // 52 fraction bits
-  uint32_t base = (uint32_t)(b >> 63) << 31 | (uint32_t)F << 23 | (uint32_t)(m >> 29);
-  const uint64_t rem = m & 0x1FFFFFFFull, half = 0x10000000ull;  // the 29 dropped bits
-  base += (rem > half || (rem == half && (base & 1u))) ? 1u : 0u;  // a carry bumps the exponent
-  *out = u2f(base);
-  return true;
+  const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+  const int Er = (int)((hi >> 20) & 0x7FF);
+  const int F = Er - 896 - e;  // biased binary32 exponent
+  const uint32_t base = (hi & 0x80000000u) | (uint32_t)F << 23 | (hi & 0xFFFFFu) << 3 | lo >> 29;
+  *out = u2f(base + (((lo & 0x1FFFFFFFu) + 0x0FFFFFFFu + (base & 1u)) >> 29));  // a carry bumps the exponent
+  return (unsigned)(Er - 1) < 2046u && (unsigned)(F - 1) < 254u;
 }
 
 // *out = 2^k * v exactly, for a finite float v whose scaled value is a normal double (zero

@@ -75,6 +75,19 @@ __device__ __forceinline__ T residual_of(T s, T phi, T rhs, T ih2) {
   return Ar<T>::fma(Ar<T>::neg(ih2), Ar<T>::fma(T(-6), phi, s), rhs);
 }
 
+// v * down rounded to binary32, as a loop (once round) so that the FP64 instructions stay behind a
+// branch: predicated off they would hold the FP64 pipe all the same.
+__device__ __forceinline__ float scale_f64(double v, double down) {
+  float f;
+  int n = blockDim.y;
+#pragma unroll 1
+  do {
+    v = __dmul_rn(v, down);
+    f = __double2float_rn(v);
+  } while (--n > 0);
+  return f;
+}
+
 // A level constant (h^2, 1/h^2; binary64 in the box table) in the kernel's type.  For binary32
 // the rounding is done with integer operations: a conversion would occupy the FP64 pipe once per
 // row and lane of an otherwise FP32 kernel.
@@ -85,7 +98,7 @@ __device__ __forceinline__ double level_const<double>(double d) { return d; }
 template <>
 __device__ __forceinline__ float level_const<float>(double d) {
   float f;
-  return bits::scale_to_f32(d, 0, &f) ? f : __double2float_rn(d);
+  return bits::scale_to_f32(d, 0, &f) ? f : scale_f64(d, 1.0);
 }
 
 constexpr int kWarps = 8;  // warps per block in the row kernels
@@ -617,32 +630,31 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) k_residual_r
   });
 }
 
-template <class T>
+// Plain restriction: G lanes per coarse x-line, the 8 children loaded first (128^3 FP64 in boxes of 32^3:
+// 14 us with a warp a line and one child at a time, 10 us now, ncu cold).
+template <class T, int G>
 __global__ void __launch_bounds__(kThreads) k_restrict(SegList L, long long nrows, long long per) {
   pdl_begin();
-  const int lane = threadIdx.x & 31;
-  for_rows(L, nrows, per, [&](const DRow& R, long long lr, int) {
+  const int lane = threadIdx.x & (G - 1);
+  for_rows<32 / G>(L, nrows, per, [&](const DRow& R, long long lr, int) {
     const int nc0 = R.n[0] >> 1, nc1 = R.n[1] >> 1;
     const int Y = (int)lr % nc1, Z = (int)lr / nc1;
-    T* c = line<T>(R.c[0], Y, Z);
-    for (int X = lane; X < nc0; X += 32) {
-      T acc = T(0);
+    T* __restrict__ c = line<T>(R.c[0], Y, Z);
+    for (int X = lane; X < nc0; X += G) {
+      T v[8];
 #pragma unroll
-      for (int k = 0; k < 2; ++k)
+      for (int q = 0; q < 8; ++q) v[q] = __ldg(line<T>(R.v[0], 2 * Y + ((q >> 1) & 1), 2 * Z + (q >> 2)) + 2 * X + (q & 1));
+      T acc = v[0];
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            T v = line<T>(R.v[0], 2 * Y + j, 2 * Z + k)[2 * X + i];
-            acc = (i | j | k) ? Ar<T>::add(acc, v) : v;
-          }
+      for (int q = 1; q < 8; ++q) acc = Ar<T>::add(acc, v[q]);
       c[X] = Ar<T>::mul(acc, (T)0.125);
     }
   });
 }
 
 // fine(c) += coarse(floor(c / 2)); c[0] addresses coarse cell floor(lo / 2).  G lanes per
-// fine x-line.
+// fine x-line.  Bound by HBM (FP64: 17 bytes a cell): 256^3 FP64 66 us with one cell a lane, 50 us with
+// pairs (5.6 TB/s, 83% of the copy rate; two pairs a step the same).
 template <class T, int G>
 __global__ void __launch_bounds__(kThreads) k_prolong_add(SegList L, long long nrows, long long per) {
   pdl_begin();
@@ -670,6 +682,13 @@ __global__ void __launch_bounds__(kThreads) k_prolong_add(SegList L, long long n
           const int xq = x + G * q;
           if (xq < n0) f[xq] = Ar<T>::add(a[q], b[q]);
         }
+      }
+    } else if (!ox && !(n0 & 1) && !((uintptr_t)f & 15)) {
+      // FP64: a lane takes both children of a parent
+      for (int x = 2 * lane; x < n0; x += 2 * G) {
+        const double2 a = *(const double2*)(f + x);
+        const T b = c[x >> 1];
+        *(double2*)(f + x) = make_double2(Ar<T>::add(a.x, b), Ar<T>::add(a.y, b));
       }
     } else {
       for (int x = lane; x < n0; x += G) f[x] = Ar<T>::add(f[x], c[(x + ox) >> 1]);
@@ -852,31 +871,44 @@ __global__ void __launch_bounds__(kThreads) k_copy_valid(SegList L, long long nr
   });
 }
 
-template <class T>
+// Max-norm of a field: G lanes per x-line, kCopyCells loads of a lane in flight (128^3 FP64 in boxes of
+// 32^3: 17.9 us with a warp a line and one load, 9.9 us now, ncu cold).
+template <class T, int G>
 __global__ void __launch_bounds__(kThreads) k_maxabs(SegList L, long long nrows, long long per,
                                                      unsigned long long* norms) {
   pdl_begin();
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & (G - 1);
   unsigned long long mx = 0;
   int cur = -1;
-  for_rows(L, nrows, per, [&](const DRow& R, long long lr, int slot) {
+  for_rows<32 / G>(L, nrows, per, [&](const DRow& R, long long lr, int slot) {
     const int idx = slot + R.solve;
-    if (idx != cur) {
-      if (cur >= 0) {
-        unsigned long long m = Ar<T>::key_to_f64bits(warp_max(mx));
-        if (lane == 0 && m) atomicMax(&norms[cur], m);
-      }
+    if (idx != cur) {  // (a lane group's own maximum: the groups of a warp may be in different solves)
+      if (cur >= 0 && mx) atomicMax(&norms[cur], Ar<T>::key_to_f64bits(mx));
       cur = idx;
       mx = 0;
     }
     const int n0 = R.n[0], n1 = R.n[1];
     const int y = (int)lr % n1, z = (int)lr / n1;
-    const T* f = line<T>(R.v[0], y, z);
-    for (int x = lane; x < n0; x += 32) {
-      unsigned long long k = Ar<T>::abskey(f[x]);
-      mx = k > mx ? k : mx;
+    const T* __restrict__ f = line<T>(R.v[0], y, z);
+    for (int x = lane; x < n0; x += kCopyCells * G) {
+      T v[kCopyCells];
+#pragma unroll
+      for (int k = 0; k < kCopyCells; ++k) v[k] = x + G * k < n0 ? f[x + G * k] : T(0);
+#pragma unroll
+      for (int k = 0; k < kCopyCells; ++k) {
+        const unsigned long long q = Ar<T>::abskey(v[k]);
+        mx = q > mx ? q : mx;
+      }
     }
   });
+  // the block's maxima, one atomic per run of equal solves over its warps; where a warp's lanes ended in
+  // different solves, one per lane group
+  const unsigned same = __match_any_sync(0xffffffffu, cur);
+  if (same != 0xffffffffu) {
+    if (cur >= 0 && mx) atomicMax(&norms[cur], Ar<T>::key_to_f64bits(mx));
+    mx = 0;
+    cur = -1;
+  }
   flush_block_max(Ar<T>::key_to_f64bits(warp_max(mx)), cur, norms);
 }
 
@@ -889,8 +921,11 @@ __device__ __forceinline__ double pow2_floor_inv(double s) { return bits::pow2(-
 
 // r32 = float(r * 2^-e) with 2^e <= ||r||_inf < 2^(e+1), from the FP64 residual stored by the
 // preceding norm check (the same values the norm was taken over), and the FP32 correction's
-// initial guess e32 = 0.  G lanes per x-line, kScaleCells cells per lane step, loads first
-// (measured: 4 beats 8, which halves the lanes per row and the bytes per load instruction).
+// initial guess e32 = 0 (where the first sweep reads it).  G lanes per x-line, kScaleCells cells per
+// lane step, loads first (measured: 4 beats 8, which halves the lanes per row and the bytes per load
+// instruction), in pairs of cells where the rows are aligned.  Bound by HBM (12 bytes a cell) and the
+// conversion in turn: 512^3 349 us with 64-bit words and single cells, 317 us now (5.1 TB/s, 75% of the
+// copy rate); 509 us where the FP64 form of the conversion was predicated off instead of branched over.
 constexpr int kScaleCells = 4;
 template <int G>
 __global__ void __launch_bounds__(kThreads) k_scale_residual_f32(SegList L, long long nrows,
@@ -908,6 +943,29 @@ __global__ void __launch_bounds__(kThreads) k_scale_residual_f32(SegList L, long
     const double s = norm_of(norms, slot + R.solve);
     const int e = bits::floor_log2(s);
     const double down = pow2_floor_inv(s);
+    // the exact scaling and the rounding in integer operations where they apply
+    auto scaled = [&](double v) {
+      float f;
+      return bits::scale_to_f32(v, e, &f) ? f : scale_f64(v, down);
+    };
+    const bool pairs = !(n0 & 1) && !((uintptr_t)r & 15) && !((uintptr_t)r32 & 7) &&
+                       (!zero || !((uintptr_t)e32 & 7));
+    if (pairs) {
+      for (int x = 2 * sub; x < n0; x += kScaleCells * G) {
+        double2 v[kScaleCells / 2];
+#pragma unroll
+        for (int k = 0; k < kScaleCells / 2; ++k)
+          if (x + 2 * G * k < n0) v[k] = __ldg((const double2*)(r + x + 2 * G * k));
+#pragma unroll
+        for (int k = 0; k < kScaleCells / 2; ++k) {
+          const int xk = x + 2 * G * k;
+          if (xk >= n0) continue;
+          *(float2*)(r32 + xk) = make_float2(scaled(v[k].x), scaled(v[k].y));
+          if (zero) *(float2*)(e32 + xk) = make_float2(0.0f, 0.0f);
+        }
+      }
+      return;
+    }
     for (int x = sub; x < n0; x += kScaleCells * G) {
       double v[kScaleCells];
 #pragma unroll
@@ -916,10 +974,7 @@ __global__ void __launch_bounds__(kThreads) k_scale_residual_f32(SegList L, long
 #pragma unroll
       for (int k = 0; k < kScaleCells; ++k) {
         if (x + G * k >= n0) continue;
-        // the exact scaling and the rounding in integer operations where they apply
-        float f;
-        if (!bits::scale_to_f32(v[k], e, &f)) f = __double2float_rn(__dmul_rn(v[k], down));
-        r32[x + G * k] = f;
+        r32[x + G * k] = scaled(v[k]);
         if (zero) e32[x + G * k] = 0.0f;
       }
     }
@@ -1210,7 +1265,7 @@ cudaError_t launch_prolong_trilinear_l(int dt, const SegList& L, long long nrows
 
 cudaError_t launch_prolong_add_l(int dt, const SegList& L, long long nrows, cudaStream_t s) {
   if (nrows <= 0) return cudaSuccess;
-  const int G = group_lanes(L.width, dt == DT_F64 ? 1 : 4, 8, 32);  // cells per lane step
+  const int G = group_lanes(L.width, dt == DT_F64 ? 2 : 4, 8, 32);  // cells per lane step
   const Grid g = row_grid(nrows, row_blocks_per_sm(L.width), kWarps * (32 / G));
   if (dt == DT_F64) prolong_add_g<double>(G, g, s, L, nrows);
   else prolong_add_g<float>(G, g, s, L, nrows);
@@ -1257,8 +1312,18 @@ cudaError_t launch_set_valid_l(int dt, const SegList& L, long long nrows, double
 cudaError_t launch_maxabs_l(int dt, const SegList& L, long long nrows, unsigned long long* norms,
                             cudaStream_t s) {
   if (nrows <= 0) return cudaSuccess;
-  Grid g = row_grid(nrows, 4);
-  GB_DISPATCH(dt, k_maxabs, g.blocks, kThreads, 0, s, L, nrows, g.per, norms);
+  const int G = group_lanes(L.width, kCopyCells, 8, 32);
+  const Grid g = row_grid(nrows, 8, kWarps * (32 / G));
+  auto go = [&](auto k) { launch_k(k, g.blocks, kThreads, 0, s, L, nrows, g.per, norms); };
+  if (dt == DT_F64) {
+    if (G == 32) go(k_maxabs<double, 32>);
+    else if (G == 16) go(k_maxabs<double, 16>);
+    else go(k_maxabs<double, 8>);
+  } else {
+    if (G == 32) go(k_maxabs<float, 32>);
+    else if (G == 16) go(k_maxabs<float, 16>);
+    else go(k_maxabs<float, 8>);
+  }
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1328,10 +1393,21 @@ cudaError_t launch_rbgs_half_store(const DRow* rows, int nbox, long long nrows, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_restrict(int dt, const DRow* rows, int nbox, long long nrows, cudaStream_t s) {
+cudaError_t launch_restrict(int dt, const DRow* rows, int nbox, long long nrows, cudaStream_t s, int width) {
   if (nrows <= 0) return cudaSuccess;
-  Grid g = row_grid(nrows, 16);
-  GB_DISPATCH(dt, k_restrict, g.blocks, kThreads, 0, s, one_seg(rows, nbox), nrows, g.per);
+  const int G = group_lanes(width, 2, 8, 32);  // rows are coarse lines of width / 2 cells
+  const Grid g = row_grid(nrows, row_blocks_per_sm(width), kWarps * (32 / G));
+  const SegList L = one_seg(rows, nbox, 0, width);
+  auto go = [&](auto k) { launch_k(k, g.blocks, kThreads, 0, s, L, nrows, g.per); };
+  if (dt == DT_F64) {
+    if (G == 32) go(k_restrict<double, 32>);
+    else if (G == 16) go(k_restrict<double, 16>);
+    else go(k_restrict<double, 8>);
+  } else {
+    if (G == 32) go(k_restrict<float, 32>);
+    else if (G == 16) go(k_restrict<float, 16>);
+    else go(k_restrict<float, 8>);
+  }
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1417,8 +1493,8 @@ cudaError_t launch_copy_valid_f32(const DRow* rows, int nbox, long long nrows, c
 }
 
 cudaError_t launch_maxabs(int dt, const DRow* rows, int nbox, long long nrows,
-                          unsigned long long* norms, cudaStream_t s) {
-  return launch_maxabs_l(dt, one_seg(rows, nbox), nrows, norms, s);
+                          unsigned long long* norms, cudaStream_t s, int width) {
+  return launch_maxabs_l(dt, one_seg(rows, nbox, 0, width), nrows, norms, s);
 }
 
 cudaError_t launch_scale_residual_f32(const DRow* rows, int nbox, long long nrows,

@@ -274,7 +274,8 @@ cudaError_t launch_half_march(const SegList& L, int mode, int color, unsigned lo
                               cudaStream_t s);
 
 // Rows are coarse x-lines.  v[0] = fine field; c[0] = coarse field.
-cudaError_t launch_restrict(int dt, const DRow* rows, int nbox, long long nrows, cudaStream_t s);
+cudaError_t launch_restrict(int dt, const DRow* rows, int nbox, long long nrows, cudaStream_t s,
+                            int width = 0);
 
 // Rows are fine x-lines.  v[0] = fine field (+=); c[0] = coarse field.
 cudaError_t launch_prolong_add(int dt, const DRow* rows, int nbox, long long nrows,
@@ -324,7 +325,7 @@ cudaError_t launch_copy_valid_f32(const DRow* rows, int nbox, long long nrows, c
 
 // max |value| over valid cells, atomicMax of bit patterns into norms[solve]; v[0] = field.
 cudaError_t launch_maxabs(int dt, const DRow* rows, int nbox, long long nrows,
-                          unsigned long long* norms, cudaStream_t s);
+                          unsigned long long* norms, cudaStream_t s, int width = 0);
 
 // Mixed precision.  v[0] = r (FP64 residual stored by the norm check), c[0] = r32 out,
 // c[1] = e32 out (FP32 views with the same box geometry): r32 = float(r * 2^-e) with

@@ -1416,7 +1416,7 @@ int mg_restrict(mg_ctx_t h, mg_fab_t fine, mg_fab_t coarse, void* stream) {
         R.c[0] = coarse_view(*fc, map[b], F.boxes[b]);
       }, c->stream);
     });
-    MG_CK(launch_restrict(ff->dtype, t.rows(), t.nbox, t.nrows, s));
+    MG_CK(launch_restrict(ff->dtype, t.rows(), t.nbox, t.nrows, s, t.width));
     return MG_OK;
   });
 }

@@ -668,7 +668,7 @@ int solve(Ctx& c, int64_t rhs_id, int64_t phi_id, const mg_bc* bc, double tol,
   unsigned long long* dn = (unsigned long long*)H.dnorm->p;
   // ||rhs||_inf and the first residual norm
   MG_CK(cudaMemsetAsync(dn, 0, 16, s));
-  MG_CK(launch_maxabs(DT_F64, H.rhsabs0.rows(), H.rhsabs0.nbox, H.rhsabs0.nrows, dn, s));
+  MG_CK(launch_maxabs(DT_F64, H.rhsabs0.rows(), H.rhsabs0.nbox, H.rhsabs0.nrows, dn, s, H.rhsabs0.width));
   if (!H.direct0) launch_fill(c, *H.phi0, bc, s, 1);
   MG_CK(launch_residual(DT_F64, H.resid0.rows(), H.resid0.nbox, H.resid0.nrows, dn, s, H.direct0, -1,
                         H.resid0.ext));
