@@ -84,9 +84,11 @@ typedef struct {
   int fixed_vcycles;  /* >= 0: run exactly this many V-cycles, no stop test; -1 default */
   double h;           /* cell size; 0 (default) means 1 / (domain x extent) */
   int coarse_cells;   /* the levels from the first one with at most this many cells down to
-                         the bottom run as ONE launch per V-cycle (one CTA per solve, levels
-                         held in shared memory; same arithmetic, bit-identical results).
-                         0 (default): 512 for FP64 levels, 4096 for FP32 levels; -1: off */
+                         the bottom run as ONE launch per V-cycle (levels held in the shared
+                         memory of one CTA per solve, or of a cluster of eight for a solve on
+                         its own; same arithmetic, bit-identical results).
+                         0 (default): 512 for FP64 levels, 4096 for FP32 levels with one CTA,
+                         and with a cluster what is fastest (16^3 cells); -1: off */
   int direct_reads;   /* 1 (default): on levels whose boxes form a regular grid, the
                          smoother, residual and residual+restriction read the neighbouring
                          boxes (or the periodic image, or the negated boundary cell across a

@@ -160,22 +160,18 @@ std::map<Ctx*, std::vector<std::shared_ptr<AmrPlan>>> g_plans;
 // Element offset of global cell (x, y, z) of a fab (the box owning it).
 struct Owner {
   const FabObj* f;
-  std::map<std::array<int, 3>, int> cell_box;  // only the cells asked about, cached
-  long long at(int x, int y, int z) {
-    const BoxArray& ba = f->ba->ba;
-    auto key = std::array<int, 3>{x, y, z};
-    auto it = cell_box.find(key);
-    int b = -1;
-    if (it != cell_box.end()) {
-      b = it->second;
-    } else {
-      for (size_t k = 0; k < ba.boxes.size(); ++k)
-        if (contains(ba.boxes[k], x, y, z)) { b = (int)k; break; }
-      if (b < 0) fail(MG_EINVAL, "internal: cell outside every box");
-      cell_box[key] = b;
+  size_t last = 0;  // the box of the last cell asked about: the next one is mostly there too
+  int box_of(int x, int y, int z) {
+    const std::vector<Box>& bs = f->ba->ba.boxes;
+    if (!contains(bs[last], x, y, z)) {
+      size_t k = 0;
+      while (k < bs.size() && !contains(bs[k], x, y, z)) ++k;
+      if (k == bs.size()) fail(MG_EINVAL, "internal: cell outside every box");
+      last = k;
     }
-    return f->lay.at(ba, b, x, y, z);
+    return (int)last;
   }
+  long long at(int x, int y, int z) { return f->lay.at(f->ba->ba, box_of(x, y, z), x, y, z); }
 };
 
 DView sub_view(const FabObj& f, int b, const int lo[3]) {
@@ -279,7 +275,7 @@ AmrPlan& get_plan(Ctx& c, int64_t rhs0, int64_t phi0, int64_t rhs1, int64_t phi1
       if (h.get() == &H) P->H = h;
   }
   // coarse/fine ghost list
-  Owner of{f1.get(), {}}, oc{f0.get(), {}};
+  Owner of{f1.get()}, oc{f0.get()};
   std::vector<CFGhost> cf;
   std::vector<CFFine> cff;
   for (int cds = 0; cds < 12; ++cds) {  // colour of the first fine cell, dimension, side
@@ -302,7 +298,7 @@ AmrPlan& get_plan(Ctx& c, int64_t rhs0, int64_t phi0, int64_t rhs1, int64_t phi1
         ef.f1 = of.at(q1[0], q1[1], q1[2]);
         ef.f2 = of.at(q2[0], q2[1], q2[2]);
         // the ghost lives in the box of the first fine cell, one cell outside along d
-        const int gb = of.cell_box[{q1[0], q1[1], q1[2]}];
+        const int gb = of.box_of(q1[0], q1[1], q1[2]);
         int gq[3] = {q1[0], q1[1], q1[2]};
         gq[d] -= step;
         ef.dst = f1->lay.at(F, gb, gq[0], gq[1], gq[2]);
@@ -325,7 +321,7 @@ AmrPlan& get_plan(Ctx& c, int64_t rhs0, int64_t phi0, int64_t rhs1, int64_t phi1
   P->cff = c.upload(cff.data(), cff.size() * sizeof(CFFine), s);
   P->cfc = c.alloc(cf.size() * sizeof(double), s);
   // coarse cells beside the fine region, with the four fine faces of their shared face
-  Owner orr{r0.get(), {}};
+  Owner orr{r0.get()};
   std::vector<RefluxCell> rf;
   for (int d = 0; d < 3; ++d) {
     const int t0 = d == 0 ? 1 : 0, t1 = d == 2 ? 1 : 2;
@@ -353,7 +349,7 @@ AmrPlan& get_plan(Ctx& c, int64_t rhs0, int64_t phi0, int64_t rhs1, int64_t phi1
               q[t0] = 2 * I + a;
               q[t1] = 2 * J + b;
               e.f[k] = of.at(q[0], q[1], q[2]);
-              const int gb = of.cell_box[{q[0], q[1], q[2]}];
+              const int gb = of.box_of(q[0], q[1], q[2]);
               q[d] -= step;
               e.g[k] = f1->lay.at(F, gb, q[0], q[1], q[2]);
             }

@@ -72,15 +72,19 @@ struct BottomJob {
   int pad_;
 };
 
-// The coarse end of a V-cycle (levels lc .. bottom) in one CTA: every level held densely in
-// shared memory (phi, then rhs, x fastest; then level lc's residuals at off_res), offsets in
-// elements of the level's type.  Level lc's cell i (dense, x fastest) lives at phi[off_phi[i]] and
-// rhs[off_rhs[i]] in its fabs: phi and rhs are gathered from there and phi scattered back.
-constexpr int kMaxCoarseLevels = 8;
+// The coarse end of a V-cycle (levels lc .. bottom) in one launch, by one CTA or a cluster of `ranks`
+// CTAs: every level held densely in shared memory (phi, then rhs, x fastest; the residuals of one
+// level at off_res), offsets in elements of the level's type, the same in every CTA.  A level is
+// either whole in the first CTA (planes 0) or in slabs of `planes` z-planes (an even number) over
+// the CTAs, phi with one plane of the neighbours' on either side; the levels in slabs come first.
+// Level lc's cell i (dense, x fastest) lives at phi[off_phi[i]] and rhs[off_rhs[i]] in its fabs:
+// phi and rhs are gathered from there and phi scattered back.
+constexpr int kMaxCoarseLevels = 8, kCoarseRanks = 8;
 struct CoarseLevel {
   int n[3];   // level domain extents
   int lo[3];  // level domain low corner (colour parity, gather offsets)
   int off_phi, off_rhs;
+  int planes, pad_;
   double h2, ih2;
 };
 struct CoarseJob {
@@ -92,6 +96,7 @@ struct CoarseJob {
   int nlev, nu1, nu2, N;
   int periodic[3];
   int off_res;
+  int ranks, nslab;  // CTAs, levels in slabs (0 with one CTA)
   CoarseLevel lev[kMaxCoarseLevels];
 };
 
@@ -207,6 +212,24 @@ __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 template <class... P, class... A>
+inline void launch_cluster_k(int cluster, void (*k)(P...), dim3 grid, dim3 block, size_t smem,
+                             cudaStream_t s, A&&... a) {
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cluster;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl_enabled() ? 2 : 1;
+  cudaLaunchKernelEx(&cfg, k, static_cast<A&&>(a)...);  // errors: cudaGetLastError()
+}
+template <class... P, class... A>
 inline void launch_k(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                      A&&... a) {
   cudaLaunchAttribute at[1];
@@ -297,14 +320,15 @@ cudaError_t launch_rbgs_fused(int dt, const DRow* rows, const int4* units, int n
 
 cudaError_t launch_bottom(int dt, const BottomJob* jobs, int njobs, int maxN, cudaStream_t s);
 
-// Shared memory of a coarse job whose levels have extents n[0..nlev); launch with the largest
-// value over the jobs.
-size_t coarse_smem_bytes(int dt, const int (*n)[3], int nlev);
+// Places of J's levels (extents set), in slabs over a cluster if `cluster` and where they are large
+// enough; sets ranks, nslab, planes and the offsets.  Returns the bytes of shared memory, or 0 if
+// `bounded` and a level is too large for its CTAs to be worth it.
+size_t coarse_layout(int dt, CoarseJob& J, bool cluster, bool bounded);
 constexpr size_t kCoarseSmemMax = 200 * 1024;
 // Raises the kernel's shared-memory limit to smem (once; call outside stream capture).
-cudaError_t coarse_opt_in(int dt, size_t smem);
+cudaError_t coarse_opt_in(int dt, size_t smem, int ranks);
 cudaError_t launch_coarse_cycle(int dt, const CoarseJob* jobs, int njobs, size_t smem,
-                                cudaStream_t s);
+                                cudaStream_t s, int ranks = 1);
 
 // v[0] += v[1] on valid cells.
 cudaError_t launch_add_valid(int dt, const DRow* rows, int nbox, long long nrows, cudaStream_t s);

@@ -8,6 +8,7 @@
 // one CUDA graph.
 #include <cuda_runtime.h>
 
+#include <climits>
 #include <cmath>
 #include <cstring>
 
@@ -213,76 +214,93 @@ void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
   J.N = (int)N;
   H.job = c.upload(&J, sizeof J, s);
   H.job_host = J;
-  // The coarse end of the cycle as one launch: from the first level with at most
-  // `limit` cells whose levels (down to the bottom) fit into shared memory.
-  H.lc = nl;
-  const int limit = H.p.coarse_cells != 0 ? H.p.coarse_cells : (H.dt == DT_F64 ? 512 : 4096);
-  // (the coarse-cycle kernel prolongs by injection: the trilinear form runs level by level)
+  // The coarse end of the cycle as one launch: from the first level with at most `limit` cells whose
+  // levels (down to the bottom) fit into shared memory.  (The coarse-cycle kernel prolongs by
+  // injection: the trilinear form runs level by level.)
   const bool one_launch = H.p.coarse_cells >= 0 && H.p.prolong == MG_PROLONG_CONSTANT;
-  for (int l = std::max(0, nl - kMaxCoarseLevels); one_launch && l + 1 < nl; ++l) {
-    if (H.L[l].bao->ba.dom.npts() > limit) continue;
-    int ext[kMaxCoarseLevels][3];
-    for (int k = l; k < nl; ++k)
-      for (int d = 0; d < 3; ++d) ext[k - l][d] = H.L[k].bao->ba.dom.len(d);
-    const size_t smem = coarse_smem_bytes(H.dt, ext, nl - l);
-    if (smem > kCoarseSmemMax) continue;
-    // level l's cells, dense and x fastest, in its phi and rhs fabs
-    const LevelData& T = H.L[l];
-    const BoxArray& tb = T.bao->ba;
-    const long long nt = tb.dom.npts();
-    std::vector<long long> offs(2 * nt);
-    for (size_t b = 0; b < tb.boxes.size(); ++b) {
-      const Box& X = tb.boxes[b];
-      for (int z = X.lo[2]; z <= X.hi[2]; ++z)
-        for (int y = X.lo[1]; y <= X.hi[1]; ++y)
-          for (int x = X.lo[0]; x <= X.hi[0]; ++x) {
-            long long i = ((long long)(z - tb.dom.lo[2]) * ext[0][1] + (y - tb.dom.lo[1])) *
-                              ext[0][0] + (x - tb.dom.lo[0]);
-            offs[i] = T.phi->lay.at(tb, (int)b, x, y, z);
-            offs[nt + i] = T.rhs->lay.at(tb, (int)b, x, y, z);
-          }
-    }
-    H.coff = c.upload(offs.data(), offs.size() * 8, s);
-    CoarseJob& C = H.cjob_host;
-    C = CoarseJob{};
-    C.off_phi = (const long long*)H.coff->p;
-    C.off_rhs = C.off_phi + nt;
-    C.phi = T.phi->base;
-    C.rhs = T.rhs->base;
-    C.Mt = J.Mt;
-    C.N = J.N;
-    C.nlev = nl - l;
-    C.nu1 = H.p.nu1;
-    C.nu2 = H.p.nu2;
-    for (int d = 0; d < 3; ++d) C.periodic[d] = per[d];
-    int off = 0;
-    for (int k = 0; k < C.nlev; ++k) {
-      const LevelData& D = H.L[l + k];
-      CoarseLevel& V = C.lev[k];
-      for (int d = 0; d < 3; ++d) {
-        V.n[d] = ext[k][d];
-        V.lo[d] = D.bao->ba.dom.lo[d];
+  struct Coarse {
+    int lc;
+    CoarseJob J;
+    DevBufP job, off;
+    size_t smem;
+  };
+  auto coarse_from = [&](int first, long long limit, bool cluster, bool bounded) {
+    Coarse R{nl, {}, nullptr, nullptr, 0};
+    for (int l = std::max(first, nl - kMaxCoarseLevels); one_launch && l + 1 < nl; ++l) {
+      if (H.L[l].bao->ba.dom.npts() > limit) continue;
+      CoarseJob& C = R.J;
+      C = CoarseJob{};
+      C.nlev = nl - l;
+      for (int k = 0; k < C.nlev; ++k) {
+        const LevelData& D = H.L[l + k];
+        CoarseLevel& V = C.lev[k];
+        for (int d = 0; d < 3; ++d) {
+          V.n[d] = D.bao->ba.dom.len(d);
+          V.lo[d] = D.bao->ba.dom.lo[d];
+        }
+        V.h2 = D.h * D.h;
+        V.ih2 = 1.0 / (D.h * D.h);
       }
-      V.h2 = D.h * D.h;
-      V.ih2 = 1.0 / (D.h * D.h);
-      V.off_phi = off;
-      off += V.n[0] * V.n[1] * V.n[2];
-      V.off_rhs = off;
-      off += V.n[0] * V.n[1] * V.n[2];
+      R.smem = coarse_layout(H.dt, C, cluster, bounded);
+      if (!R.smem || R.smem > kCoarseSmemMax) continue;
+      // level l's cells, dense and x fastest, in its phi and rhs fabs
+      const LevelData& T = H.L[l];
+      const BoxArray& tb = T.bao->ba;
+      const long long nt = tb.dom.npts();
+      std::vector<long long> offs(2 * nt);
+      for (size_t b = 0; b < tb.boxes.size(); ++b) {
+        const Box& X = tb.boxes[b];
+        for (int z = X.lo[2]; z <= X.hi[2]; ++z)
+          for (int y = X.lo[1]; y <= X.hi[1]; ++y)
+            for (int x = X.lo[0]; x <= X.hi[0]; ++x) {
+              long long i = ((long long)(z - tb.dom.lo[2]) * C.lev[0].n[1] + (y - tb.dom.lo[1])) *
+                                C.lev[0].n[0] + (x - tb.dom.lo[0]);
+              offs[i] = T.phi->lay.at(tb, (int)b, x, y, z);
+              offs[nt + i] = T.rhs->lay.at(tb, (int)b, x, y, z);
+            }
+      }
+      R.off = c.upload(offs.data(), offs.size() * 8, s);
+      C.off_phi = (const long long*)R.off->p;
+      C.off_rhs = C.off_phi + nt;
+      C.phi = T.phi->base;
+      C.rhs = T.rhs->base;
+      C.Mt = J.Mt;
+      C.N = J.N;
+      C.nu1 = H.p.nu1;
+      C.nu2 = H.p.nu2;
+      for (int d = 0; d < 3; ++d) C.periodic[d] = per[d];
+      MG_CK(coarse_opt_in(H.dt, R.smem, C.ranks));
+      R.job = c.upload(&C, sizeof C, s);
+      R.lc = l;
+      break;
     }
-    C.off_res = off;
-    H.csmem = smem;
-    MG_CK(coarse_opt_in(H.dt, smem));
-    H.cjob = c.upload(&C, sizeof C, s);
-    H.lc = l;
-    break;
+    return R;
+  };
+  const bool set = H.p.coarse_cells != 0;
+  const int limit = set ? H.p.coarse_cells : (H.dt == DT_F64 ? 512 : 4096);
+  Coarse one = coarse_from(0, limit, false, false);
+  H.lc = H.slc = one.lc;
+  H.cjob_host = one.J;
+  H.csmem = one.smem;
+  H.cjob = std::move(one.job);
+  H.coff = std::move(one.off);
+  if (one.lc > 0 && one.lc < nl) {
+    // (from level 1 at the finest: the finest level of a solve keeps its half-sweeps)
+    Coarse many = coarse_from(1, set ? limit : LLONG_MAX, true, !set);
+    if (many.lc < nl && many.J.ranks > 1) {
+      H.slc = many.lc;
+      H.sranks = many.J.ranks;
+      H.scsmem = many.smem;
+      H.scjob = std::move(many.job);
+      H.scoff = std::move(many.off);
+    }
   }
   for (int l = 0; l + 1 < nl; ++l) {
     LevelData& D = H.L[l];
     if (!D.wide_rr) continue;
     std::vector<RestrictGrid> q{D.rr_grid};
     // (a coarser level that starts its sweeps from zero needs no zeros)
-    if (H.L[l + 1].zero_start && l + 1 < H.lc) q[0].cphi.base = nullptr;
+    if (H.L[l + 1].zero_start && l + 1 < H.slc) q[0].cphi.base = nullptr;
     D.rr_plan = plan_restrict(q);
     D.rr_dev = c.upload(q.data(), sizeof(RestrictGrid), s);
   }
@@ -502,7 +520,7 @@ void smooth(Ctx& c, Hierarchy& H, LevelData& D, int sweeps, cudaStream_t s,
 void enqueue_vcycle(Ctx& c, Hierarchy& H, cudaStream_t s, unsigned long long* norm0 = nullptr,
                     bool skip_first_red = false, bool zero0 = false) {
   const int nl = (int)H.L.size();
-  const int top = H.lc < nl ? H.lc : nl - 1;  // levels below `top` run stage by stage
+  const int top = H.slc < nl ? H.slc : nl - 1;  // levels below `top` run stage by stage
   for (int l = 0; l < top; ++l) {
     LevelData& D = H.L[l];
     if (D.fused) launch_fill(c, *D.rhs, &H.bc, s, 1);  // rhs ghosts for the redundant ring
@@ -518,7 +536,10 @@ void enqueue_vcycle(Ctx& c, Hierarchy& H, cudaStream_t s, unsigned long long* no
       MG_CK(launch_residual_restrict(H.dt, D.rr.rows(), D.rr.nbox, D.rr.nrows, s, D.direct,
                                      D.rr.width, stored, D.rr.ext));
   }
-  if (H.lc < nl) MG_CK(launch_coarse_cycle(H.dt, (const CoarseJob*)H.cjob->p, 1, H.csmem, s));
+  if (H.sranks > 1)
+    MG_CK(launch_coarse_cycle(H.dt, (const CoarseJob*)H.scjob->p, 1, H.scsmem, s, H.sranks));
+  else if (H.slc < nl)
+    MG_CK(launch_coarse_cycle(H.dt, (const CoarseJob*)H.cjob->p, 1, H.csmem, s));
   else MG_CK(launch_bottom(H.dt, (const BottomJob*)H.job->p, 1, H.N, s));
   for (int l = top - 1; l >= 0; --l) {
     LevelData& D = H.L[l];

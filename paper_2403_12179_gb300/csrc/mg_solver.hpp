@@ -54,6 +54,11 @@ struct Hierarchy {
   size_t csmem = 0;
   DevBufP cjob, coff;
   CoarseJob cjob_host{};
+  // the same of a solve on its own, by a cluster of CTAs, from a finer level (slc <= lc; a batch, whose
+  // jobs fill the SMs, takes one CTA a job)
+  int slc = 0, sranks = 1;
+  size_t scsmem = 0;
+  DevBufP scjob, scoff;
   DevBufP dnorm;  // [0] residual norm bits, [1] rhs norm bits
   unsigned long long* hnorm = nullptr;
   BottomJob job_host{};
