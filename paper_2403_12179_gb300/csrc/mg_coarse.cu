@@ -329,19 +329,24 @@ __device__ void prolong_add(const Lev<T>& C, const Lev<T>& F) {
   }
 }
 
-template <class T>
-__device__ void bottom(const Lev<T>& B, const double* __restrict__ Mt, int N) {
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+// Rows [i0, i1) of the exact bottom solve; phi(i, value) takes them.
+template <class T, class F>
+__device__ void bottom(const T* rhs, const double* __restrict__ Mt, int N, int i0, int i1, F&& phi) {
+  for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
     double s = 0.0;
-#pragma unroll 8
-    for (int j = 0; j < N; ++j) s = __dadd_rn(s, __dmul_rn(Mt[(long long)j * N + i], (double)B.rhs[j]));
-    B.phi[i] = (T)s;
+#pragma unroll 16
+    for (int j = 0; j < N; ++j) s = __dadd_rn(s, __dmul_rn(Mt[(long long)j * N + i], (double)rhs[j]));
+    phi(i, (T)s);
   }
 }
+// Cells from which the bottom solve's rows are spread over the CTAs of a cluster: one SM's FP64 pipe
+// takes 2 N^2 / 1.68 clocks (27 us for 210 cells).
+constexpr int kBottomSpread = 64;
 
 // 512 threads for FP64 (128 registers each), 1024 for FP32.  RANKS: CTAs of a job, a cluster.
 // Every CTA of a cluster passes the same cluster barriers: one after the gather, those of the levels
-// in slabs, and one between the levels of the first CTA alone and theirs.
+// in slabs, two around a bottom solve that is spread, and one between the levels of the first CTA alone
+// and those in slabs.
 template <class T, int RANKS>
 __global__ void __launch_bounds__(sizeof(T) == 8 ? 512 : 1024, 1) k_coarse_cycle(const CoarseJob* __restrict__ jobs) {
   constexpr bool CL = RANKS > 1;
@@ -384,8 +389,19 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 512 : 1024, 1) k_coarse_cycle
     smooth<T, CL>(L[k], M, per, J.nu1, ints);
     residual_restrict<T, CL>(L[k], M, L[k + 1], res, per, ints);
   }
+  const Lev<T>& B = L[nl - 1];
+  const bool spread = CL && J.N >= kBottomSpread;
+  if (spread) {
+    cluster_sync();
+    if (rank)
+      for (int i = threadIdx.x; i < J.N; i += blockDim.x) ld_peer(peer(B.rhs + i, 0), B.rhs[i]);
+    __syncthreads();
+    bottom(B.rhs, J.Mt, J.N, J.N * rank / RANKS, J.N * (rank + 1) / RANKS,
+           [&](int i, T v) { st_peer(peer(B.phi + i, 0), v); });
+    cluster_sync();
+  }
   if (!CL || !rank) {
-    bottom(L[nl - 1], J.Mt, J.N);
+    if (!spread) bottom(B.rhs, J.Mt, J.N, 0, J.N, [&](int i, T v) { B.phi[i] = v; });
     __syncthreads();
     for (int k = nl - 2; k >= ns; --k) {
       if (k < nl - 2) M.init(L[k], per);

@@ -284,7 +284,7 @@ void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
   H.csmem = one.smem;
   H.cjob = std::move(one.job);
   H.coff = std::move(one.off);
-  if (one.lc > 0 && one.lc < nl) {
+  if (one.lc > 0) {
     // (from level 1 at the finest: the finest level of a solve keeps its half-sweeps)
     Coarse many = coarse_from(1, set ? limit : LLONG_MAX, true, !set);
     if (many.lc < nl && many.J.ranks > 1) {

@@ -12,7 +12,7 @@ F64, MIXED = mg.MG_PREC_F64, mg.MG_PREC_MIXED
 CASES = [((32, 32, 32), F64, 0), ((64, 16, 16), F64, 0), ((24, 32, 40), F64, 0), ((48, 48, 48), F64, 0),
          ((16, 16, 64), F64, 0), ((64, 64, 8), F64, 4096), ((32, 32, 32), F64, 4096), ((64, 64, 64), F64, 32768),
          ((32, 32, 32), MIXED, 0), ((64, 64, 64), MIXED, 0), ((64, 64, 64), MIXED, 32768), ((24, 40, 112), MIXED, 0),
-         ((32, 48, 72), MIXED, 40000)]
+         ((32, 48, 72), MIXED, 40000), ((48, 40, 56), F64, 0), ((24, 20, 28), F64, 2000), ((48, 40, 56), MIXED, 4000)]
 
 
 def _solve(ctx, n, per, prec, cells, nu):
