@@ -1480,14 +1480,21 @@ cudaError_t launch_dense_copy(int dt, const DRow* rows, int nbox, long long nrow
   return cudaGetLastError();
 }
 
-cudaError_t launch_copy_valid_f32(const DRow* rows, int nbox, long long nrows, cudaStream_t s, int width) {
+cudaError_t launch_copy_valid(int dt, const DRow* rows, int nbox, long long nrows, cudaStream_t s, int width) {
   if (nrows <= 0) return cudaSuccess;
   const int G = group_lanes(width, kCopyCells, 8, 32);
   const Grid g = row_grid(nrows, row_blocks_per_sm(width), kWarps * (32 / G));
   const SegList L = one_seg(rows, nbox, 0, width);
-  if (G == 32) launch_k(k_copy_valid<float, 32>, g.blocks, kThreads, 0, s, L, nrows, g.per);
-  else if (G == 16) launch_k(k_copy_valid<float, 16>, g.blocks, kThreads, 0, s, L, nrows, g.per);
-  else launch_k(k_copy_valid<float, 8>, g.blocks, kThreads, 0, s, L, nrows, g.per);
+  auto go = [&](auto k) { launch_k(k, g.blocks, kThreads, 0, s, L, nrows, g.per); };
+  if (dt == DT_F64) {
+    if (G == 32) go(k_copy_valid<double, 32>);
+    else if (G == 16) go(k_copy_valid<double, 16>);
+    else go(k_copy_valid<double, 8>);
+  } else {
+    if (G == 32) go(k_copy_valid<float, 32>);
+    else if (G == 16) go(k_copy_valid<float, 16>);
+    else go(k_copy_valid<float, 8>);
+  }
   count_launches(1);
   return cudaGetLastError();
 }

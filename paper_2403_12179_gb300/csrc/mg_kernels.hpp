@@ -345,7 +345,7 @@ cudaError_t launch_dense_copy(int dt, const DRow* rows, int nbox, long long nrow
                               const int dom_lo[3], const int dom_n[3], int ncomp, int to_dense,
                               cudaStream_t s, int width = 0);
 // v[0] = v[1] on valid cells (FP32).
-cudaError_t launch_copy_valid_f32(const DRow* rows, int nbox, long long nrows, cudaStream_t s, int width);
+cudaError_t launch_copy_valid(int dt, const DRow* rows, int nbox, long long nrows, cudaStream_t s, int width);
 
 // max |value| over valid cells, atomicMax of bit patterns into norms[solve]; v[0] = field.
 cudaError_t launch_maxabs(int dt, const DRow* rows, int nbox, long long nrows,

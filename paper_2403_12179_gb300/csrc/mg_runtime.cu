@@ -1248,7 +1248,7 @@ int mg_smooth(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double hh
       if (st.ok) {
         launch_fill(*c, *fr, bc, s);
         MG_CK(launch_sweep_f32_fabs((const SweepGrid*)st.grid->p, st.plan, fp->lay.g, s));
-        MG_CK(launch_copy_valid_f32(st.back.rows(), st.back.nbox, st.back.nrows, s, st.back.width));
+        MG_CK(launch_copy_valid(DT_F32, st.back.rows(), st.back.nbox, st.back.nrows, s, st.back.width));
         return MG_OK;
       }
     }

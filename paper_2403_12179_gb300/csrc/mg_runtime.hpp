@@ -345,6 +345,7 @@ struct SolveParams {
   int prolong = MG_PROLONG_CONSTANT;
   int inner = kDefaultInnerCycles;  // FP32 V-cycles per outer iteration (mixed form)
   double h = 0.0;
+  bool single = false;  // a solve on its own: its finest level may be staged (Hierarchy::staged)
 };
 SolveParams params_from(const mg_options* o, const BoxArray& ba);
 

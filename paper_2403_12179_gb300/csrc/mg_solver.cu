@@ -67,6 +67,14 @@ bool on_lattice(const BoxArray& ba) {
   return true;
 }
 
+// Whether a level of our own over these boxes is better one box: they are not of one size on a
+// lattice, so that stencils would need ghost fills (FP64 boxes wider than the marching kernels take stay
+// as they are).
+bool better_one_box(const BoxArray& ba, const SolveParams& p, int dt) {
+  return p.direct_reads && p.smoother != MG_SMOOTH_FUSED && !on_lattice(ba) &&
+         (dt == DT_F32 || ba.dom.len(0) <= kMarchMaxX);
+}
+
 }  // namespace
 
 namespace {
@@ -322,8 +330,9 @@ Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, cons
   std::lock_guard<std::recursive_mutex> lk(c.hier_mu);
   int per[3];
   int key = bc_code(bc, per);
+  const bool staged = p.single && p.precision == MG_PREC_F64 && better_one_box(phi.ba->ba, p, DT_F64);
   for (auto& h : c.hier) {
-    if (h->rhs_id == rhs.id && h->phi_id == phi.id && h->bc_key == key &&
+    if (h->rhs_id == rhs.id && h->phi_id == phi.id && h->bc_key == key && h->staged == staged &&
         h->p.nu1 == p.nu1 && h->p.nu2 == p.nu2 && h->p.precision == p.precision &&
         h->p.smoother == p.smoother && h->p.h == p.h &&
         h->p.coarse_cells == p.coarse_cells && h->p.direct_reads == p.direct_reads &&
@@ -349,6 +358,25 @@ Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, cons
   H->phi0 = c.get_fab(phi.id);
   H->rhs0 = c.get_fab(rhs.id);
   cudaStream_t s = c.stream;
+  if (staged) {
+    auto one = std::make_shared<BoxArrayObj>();
+    one->ba = phi.ba->ba;
+    one->ba.boxes.assign(1, one->ba.dom);
+    std::shared_ptr<FabObj> up = H->phi0, ur = H->rhs0;
+    H->staged = true;
+    H->phi0 = internal_fab(c, one, 1, DT_F64);
+    H->rhs0 = internal_fab(c, one, 0, DT_F64);
+    const BoxArray& ub = phi.ba->ba;
+    auto copies = [&](const FabObj& to, const FabObj& from) {
+      return make_table(c, ub, 0, p.h, 0, [&](int b, DRow& R) {
+        R.v[0] = view_of(to, ub.boxes[b]);
+        R.v[1] = view_of(from, ub.boxes[b]);
+      }, s);
+    };
+    H->stage_phi = copies(*H->phi0, *up);
+    H->stage_rhs = copies(*H->rhs0, *ur);
+    H->unstage_phi = copies(*up, *H->phi0);
+  }
   const int nl = (int)lev.size();
   H->L.resize(nl);
   double h = p.h;
@@ -357,7 +385,7 @@ Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, cons
     D.h = h;
     h *= 2.0;
     const bool internal = l > 0 || H->mixed;  // the level's fields are the hierarchy's own
-    if (!internal) D.bao = phi.ba;
+    if (!internal) D.bao = H->phi0->ba;
     else {
       D.bao = std::make_shared<BoxArrayObj>();
       D.bao->ba = lev[l];
@@ -365,8 +393,7 @@ Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, cons
       // of our own is one box, whose stencils need no ghost fills and take the whole sweeps (measured
       // on GB300: 96 x 80 x 112 in boxes of 48, FP64 3.24 -> 2.81 ms; 24 served problems, those of 48^3
       // and 96^3 in ragged boxes, 12.4 -> 9.0 ms)
-      if (p.direct_reads && p.smoother != MG_SMOOTH_FUSED && !on_lattice(lev[l]))
-        D.bao->ba.boxes.assign(1, lev[l].dom);
+      if (better_one_box(lev[l], p, H->dt)) D.bao->ba.boxes.assign(1, lev[l].dom);
     }
     // FP64 levels default to half-sweeps: on GB300 they are bound by the FP64 pipe, and the
     // fused sweep's redundant ring updates add FP64 work; large FP32 levels are bound by HBM
@@ -676,6 +703,18 @@ void destroy_hierarchies(Ctx& c) {
   c.hier.clear();
 }
 
+// The hierarchy of a solve on its own; not staged where there is no memory for that.
+static Hierarchy& single_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, SolveParams p) {
+  p.single = true;
+  try {
+    return get_hierarchy(c, rhs, phi, bc, p);
+  } catch (const MgError& e) {
+    if (e.code != MG_ENOMEM) throw;
+  }
+  p.single = false;
+  return get_hierarchy(c, rhs, phi, bc, p);
+}
+
 int solve(Ctx& c, int64_t rhs_id, int64_t phi_id, const mg_bc* bc, double tol,
           const SolveParams& p, mg_result* res) {
   c.require_device();
@@ -683,10 +722,17 @@ int solve(Ctx& c, int64_t rhs_id, int64_t phi_id, const mg_bc* bc, double tol,
   auto rhs = c.get_fab(rhs_id);
   auto phi = c.get_fab(phi_id);
   double t_start = c.now();
-  Hierarchy& H = get_hierarchy(c, *rhs, *phi, bc, p);
+  Hierarchy& H = single_hierarchy(c, *rhs, *phi, bc, p);
   cudaStream_t s = c.stream;
   if (!H.hnorm) MG_CK(cudaMallocHost(&H.hnorm, 16));
   unsigned long long* dn = (unsigned long long*)H.dnorm->p;
+  auto copy = [&](const OpTable& t) {
+    MG_CK(launch_copy_valid(DT_F64, t.rows(), t.nbox, t.nrows, s, t.width));
+  };
+  if (H.staged) {
+    copy(H.stage_phi);
+    copy(H.stage_rhs);
+  }
   // ||rhs||_inf and the first residual norm
   MG_CK(cudaMemsetAsync(dn, 0, 16, s));
   MG_CK(launch_maxabs(DT_F64, H.rhsabs0.rows(), H.rhsabs0.nbox, H.rhsabs0.nrows, dn, s, H.rhsabs0.width));
@@ -739,6 +785,11 @@ int solve(Ctx& c, int64_t rhs_id, int64_t phi_id, const mg_bc* bc, double tol,
       }
       ++it;
     }
+  }
+  if (H.staged) {  // phi back, with the ghost layer that the norm checks on its own boxes leave
+    copy(H.unstage_phi);
+    launch_fill(c, *phi, bc, s, 1);
+    MG_CK(cudaStreamSynchronize(s));
   }
   check_device_error(c);
   r.status = status;
