@@ -2,8 +2,10 @@
 // Gauss-Seidel half-sweeps, residual with fused max-norm, fused residual + restriction,
 // restriction, prolongation, bottom solve and the mixed-precision scale / correction.
 //
-// All stencil kernels are bounded by HBM bandwidth (about 1 flop per byte), so none of them
-// uses the tensor cores.  Each launch covers every box of its table (Sec. 3.2 kernel fusing).
+// The FP32 stencils are bound by HBM, the FP64 ones by the FP64 pipe, and none is a contraction, so
+// none uses the tensor cores.  Each launch covers every box of its table (Sec. 3.2 kernel fusing).
+// These forms take any layout; whole FP32 sweeps on lattices of boxes are in mg_sweep.cu, FP64 stencils on
+// boxes up to 256 wide in mg_march.cu.
 // Arithmetic goes through __{d,f}{add,mul,fma}_rn intrinsics in a fixed order, each one IEEE
 // round-to-nearest step, so results match the documented formulas bit for bit.  On GB300
 // FP64 instructions are scarce (the FP64 pipe issues far fewer lanes per clock than FP32), so

@@ -776,7 +776,9 @@ int solve(Ctx& c, int64_t rhs_id, int64_t phi_id, const mg_bc* bc, double tol,
       MG_CK(cudaStreamSynchronize(s));
       pending = (bool)H.save0;
       rn = bits_to_double(H.hnorm[0]);
-      if (H.graph_timed && H.lc > 0 && !H.L[0].fused) {
+      // (the events are recorded where the finest level's first pre-smoothing sweep is two half-sweeps)
+      if (H.graph_timed && H.lc > 0 && !H.L[0].fused && H.p.nu1 >= 1 &&
+          !(H.L[0].sweep_plan.tiles && H.p.nu1 >= 2)) {
         float ms = 0.f;
         if (cudaEventElapsedTime(&ms, H.sweep_ev[0], H.sweep_ev[1]) == cudaSuccess) {
           c.sweep_ms += ms;

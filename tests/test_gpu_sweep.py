@@ -100,3 +100,25 @@ def test_ragged_boxes_equal_even_ones(n, ragged, even, per, precision):
             np.testing.assert_array_equal(got[0].view(np.int64), g.view(np.int64))
     finally:
         mg.mg_finalize(ctx)
+
+
+@pytest.mark.parametrize("kw", [{"precision": mg.MG_PREC_MIXED}, {"precision": mg.MG_PREC_MIXED, "nu1": 1},
+                                {"nu1": 0}, {"nu1": 0, "use_graph": 0}, {}])
+def test_calls_after_a_timed_solve(kw):
+    """A solve whose finest level has no half-sweep to time (whole sweeps, no pre-smoothing) leaves no
+    error behind for the next call."""
+    ctx = mg.mg_init(0)
+    try:
+        ba = mg.mg_box_array_create(ctx, (0, 0, 0), (63, 63, 63), (32, 32, 32))
+        fr, fp = mg.mg_fab_alloc(ctx, ba, 1, 0), mg.mg_fab_alloc(ctx, ba, 1, 1)
+        mg.mg_fab_set_val(ctx, fr, 1.0)
+        mg.mg_fab_set_val(ctx, fp, 0.0)
+        bc = mg.make_bc((0, 0, 0))
+        mg.mg_sweep_timing(ctx, True)
+        res = mg.mg_solve(ctx, fr, fp, bc, 1e-8, mg.make_options(fixed_vcycles=2, **kw))
+        mg.mg_fill_boundary(ctx, fp, bc)
+        _, count = mg.mg_sweep_timing(ctx, False)
+        assert res.status == 0 and res.vcycles == 2
+        assert count == (0 if kw.get("nu1") == 0 or kw == {"precision": mg.MG_PREC_MIXED} else 2)
+    finally:
+        mg.mg_finalize(ctx)
