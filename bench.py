@@ -169,7 +169,7 @@ def whole_job_rate(world, steps, max_total_ms):
 
 # Source files whose contents define each profiled kernel (its launch configuration included).
 KERNEL_SOURCES = {
-    "rbgs_half_f64": ["mg_kernels.cu", "mg_kernels.hpp"],
+    "rbgs_half_f64": ["mg_march.cu", "mg_isum.hpp", "mg_isum_dev.cuh", "mg_kernels.hpp"],
     "rbgs_fused_f32": ["mg_fused.cu", "mg_kernels.hpp", "mg_runtime.cu"],
     "copy_tags_f64": ["mg_kernels.cu", "mg_kernels.hpp", "mg_runtime.cu"],
 }
@@ -496,17 +496,20 @@ def roofline(kt, wl_name, f64, fp64, in_solve_launches=0):
                           "dram_min_frac": round(12 * cells / kt["rbgs_half_f32"] / 1e9 / hbm, 4)},
     }
     extra["note"] = ("the FP64 kernels (half-sweep, residual) are bound by GB300's FP64 issue "
-                     "rate, measured by fp64_peak: at 100% of it a half-sweep moves about 42% of "
-                     "the HBM copy peak, so the 70%-of-HBM target applies to the FP32 kernels "
-                     "(rbgs_fused_f32, rbgs_half_f32) only")
+                     "rate, measured by fp64_peak, and by the integer units, on which half of the "
+                     "warps make the six-addend sums (and all the multiplications by 1/6), bit for "
+                     "bit: fp64_frac counts every FP64 operation of the algorithm against the FP64 "
+                     "rate alone, so it can exceed 1; at 100% of that rate a half-sweep moves about "
+                     "42% of the HBM copy peak")
     if f64:
         ach = half_ops / t / 1e9
         where = (f"average of {in_solve_launches} launches inside the timed solves (CUDA events "
                  "on the solve stream)" if in_solve_launches else "separate timing loop")
-        return {"kernel": "k_rbgs_half<double> (one colour, finest level, neighbour boxes read directly)",
+        return {"kernel": "k_half_march<plain> (FP64, one colour, finest level, neighbour boxes read directly)",
                 "bound": "alu", "measured": where,
                 "achieved": round(ach, 1), "peak": round(fp64_peak, 1),
-                "unit": "G FP64 lane-ops/s", "frac": round(ach / fp64_peak, 4),
+                "unit": "G FP64 lane-ops/s (of the algorithm; part of them run on the integer units)",
+                "frac": round(ach / fp64_peak, 4),
                 "peak_source": "measured: mg_calib_fp64 (independent DFMA chains on every SM, "
                                "CUDA events; see fp64_peak)",
                 "hbm": {"achieved_gbs": round(16 * cells / t / 1e9, 1), "peak": hbm,
@@ -516,7 +519,7 @@ def roofline(kt, wl_name, f64, fp64, in_solve_launches=0):
                 "traffic": roofline_traffic("rbgs_half_f64", wl_name), "kernels": extra}
     t = kt["rbgs_fused_f32"]
     ach = 12 * cells / t / 1e9
-    return {"kernel": "k_rbgs_fused<float> (full sweep, fine level)", "bound": "hbm",
+    return {"kernel": "k_rbgs_fused<float> (full sweep, fine level, mg_smooth_fused)", "bound": "hbm",
             "achieved": round(ach, 1), "peak": hbm, "unit": "GB/s", "frac": round(ach / hbm, 4),
             "peak_source": src, "algorithmic_bytes_per_launch": 12 * cells,
             "traffic": roofline_traffic("rbgs_fused_f32", wl_name), "kernels": extra}
