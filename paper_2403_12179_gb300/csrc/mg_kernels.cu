@@ -1268,7 +1268,8 @@ cudaError_t launch_prolong_trilinear_l(int dt, const SegList& L, long long nrows
 cudaError_t launch_prolong_add_l(int dt, const SegList& L, long long nrows, cudaStream_t s) {
   if (nrows <= 0) return cudaSuccess;
   const int G = group_lanes(L.width, dt == DT_F64 ? 2 : 4, 8, 32);  // cells per lane step
-  const Grid g = row_grid(nrows, row_blocks_per_sm(L.width), kWarps * (32 / G));
+  // FP64: the blocks that are resident (128^3 in boxes of 32^3: 12.7 us against 15.7 with four times as many)
+  const Grid g = row_grid(nrows, dt == DT_F64 ? 8 : row_blocks_per_sm(L.width), kWarps * (32 / G));
   if (dt == DT_F64) prolong_add_g<double>(G, g, s, L, nrows);
   else prolong_add_g<float>(G, g, s, L, nrows);
   count_launches(1);
@@ -1398,7 +1399,7 @@ cudaError_t launch_rbgs_half_store(const DRow* rows, int nbox, long long nrows, 
 cudaError_t launch_restrict(int dt, const DRow* rows, int nbox, long long nrows, cudaStream_t s, int width) {
   if (nrows <= 0) return cudaSuccess;
   const int G = group_lanes(width, 2, 8, 32);  // rows are coarse lines of width / 2 cells
-  const Grid g = row_grid(nrows, row_blocks_per_sm(width), kWarps * (32 / G));
+  const Grid g = row_grid(nrows, 8, kWarps * (32 / G));
   const SegList L = one_seg(rows, nbox, 0, width);
   auto go = [&](auto k) { launch_k(k, g.blocks, kThreads, 0, s, L, nrows, g.per); };
   if (dt == DT_F64) {
@@ -1437,7 +1438,8 @@ cudaError_t launch_bottom(int dt, const BottomJob* jobs, int njobs, int maxN, cu
 
 cudaError_t launch_add_valid(int dt, const DRow* rows, int nbox, long long nrows, cudaStream_t s) {
   if (nrows <= 0) return cudaSuccess;
-  Grid g = row_grid(nrows, 16);
+  // (8 resident blocks an SM: 128^3 in boxes of 32^3 13.3 us, 14.0 with 16)
+  Grid g = row_grid(nrows, 8);
   GB_DISPATCH(dt, k_add_valid, g.blocks, kThreads, 0, s, one_seg(rows, nbox), nrows, g.per);
   count_launches(1);
   return cudaGetLastError();
