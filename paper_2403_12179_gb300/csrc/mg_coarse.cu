@@ -340,7 +340,8 @@ __device__ void bottom(const T* rhs, const double* __restrict__ Mt, int N, int i
   }
 }
 // Cells from which the bottom solve's rows are spread over the CTAs of a cluster: one SM's FP64 pipe
-// takes 2 N^2 / 1.68 clocks (27 us for 210 cells).
+// takes 2 N^2 / 1.68 clocks (27 us for 210 cells).  Against stage launches and the bottom kernel: 88 x 88 x 56
+// (bottom of 847 cells) 2.10 -> 2.00 ms, 88 x 56 x 56 (539) 1.69 -> 1.55, 72 x 72 x 40 (405) 1.43 -> 1.32.
 constexpr int kBottomSpread = 64;
 
 // 512 threads for FP64 (128 registers each), 1024 for FP32.  RANKS: CTAs of a job, a cluster.
