@@ -148,8 +148,10 @@ struct JobB {
   std::vector<BottomJob> v;
   int maxN = 0;
   size_t off = 0;
+  bool shared = false;
   void add(const Hierarchy& H) {
     v.push_back(H.job_host);
+    shared = shared || H.job_shared;
     maxN = std::max(maxN, H.N);
   }
 };
@@ -394,7 +396,7 @@ void enqueue_step(Ctx& c, StepLists& S, const unsigned char* dev, unsigned long 
     }
     if (!S.bottom.v.empty())
       MG_CK(launch_bottom(S.dt, (const BottomJob*)(dev + S.bottom.off), (int)S.bottom.v.size(),
-                          S.bottom.maxN, s));
+                          S.bottom.maxN, s, S.bottom.shared));
     if (!S.coarse.v.empty())
       MG_CK(launch_coarse_cycle(S.dt, (const CoarseJob*)(dev + S.coarse.off), (int)S.coarse.v.size(),
                                 S.coarse.smem, s));

@@ -802,22 +802,24 @@ __global__ void k_set_flat(T* p, long long n, T value) {
     p[i] = value;
 }
 
-// Exact bottom solve: one warp-sized block per 32 rows of a job, rhs gathered to shared memory in
-// FP64.  The FP64 pipe of an SM bounds it (2 N operations a row at 1.68 lanes a clock: 210 rows in one
-// block took 39 us, 32 spread over SMs; ncu, cold), with 16 matrix loads ahead of the chain of
-// additions (64 ahead, 160 registers: 43 us).
-constexpr int kBottomRows = 32;
-template <class T>
-__global__ void __launch_bounds__(kBottomRows) k_bottom(const BottomJob* __restrict__ jobs, int chunks) {
+// Exact bottom solve: a block per ROWS rows of a job, rhs gathered to shared memory in FP64.  The FP64
+// pipe of an SM bounds it (2 N operations a row at 1.68 lanes a clock: 210 rows in one block took 39
+// us, 32 spread over SMs by warp-sized blocks; ncu, cold), with 16 matrix loads ahead of the chain of
+// additions (64 ahead, 160 registers: 43 us).  Where phi shares memory with rhs, one block takes a whole
+// job (ROWS 1024): no row is written before all of rhs has been gathered.
+constexpr int kBottomRows = 32, kBottomMaxRows = 1024;
+template <class T, int ROWS>
+__global__ void __launch_bounds__(ROWS) k_bottom(const BottomJob* __restrict__ jobs, int chunks) {
   pdl_begin();
   extern __shared__ double sb[];
   const BottomJob J = jobs[blockIdx.x / chunks];
-  const int i = (blockIdx.x % chunks) * kBottomRows + threadIdx.x;
+  const int i = (blockIdx.x % chunks) * ROWS + threadIdx.x;
   if (i - (int)threadIdx.x >= J.N) return;
   const T* rhs = (const T*)J.rhs;
   T* phi = (T*)J.phi;
-  for (int j = threadIdx.x; j < J.N; j += kBottomRows) sb[j] = (double)rhs[J.off_rhs[j]];
-  __syncwarp();
+  for (int j = threadIdx.x; j < J.N; j += ROWS) sb[j] = (double)rhs[J.off_rhs[j]];
+  if (ROWS > 32) __syncthreads();
+  else __syncwarp();
   if (i >= J.N) return;
   double s = 0.0;
 #pragma unroll 16
@@ -1425,13 +1427,21 @@ cudaError_t launch_prolong_trilinear(int dt, const DRow* rows, int nbox, long lo
   return launch_prolong_trilinear_l(dt, one_seg(rows, nbox, 0, width), nrows, s);
 }
 
-cudaError_t launch_bottom(int dt, const BottomJob* jobs, int njobs, int maxN, cudaStream_t s) {
+cudaError_t launch_bottom(int dt, const BottomJob* jobs, int njobs, int maxN, cudaStream_t s,
+                          bool shared) {
   if (njobs <= 0) return cudaSuccess;
-  const int chunks = (maxN + kBottomRows - 1) / kBottomRows;
-  const size_t smem = (size_t)maxN * sizeof(double);
-  const unsigned blocks = (unsigned)(njobs * chunks);
-  if (dt == DT_F64) launch_k(k_bottom<double>, blocks, kBottomRows, smem, s, jobs, chunks);
-  else launch_k(k_bottom<float>, blocks, kBottomRows, smem, s, jobs, chunks);
+  if (shared && maxN > kBottomMaxRows) return cudaErrorInvalidValue;
+  const int rows = shared ? kBottomMaxRows : kBottomRows, chunks = (maxN + rows - 1) / rows;
+  auto go = [&](auto k) {
+    launch_k(k, (unsigned)(njobs * chunks), rows, (size_t)maxN * sizeof(double), s, jobs, chunks);
+  };
+  if (dt == DT_F64) {
+    if (shared) go(k_bottom<double, kBottomMaxRows>);
+    else go(k_bottom<double, kBottomRows>);
+  } else {
+    if (shared) go(k_bottom<float, kBottomMaxRows>);
+    else go(k_bottom<float, kBottomRows>);
+  }
   count_launches(1);
   return cudaGetLastError();
 }

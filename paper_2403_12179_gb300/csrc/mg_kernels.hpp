@@ -318,7 +318,9 @@ cudaError_t launch_rbgs_fused(int dt, const DRow* rows, const int4* units, int n
                               int depth, int max_pitch, int max_pitch_r, bool rhs_smem, int* err,
                               cudaStream_t s);
 
-cudaError_t launch_bottom(int dt, const BottomJob* jobs, int njobs, int maxN, cudaStream_t s);
+// shared: some job's phi shares memory with its rhs.
+cudaError_t launch_bottom(int dt, const BottomJob* jobs, int njobs, int maxN, cudaStream_t s,
+                          bool shared = false);
 
 // Places of J's levels (extents set), in slabs over a cluster if `cluster` and where they are large
 // enough; sets ranks, nslab, planes and the offsets.  Returns the bytes of shared memory, or 0 if

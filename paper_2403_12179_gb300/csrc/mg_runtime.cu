@@ -1503,7 +1503,7 @@ int mg_bottom_solve(mg_ctx_t h, mg_fab_t rhs, mg_fab_t phi, const mg_bc* bc, dou
     J.phi = fp->base;
     J.N = (int)N;
     DevBufP dj = c->upload(&J, sizeof J, s);
-    MG_CK(launch_bottom(fp->dtype, (const BottomJob*)dj->p, 1, (int)N, s));
+    MG_CK(launch_bottom(fp->dtype, (const BottomJob*)dj->p, 1, (int)N, s, fp->shares_memory(*fr)));
     dj->reset(s);
     dp->reset(s);
     dr->reset(s);

@@ -128,6 +128,10 @@ struct FabObj {
   }
   DView view(int b) const;
   int esize() const { return dtype == DT_F64 ? 8 : 4; }
+  // whether the two fabs' storage shares bytes (one fab, or wrapped memory)
+  bool shares_memory(const FabObj& o) const {
+    return (const char*)base < (const char*)o.base + o.bytes && (const char*)o.base < (const char*)base + bytes;
+  }
 };
 
 // Face reads of the stencil kernels (DRow::nbd / nbf) for the boxes of fab f under the given

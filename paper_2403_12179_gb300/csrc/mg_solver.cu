@@ -222,6 +222,7 @@ void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
   J.N = (int)N;
   H.job = c.upload(&J, sizeof J, s);
   H.job_host = J;
+  H.job_shared = B.phi->shares_memory(*B.rhs);
   // The coarse end of the cycle as one launch: from the first level with at most `limit` cells whose
   // levels (down to the bottom) fit into shared memory.  (The coarse-cycle kernel prolongs by
   // injection: the trilinear form runs level by level.)
@@ -567,7 +568,7 @@ void enqueue_vcycle(Ctx& c, Hierarchy& H, cudaStream_t s, unsigned long long* no
     MG_CK(launch_coarse_cycle(H.dt, (const CoarseJob*)H.scjob->p, 1, H.scsmem, s, H.sranks));
   else if (H.slc < nl)
     MG_CK(launch_coarse_cycle(H.dt, (const CoarseJob*)H.cjob->p, 1, H.csmem, s));
-  else MG_CK(launch_bottom(H.dt, (const BottomJob*)H.job->p, 1, H.N, s));
+  else MG_CK(launch_bottom(H.dt, (const BottomJob*)H.job->p, 1, H.N, s, H.job_shared));
   for (int l = top - 1; l >= 0; --l) {
     LevelData& D = H.L[l];
     if (H.p.prolong == MG_PROLONG_TRILINEAR) {

@@ -68,6 +68,7 @@ struct Hierarchy {
   DevBufP dnorm;  // [0] residual norm bits, [1] rhs norm bits
   unsigned long long* hnorm = nullptr;
   BottomJob job_host{};
+  bool job_shared = false;  // (a bottom level of the caller's fabs that share memory)
   // FP64 solves whose finest level starts each V-cycle with a red half-sweep: that
   // half-sweep of the next cycle also takes the red cells' residual norm of the current
   // iterate (it computes the same neighbour sums), replacing a separate residual pass; it
