@@ -179,16 +179,21 @@ static void split_dim(int a, int b, int dlo, int dhi, bool periodic, std::vector
   if (b > dhi) out->push_back({std::max(a, dhi + 1), b, +1, 0});
 }
 
-bool make_copy_tags(const BoxArray& ba, const int periodic[3], int g, std::vector<CopyTag>* tags,
-                    std::string* err) {
-  tags->clear();
+bool fillable(const BoxArray& ba, const int periodic[3], int g, std::string* err) {
   if (g < 0) { *err = "negative ghost width"; return false; }
-  if (g == 0) return true;
   for (int d = 0; d < 3; ++d)
     if (!periodic[d] && g > ba.dom.len(d)) {
       *err = "ghost width exceeds a Dirichlet domain extent";
       return false;
     }
+  return true;
+}
+
+bool make_copy_tags(const BoxArray& ba, const int periodic[3], int g, std::vector<CopyTag>* tags,
+                    std::string* err) {
+  tags->clear();
+  if (!fillable(ba, periodic, g, err)) return false;
+  if (g == 0) return true;
   const Box& D = ba.dom;
   std::vector<Piece> pcs[3];
   for (size_t bi = 0; bi < ba.boxes.size(); ++bi) {

@@ -59,6 +59,9 @@ struct CopyTag {
   int sign;
 };
 
+// Whether g ghost layers can be filled: none is wider than a Dirichlet dimension of the domain.
+bool fillable(const BoxArray& ba, const int periodic[3], int g, std::string* err);
+
 // Tags filling every ghost cell (grow(box, g) minus box) of every box: periodic images and
 // other boxes by box intersection; -(mirror) across a single Dirichlet face; 0 when the
 // ghost is outside the domain in two or more non-periodic dimensions.

@@ -1231,6 +1231,12 @@ int mg_smooth(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double hh
       }
     }
     if (color < 0 || color > 2) fail(MG_EINVAL, "color must be 0, 1 or 2 (0 / 1 may add MG_SMOOTH_DIRECT_READS)");
+    if (color == 2) {  // phi's ghosts, filled or read past: refused before anything is launched
+      int per[3];
+      bc_code(bc, per);
+      std::string err;
+      if (!fillable(fp->ba->ba, per, fp->lay.g, &err)) fail(MG_EINVAL, err);
+    }
     cudaStream_t s = S(stream);
     double hv = default_h(*fp, hh);
     const OpTable& t = op_table(*c, "smooth", {phi, rhs}, hv, [&] {
