@@ -380,6 +380,22 @@ Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, cons
   }
   const int nl = (int)lev.size();
   H->L.resize(nl);
+  if (H->mixed) H->r0 = internal_fab(c, phi.ba, 0, DT_F64);
+  // The second phi of the whole sweeps lies in r0: within an outer iteration r0 is read by the scaling,
+  // before the first sweep, and written by the norm check, after the last.  (Levels of its own took 4 bytes
+  // a cell more: 128^3 in boxes of 32^3 46.5 MB, 36.9 MB now.)
+  size_t lent = 0;  // bytes of r0
+  auto second_phi = [&](const LevelData& D) {
+    if (!D.wide || lent + D.phi->bytes > H->r0->bytes) return internal_fab(c, D.bao, D.phi->lay.g, H->dt);
+    auto f = std::make_shared<FabObj>();
+    f->ba = D.bao;
+    f->dtype = H->dt;
+    f->lay = D.phi->lay;
+    f->bytes = D.phi->bytes;
+    f->base = (char*)H->r0->base + lent;
+    lent += f->bytes;
+    return f;
+  };
   double h = p.h;
   for (int l = 0; l < nl; ++l) {
     LevelData& D = H->L[l];
@@ -422,9 +438,8 @@ Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, cons
       D.phi = internal_fab(c, D.bao, D.wide ? 0 : D.fused ? 2 : 1, H->dt);
       D.rhs = internal_fab(c, D.bao, D.fused ? 1 : 0, H->dt);
     }
-    if (D.fused || D.wide) D.phi2 = internal_fab(c, D.bao, D.phi->lay.g, H->dt);
+    if (D.fused || D.wide) D.phi2 = second_phi(D);
   }
-  if (H->mixed) H->r0 = internal_fab(c, phi.ba, 0, DT_F64);
   build_tables(c, *H, s);
   {
     // speculative red half-sweep with the norm check (see Hierarchy::save0): FP64, the

@@ -50,7 +50,8 @@ struct Hierarchy {
   // copies and the last fill take 25 us).
   bool staged = false;
   OpTable stage_phi, stage_rhs, unstage_phi;
-  std::shared_ptr<FabObj> r0;          // mixed: FP64 residual stored by each norm check
+  std::shared_ptr<FabObj> r0;          // mixed: FP64 residual stored by each norm check (between the
+                                       // scaling and that check, the second phi of the whole sweeps)
   bool direct0 = false;                // the norm check reads neighbouring boxes directly
   OpTable resid0, rhsabs0, scale0, correct0, zero0_64;
   DevBufP Mt, offr, offp, job;
