@@ -417,6 +417,7 @@ AmrPlan& get_plan(Ctx& c, int64_t rhs0, int64_t phi0, int64_t rhs1, int64_t phi1
   fill_plan(c, *f1, &P->fine_bc, 1);
   fill_plan(c, *f0, bc, 1);
   P->dnorm = c.alloc(16, s);
+  prepare_alone(c, *P->H);
   MG_CK(cudaMallocHost(&P->hnorm, 16));
   MG_CK(cudaStreamSynchronize(s));
   g_plans[&c].push_back(P);

@@ -88,8 +88,8 @@ struct CoarseLevel {
   double h2, ih2;
 };
 struct CoarseJob {
-  const long long* off_phi;
-  const long long* off_rhs;
+  const int* off_phi;
+  const int* off_rhs;
   void* phi;
   const void* rhs;
   const double* Mt;  // bottom (pseudo-)inverse, transposed, over the last level's cells

@@ -102,6 +102,75 @@ bool coarse_field(const FabObj& f, CoarseField* out) {
 // 2^25 and fusing every level.
 constexpr long long kFusedMinCells = 1ll << 24;
 
+// The coarse end of the cycle as one launch: from the first level with at most `limit` cells whose
+// levels (down to the bottom) fit into shared memory; lc == levels: none.  (The coarse-cycle kernel
+// prolongs by injection: the trilinear form runs level by level.)
+struct Coarse {
+  int lc;
+  CoarseJob J;
+  DevBufP job, off;
+  size_t smem;
+};
+Coarse coarse_from(Ctx& c, Hierarchy& H, int first, long long limit, bool cluster, bool bounded, cudaStream_t s) {
+  const int nl = (int)H.L.size();
+  const bool one_launch = H.p.coarse_cells >= 0 && H.p.prolong == MG_PROLONG_CONSTANT;
+  int per[3];
+  bc_code(&H.bc, per);
+  Coarse R{nl, {}, nullptr, nullptr, 0};
+  for (int l = std::max(first, nl - kMaxCoarseLevels); one_launch && l + 1 < nl; ++l) {
+    const LevelData& T = H.L[l];
+    const BoxArray& tb = T.bao->ba;
+    if (tb.dom.npts() > limit || T.phi->lay.total > INT_MAX || T.rhs->lay.total > INT_MAX) continue;
+    CoarseJob& C = R.J;
+    C = CoarseJob{};
+    C.nlev = nl - l;
+    for (int k = 0; k < C.nlev; ++k) {
+      const LevelData& D = H.L[l + k];
+      CoarseLevel& V = C.lev[k];
+      for (int d = 0; d < 3; ++d) {
+        V.n[d] = D.bao->ba.dom.len(d);
+        V.lo[d] = D.bao->ba.dom.lo[d];
+      }
+      V.h2 = D.h * D.h;
+      V.ih2 = 1.0 / (D.h * D.h);
+    }
+    R.smem = coarse_layout(H.dt, C, cluster, bounded);
+    if (!R.smem || R.smem > kCoarseSmemMax) continue;
+    // level l's cells, dense and x fastest, in its phi and rhs fabs
+    const long long nt = tb.dom.npts();
+    std::vector<int> offs(2 * nt);
+    for (size_t b = 0; b < tb.boxes.size(); ++b) {
+      const Box& X = tb.boxes[b];
+      for (int z = X.lo[2]; z <= X.hi[2]; ++z)
+        for (int y = X.lo[1]; y <= X.hi[1]; ++y)
+          for (int x = X.lo[0]; x <= X.hi[0]; ++x) {
+            long long i = ((long long)(z - tb.dom.lo[2]) * C.lev[0].n[1] + (y - tb.dom.lo[1])) *
+                              C.lev[0].n[0] + (x - tb.dom.lo[0]);
+            offs[i] = (int)T.phi->lay.at(tb, (int)b, x, y, z);
+            offs[nt + i] = (int)T.rhs->lay.at(tb, (int)b, x, y, z);
+          }
+    }
+    R.off = c.upload(offs.data(), offs.size() * sizeof(int), s);
+    C.off_phi = (const int*)R.off->p;
+    C.off_rhs = C.off_phi + nt;
+    C.phi = T.phi->base;
+    C.rhs = T.rhs->base;
+    C.Mt = (const double*)H.Mt->p;
+    C.N = H.N;
+    C.nu1 = H.p.nu1;
+    C.nu2 = H.p.nu2;
+    for (int d = 0; d < 3; ++d) C.periodic[d] = per[d];
+    MG_CK(coarse_opt_in(H.dt, R.smem, C.ranks));
+    R.job = c.upload(&C, sizeof C, s);
+    R.lc = l;
+    break;
+  }
+  return R;
+}
+int coarse_limit(const Hierarchy& H) {
+  return H.p.coarse_cells != 0 ? H.p.coarse_cells : (H.dt == DT_F64 ? 512 : 4096);
+}
+
 void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
   const int nl = (int)H.L.size();
   int per[3];
@@ -124,18 +193,10 @@ void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
       D.sweep_ab.src = (const float*)D.phi->base;
       D.sweep_ab.rhs = (const float*)D.rhs->base;
       D.sweep_ab.dst = (float*)D.phi2->base;
-      const bool coarse = coarse_field(*H.L[l + 1].phi, &D.sweep_ab.coarse);
+      coarse_field(*H.L[l + 1].phi, &D.sweep_ab.coarse);
       D.sweep_ba = D.sweep_ab;
       D.sweep_ba.src = (const float*)D.phi2->base;
       D.sweep_ba.dst = (float*)D.phi->base;
-      if (D.cells() >= kSweepMinCells) {
-        std::vector<SweepGrid> ab{D.sweep_ab}, ba{D.sweep_ba};
-        D.sweep_plan = plan_sweep(ab, ba);
-        D.zero_start = H.p.nu1 >= 2;
-        D.add_start = H.p.nu2 >= 2 && coarse;
-        ab.push_back(ba[0]);
-        D.sweep_dev = c.upload(ab.data(), ab.size() * sizeof(SweepGrid), s);
-      }
     }
     if (D.fused) {
       D.f_ab = make_fused(c, ba, D.h, *D.phi, *D.rhs, *D.phi2, per, s);
@@ -223,79 +284,49 @@ void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
   H.job = c.upload(&J, sizeof J, s);
   H.job_host = J;
   H.job_shared = B.phi->shares_memory(*B.rhs);
-  // The coarse end of the cycle as one launch: from the first level with at most `limit` cells whose
-  // levels (down to the bottom) fit into shared memory.  (The coarse-cycle kernel prolongs by
-  // injection: the trilinear form runs level by level.)
-  const bool one_launch = H.p.coarse_cells >= 0 && H.p.prolong == MG_PROLONG_CONSTANT;
-  struct Coarse {
-    int lc;
-    CoarseJob J;
-    DevBufP job, off;
-    size_t smem;
-  };
-  auto coarse_from = [&](int first, long long limit, bool cluster, bool bounded) {
-    Coarse R{nl, {}, nullptr, nullptr, 0};
-    for (int l = std::max(first, nl - kMaxCoarseLevels); one_launch && l + 1 < nl; ++l) {
-      if (H.L[l].bao->ba.dom.npts() > limit) continue;
-      CoarseJob& C = R.J;
-      C = CoarseJob{};
-      C.nlev = nl - l;
-      for (int k = 0; k < C.nlev; ++k) {
-        const LevelData& D = H.L[l + k];
-        CoarseLevel& V = C.lev[k];
-        for (int d = 0; d < 3; ++d) {
-          V.n[d] = D.bao->ba.dom.len(d);
-          V.lo[d] = D.bao->ba.dom.lo[d];
-        }
-        V.h2 = D.h * D.h;
-        V.ih2 = 1.0 / (D.h * D.h);
-      }
-      R.smem = coarse_layout(H.dt, C, cluster, bounded);
-      if (!R.smem || R.smem > kCoarseSmemMax) continue;
-      // level l's cells, dense and x fastest, in its phi and rhs fabs
-      const LevelData& T = H.L[l];
-      const BoxArray& tb = T.bao->ba;
-      const long long nt = tb.dom.npts();
-      std::vector<long long> offs(2 * nt);
-      for (size_t b = 0; b < tb.boxes.size(); ++b) {
-        const Box& X = tb.boxes[b];
-        for (int z = X.lo[2]; z <= X.hi[2]; ++z)
-          for (int y = X.lo[1]; y <= X.hi[1]; ++y)
-            for (int x = X.lo[0]; x <= X.hi[0]; ++x) {
-              long long i = ((long long)(z - tb.dom.lo[2]) * C.lev[0].n[1] + (y - tb.dom.lo[1])) *
-                                C.lev[0].n[0] + (x - tb.dom.lo[0]);
-              offs[i] = T.phi->lay.at(tb, (int)b, x, y, z);
-              offs[nt + i] = T.rhs->lay.at(tb, (int)b, x, y, z);
-            }
-      }
-      R.off = c.upload(offs.data(), offs.size() * 8, s);
-      C.off_phi = (const long long*)R.off->p;
-      C.off_rhs = C.off_phi + nt;
-      C.phi = T.phi->base;
-      C.rhs = T.rhs->base;
-      C.Mt = J.Mt;
-      C.N = J.N;
-      C.nu1 = H.p.nu1;
-      C.nu2 = H.p.nu2;
-      for (int d = 0; d < 3; ++d) C.periodic[d] = per[d];
-      MG_CK(coarse_opt_in(H.dt, R.smem, C.ranks));
-      R.job = c.upload(&C, sizeof C, s);
-      R.lc = l;
-      break;
-    }
-    return R;
-  };
-  const bool set = H.p.coarse_cells != 0;
-  const int limit = set ? H.p.coarse_cells : (H.dt == DT_F64 ? 512 : 4096);
-  Coarse one = coarse_from(0, limit, false, false);
+  Coarse one = coarse_from(c, H, 0, coarse_limit(H), false, false, s);
   H.lc = H.slc = one.lc;
   H.cjob_host = one.J;
   H.csmem = one.smem;
   H.cjob = std::move(one.job);
   H.coff = std::move(one.off);
-  if (one.lc > 0) {
-    // (from level 1 at the finest: the finest level of a solve keeps its half-sweeps)
-    Coarse many = coarse_from(1, set ? limit : LLONG_MAX, true, !set);
+  // fill plans must exist before any graph capture
+  for (auto& D : H.L) {
+    fill_plan(c, *D.phi, &H.bc, 1);
+    if (D.fused) {
+      fill_plan(c, *D.phi, &H.bc, 2);
+      fill_plan(c, *D.phi2, &H.bc, 2);
+      fill_plan(c, *D.rhs, &H.bc, 1);
+    }
+  }
+  fill_plan(c, *H.phi0, &H.bc, 1);
+}
+
+}  // namespace
+
+void prepare_alone(Ctx& c, Hierarchy& H) {
+  if (H.alone) return;
+  cudaStream_t s = c.stream;
+  const int nl = (int)H.L.size();
+  for (LevelData& D : H.L) {
+    if (!D.wide || D.cells() < kSweepMinCells) continue;
+    std::vector<SweepGrid> ab{D.sweep_ab}, ba{D.sweep_ba};
+    D.sweep_plan = plan_sweep(ab, ba);
+    D.zero_start = H.p.nu1 >= 2;
+    D.add_start = H.p.nu2 >= 2 && D.sweep_ab.coarse.base;
+    ab.push_back(ba[0]);
+    D.sweep_dev = c.upload(ab.data(), ab.size() * sizeof(SweepGrid), s);
+  }
+  if (H.lc > 0) {
+    // (from level 1 at the finest: the finest level of a solve keeps its half-sweeps; where there is no
+    // memory for its tables, the one CTA's stay)
+    const bool set = H.p.coarse_cells != 0;
+    Coarse many{nl, {}, nullptr, nullptr, 0};
+    try {
+      many = coarse_from(c, H, 1, set ? coarse_limit(H) : LLONG_MAX, true, !set, s);
+    } catch (const MgError& e) {
+      if (e.code != MG_ENOMEM) throw;
+    }
     if (many.lc < nl && many.J.ranks > 1) {
       H.slc = many.lc;
       H.sranks = many.J.ranks;
@@ -313,19 +344,9 @@ void build_tables(Ctx& c, Hierarchy& H, cudaStream_t s) {
     D.rr_plan = plan_restrict(q);
     D.rr_dev = c.upload(q.data(), sizeof(RestrictGrid), s);
   }
-  // fill plans must exist before any graph capture
-  for (auto& D : H.L) {
-    fill_plan(c, *D.phi, &H.bc, 1);
-    if (D.fused) {
-      fill_plan(c, *D.phi, &H.bc, 2);
-      fill_plan(c, *D.phi2, &H.bc, 2);
-      fill_plan(c, *D.rhs, &H.bc, 1);
-    }
-  }
-  fill_plan(c, *H.phi0, &H.bc, 1);
+  MG_CK(cudaStreamSynchronize(s));
+  H.alone = true;
 }
-
-}  // namespace
 
 Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, const SolveParams& p) {
   std::lock_guard<std::recursive_mutex> lk(c.hier_mu);
@@ -739,6 +760,7 @@ int solve(Ctx& c, int64_t rhs_id, int64_t phi_id, const mg_bc* bc, double tol,
   auto phi = c.get_fab(phi_id);
   double t_start = c.now();
   Hierarchy& H = single_hierarchy(c, *rhs, *phi, bc, p);
+  prepare_alone(c, H);
   cudaStream_t s = c.stream;
   if (!H.hnorm) MG_CK(cudaMallocHost(&H.hnorm, 16));
   unsigned long long* dn = (unsigned long long*)H.dnorm->p;

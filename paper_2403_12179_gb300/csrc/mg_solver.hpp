@@ -62,10 +62,11 @@ struct Hierarchy {
   DevBufP cjob, coff;
   CoarseJob cjob_host{};
   // the same of a solve on its own, by a cluster of CTAs, from a finer level (slc <= lc; a batch, whose
-  // jobs fill the SMs, takes one CTA a job)
+  // jobs fill the SMs, takes one CTA a job; prepare_alone)
   int slc = 0, sranks = 1;
   size_t scsmem = 0;
   DevBufP scjob, scoff;
+  bool alone = false;  // prepare_alone has run
   DevBufP dnorm;  // [0] residual norm bits, [1] rhs norm bits
   unsigned long long* hnorm = nullptr;
   BottomJob job_host{};
@@ -102,6 +103,11 @@ struct Hierarchy {
 
 // Cached per (rhs fab, phi fab, bc, options); builds coarse levels, tables and plans.
 Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, const SolveParams& p);
+// The tables that only a solve on its own launches from (whole sweeps, residual + restriction and coarse
+// cycle of one hierarchy), once per hierarchy, before its cycles are enqueued or captured: members of
+// batches go without (64^3 FP64 members: 74 KB each of 2.9 MB, and 0.4 of 4.1 ms for the first batch of
+// sixteen 32^3 mixed problems).
+void prepare_alone(Ctx& c, Hierarchy& H);
 
 // One V-cycle for the hierarchy's problem from a zero guess: phi (the caller's level-0 fab,
 // ghosts included) is zeroed, then the cycle is enqueued on s; no norm is taken.

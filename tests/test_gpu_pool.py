@@ -2,6 +2,7 @@
 import pytest
 
 from paper_2403_12179_gb300 import mg
+from tests import gpu_util as gu
 
 pytestmark = pytest.mark.gpu
 
@@ -34,3 +35,30 @@ def test_mixed_levels_take_phi_rhs_and_the_residual(n, box, batch):
     cells = n[0] * n[1] * n[2]
     tables = 0.5e6 if batch > 1 else 1e6
     assert _kept(n, box, batch, precision=mg.MG_PREC_MIXED) <= batch * (cells * (8 + 8 * 8 / 7) + tables)
+
+
+@pytest.mark.parametrize("n,box", [((64, 64, 64), (32, 32, 32)), ((32, 32, 32), (32, 32, 32))])
+@pytest.mark.parametrize("precision", [mg.MG_PREC_F64, mg.MG_PREC_MIXED])
+def test_solve_fits_where_a_batch_of_one_fits(n, box, precision):
+    """The tables that only a solve on its own launches from are not kept for members of a batch, and a
+    solve goes without the cluster's (at least 4096 cells of 8 bytes here) where the pool has no room:
+    the same bits.  (16 KB are left for its other tables, some hundred bytes a level.)"""
+    def run(pool, batch):
+        ctx = mg.mg_init(0, pool)
+        try:
+            ba = mg.mg_box_array_create(ctx, (0, 0, 0), tuple(v - 1 for v in n), box)
+            r, u = mg.mg_fab_alloc(ctx, ba, 1, 0), mg.mg_fab_alloc(ctx, ba, 1, 1)
+            mg.mg_fab_set_val(ctx, r, 1.0)
+            bc, opt = mg.make_bc((0, 0, 0)), mg.make_options(fixed_vcycles=3, precision=precision)
+            if batch:
+                res = mg.mg_solve_batch(ctx, [r], [u], [bc], 1e-10, opt)[0]
+            else:
+                res = mg.mg_solve(ctx, r, u, bc, 1e-10, opt)
+            return mg.mg_pool_info(ctx)[1], res.rel_resid, gu.fab_dense(ctx, u, n[::-1]).tobytes()
+        finally:
+            mg.mg_finalize(ctx)
+
+    alone, in_batch = run(0, False), run(0, True)
+    assert alone[0] >= in_batch[0] + 4096 * 8
+    tight = run(in_batch[0] + (16 << 10), False)
+    assert tight[1:] == alone[1:] == in_batch[1:]
