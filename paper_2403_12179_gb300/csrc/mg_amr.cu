@@ -268,12 +268,7 @@ AmrPlan& get_plan(Ctx& c, int64_t rhs0, int64_t phi0, int64_t rhs1, int64_t phi1
   SolveParams pc = p;
   pc.h = P->h0;
   pc.precision = MG_PREC_F64;
-  {
-    std::lock_guard<std::recursive_mutex> hl(c.hier_mu);
-    Hierarchy& H = get_hierarchy(c, *r0, *e0, bc, pc);
-    for (auto& h : c.hier)
-      if (h.get() == &H) P->H = h;
-  }
+  P->H = get_hierarchy(c, *r0, *e0, bc, pc);
   // coarse/fine ghost list
   Owner of{f1.get()}, oc{f0.get()};
   std::vector<CFGhost> cf;

@@ -511,11 +511,7 @@ int solve_batch(Ctx& c, int n, const int64_t* rhs, const int64_t* phi, const mg_
       if (phi[j] == phi[i]) fail(MG_EINVAL, "a phi fab appears twice in the batch");
     SolveParams pi = p;  // the default cell size belongs to each solve's own domain
     if (!(pi.h > 0)) pi.h = 1.0 / fp->ba->ba.dom.len(0);
-    std::lock_guard<std::recursive_mutex> hl(c.hier_mu);
-    Hierarchy& H = get_hierarchy(c, *fr, *fp, &bcs[i], pi);
-    for (auto& h : c.hier)
-      if (h.get() == &H) M[i].H = h;
-    if (!M[i].H) fail(MG_EINVAL, "internal: hierarchy not found");
+    M[i].H = get_hierarchy(c, *fr, *fp, &bcs[i], pi);
     M[i].slot = 2 * i;
     M[i].tol = tol;
     M[i].res.t_start = t0;
@@ -709,7 +705,6 @@ void server_loop(Ctx* c) {
                 m->own_phi = add_pool_fab(*c, r.hba, m->own_ba, 1, 2, DT_F64, s);
                 auto fr = c->get_fab(m->own_rhs);
                 auto fp = c->get_fab(m->own_phi);
-                std::lock_guard<std::recursive_mutex> hl(c->hier_mu);
                 get_hierarchy(*c, *fr, *fp, &r.bc, r.p);
                 break;
               } catch (const MgError& e) {
@@ -729,10 +724,7 @@ void server_loop(Ctx* c) {
         }
         auto fr = c->get_fab(rid);
         auto fp = c->get_fab(pid);
-        std::lock_guard<std::recursive_mutex> hl(c->hier_mu);
-        Hierarchy& H = get_hierarchy(*c, *fr, *fp, &r.bc, r.p);
-        for (auto& h : c->hier)
-          if (h.get() == &H) m->H = h;
+        m->H = get_hierarchy(*c, *fr, *fp, &r.bc, r.p);
       } catch (const MgError& e) {
         cudaStreamSynchronize(cs);  // a copy in may have started
         release_own(*c, *m, s);

@@ -47,10 +47,15 @@ void DevBuf::reset(cudaStream_t s) {
   bytes = 0;
 }
 
+static thread_local int g_spare = 0;
+SpareMemory::SpareMemory() { ++g_spare; }
+SpareMemory::~SpareMemory() { --g_spare; }
+
 DevBufP Ctx::alloc(size_t n, cudaStream_t s) {
   require_device();
   if (n == 0) n = 16;
   n = (n + 255) / 256 * 256;
+  if (in_use.load() + n > pool_cap && g_spare == 0) give_back(*this);
   size_t cur = in_use.load();
   if (cur + n > pool_cap) {
     std::ostringstream o;
@@ -60,6 +65,11 @@ DevBufP Ctx::alloc(size_t n, cudaStream_t s) {
   }
   void* p = nullptr;
   cudaError_t e = cudaMallocFromPoolAsync(&p, n, pool, s);
+  if (e == cudaErrorMemoryAllocation && g_spare == 0) {
+    cudaGetLastError();
+    give_back(*this);
+    e = cudaMallocFromPoolAsync(&p, n, pool, s);
+  }
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
     fail(MG_ENOMEM, "device out of memory");

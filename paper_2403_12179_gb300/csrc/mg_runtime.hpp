@@ -358,6 +358,16 @@ int solve(Ctx& c, int64_t rhs, int64_t phi, const mg_bc* bc, double tol, const S
 int solve_batch(Ctx& c, int n, const int64_t* rhs, const int64_t* phi, const mg_bc* bcs,
                 double tol, const SolveParams& p, mg_result* res);
 void drop_hierarchies_of(Ctx& c, int64_t fab_id);
+// Releases the cached hierarchies of solves not running now that hold more of the pool than they need (a
+// box of their own for phi and rhs, the cluster's tables); their next solve builds them anew.
+void give_back(Ctx& c);
+// While one lives, allocations of this thread are for memory that its work can do without: they fail
+// rather than have others give theirs back.
+struct SpareMemory {
+  SpareMemory();
+  ~SpareMemory();
+  SpareMemory(const SpareMemory&) = delete;
+};
 void destroy_hierarchies(Ctx& c);
 
 // Serving

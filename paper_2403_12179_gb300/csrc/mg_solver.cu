@@ -323,6 +323,7 @@ void prepare_alone(Ctx& c, Hierarchy& H) {
     const bool set = H.p.coarse_cells != 0;
     Coarse many{nl, {}, nullptr, nullptr, 0};
     try {
+      SpareMemory spare;
       many = coarse_from(c, H, 1, set ? coarse_limit(H) : LLONG_MAX, true, !set, s);
     } catch (const MgError& e) {
       if (e.code != MG_ENOMEM) throw;
@@ -348,19 +349,31 @@ void prepare_alone(Ctx& c, Hierarchy& H) {
   H.alone = true;
 }
 
-Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, const SolveParams& p) {
+static bool wants_staging(const FabObj& phi, const SolveParams& p) {
+  return p.single && p.precision == MG_PREC_F64 && better_one_box(phi.ba->ba, p, DT_F64);
+}
+
+// The cached hierarchy, or null.
+static std::shared_ptr<Hierarchy> find_hierarchy(Ctx& c, const FabObj& rhs, const FabObj& phi, int key, bool staged,
+                                                 const SolveParams& p) {
   std::lock_guard<std::recursive_mutex> lk(c.hier_mu);
-  int per[3];
-  int key = bc_code(bc, per);
-  const bool staged = p.single && p.precision == MG_PREC_F64 && better_one_box(phi.ba->ba, p, DT_F64);
   for (auto& h : c.hier) {
     if (h->rhs_id == rhs.id && h->phi_id == phi.id && h->bc_key == key && h->staged == staged &&
         h->p.nu1 == p.nu1 && h->p.nu2 == p.nu2 && h->p.precision == p.precision &&
         h->p.smoother == p.smoother && h->p.h == p.h &&
         h->p.coarse_cells == p.coarse_cells && h->p.direct_reads == p.direct_reads &&
         h->p.prolong == p.prolong && h->p.inner == p.inner)
-      return *h;
+      return h;
   }
+  return nullptr;
+}
+
+std::shared_ptr<Hierarchy> get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, const SolveParams& p) {
+  std::lock_guard<std::recursive_mutex> lk(c.hier_mu);
+  int per[3];
+  int key = bc_code(bc, per);
+  const bool staged = wants_staging(phi, p);
+  if (auto h = find_hierarchy(c, rhs, phi, key, staged, p)) return h;
   if (rhs.dtype != DT_F64 || phi.dtype != DT_F64) fail(MG_EINVAL, "mg_solve needs FP64 fabs");
   if (rhs.lay.ncomp != 1 || phi.lay.ncomp != 1) fail(MG_EINVAL, "mg_solve needs 1-component fabs");
   if (!same_boxes(rhs.ba->ba, phi.ba->ba)) fail(MG_EINVAL, "rhs and phi are on different box arrays");
@@ -398,6 +411,7 @@ Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, cons
     H->stage_phi = copies(*H->phi0, *up);
     H->stage_rhs = copies(*H->rhs0, *ur);
     H->unstage_phi = copies(*up, *H->phi0);
+    fill_plan(c, *up, bc, 1);  // (of the last fill)
   }
   const int nl = (int)lev.size();
   H->L.resize(nl);
@@ -531,7 +545,7 @@ Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, cons
   H->dnorm = c.alloc(16, s);
   MG_CK(cudaStreamSynchronize(s));
   c.hier.push_back(std::move(H));
-  return *c.hier.back();
+  return c.hier.back();
 }
 
 namespace {
@@ -740,16 +754,35 @@ void destroy_hierarchies(Ctx& c) {
   c.hier.clear();
 }
 
-// The hierarchy of a solve on its own; not staged where there is no memory for that.
-static Hierarchy& single_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, SolveParams p) {
+void give_back(Ctx& c) {
+  std::unique_lock<std::recursive_mutex> lk(c.hier_mu, std::try_to_lock);
+  if (!lk) return;  // (another thread is building one)
+  std::vector<std::shared_ptr<Hierarchy>> keep;
+  for (auto& h : c.hier)
+    if (h.use_count() > 1 || !(h->staged || h->sranks > 1)) keep.push_back(std::move(h));
+  c.hier.swap(keep);
+}
+
+// The hierarchy of a solve on its own; not staged where there is no room for that.
+static std::shared_ptr<Hierarchy> single_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, SolveParams p) {
   p.single = true;
+  if (!wants_staging(phi, p)) return get_hierarchy(c, rhs, phi, bc, p);
+  int per[3];
+  const int key = bc_code(bc, per);
+  auto room = [&] { return c.pool_cap - std::min(c.pool_cap, c.in_use.load()); };
+  auto h = find_hierarchy(c, rhs, phi, key, false, p);
+  if (h && h->unstaged && room() <= h->unstaged_room) return h;
   try {
+    SpareMemory spare;
     return get_hierarchy(c, rhs, phi, bc, p);
   } catch (const MgError& e) {
     if (e.code != MG_ENOMEM) throw;
   }
   p.single = false;
-  return get_hierarchy(c, rhs, phi, bc, p);
+  h = get_hierarchy(c, rhs, phi, bc, p);
+  h->unstaged = true;
+  h->unstaged_room = room();
+  return h;
 }
 
 int solve(Ctx& c, int64_t rhs_id, int64_t phi_id, const mg_bc* bc, double tol,
@@ -759,7 +792,8 @@ int solve(Ctx& c, int64_t rhs_id, int64_t phi_id, const mg_bc* bc, double tol,
   auto rhs = c.get_fab(rhs_id);
   auto phi = c.get_fab(phi_id);
   double t_start = c.now();
-  Hierarchy& H = single_hierarchy(c, *rhs, *phi, bc, p);
+  const std::shared_ptr<Hierarchy> held = single_hierarchy(c, *rhs, *phi, bc, p);
+  Hierarchy& H = *held;
   prepare_alone(c, H);
   cudaStream_t s = c.stream;
   if (!H.hnorm) MG_CK(cudaMallocHost(&H.hnorm, 16));

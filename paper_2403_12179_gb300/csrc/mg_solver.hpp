@@ -48,7 +48,10 @@ struct Hierarchy {
   // copied there before the first cycle and phi back after the last, in place of a ghost fill before
   // every half-sweep of the finest level (GB300: 96 x 80 x 112 in boxes of 48, 2462 -> 2131 us; the three
   // copies and the last fill take 25 us).
-  bool staged = false;
+  // Where the pool has no room for that the solve works on the caller's boxes, and tries again when
+  // there is more room than there was (unstaged_room, of a hierarchy that is not staged for that reason).
+  bool staged = false, unstaged = false;
+  size_t unstaged_room = 0;
   OpTable stage_phi, stage_rhs, unstage_phi;
   std::shared_ptr<FabObj> r0;          // mixed: FP64 residual stored by each norm check (between the
                                        // scaling and that check, the second phi of the whole sweeps)
@@ -102,7 +105,7 @@ struct Hierarchy {
 
 
 // Cached per (rhs fab, phi fab, bc, options); builds coarse levels, tables and plans.
-Hierarchy& get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, const SolveParams& p);
+std::shared_ptr<Hierarchy> get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, const SolveParams& p);
 // The tables that only a solve on its own launches from (whole sweeps, residual + restriction and coarse
 // cycle of one hierarchy), once per hierarchy, before its cycles are enqueued or captured: members of
 // batches go without (64^3 FP64 members: 74 KB each of 2.9 MB, and 0.4 of 4.1 ms for the first batch of

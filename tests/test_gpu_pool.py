@@ -62,3 +62,44 @@ def test_solve_fits_where_a_batch_of_one_fits(n, box, precision):
     assert alone[0] >= in_batch[0] + 4096 * 8
     tight = run(in_batch[0] + (16 << 10), False)
     assert tight[1:] == alone[1:] == in_batch[1:]
+
+
+def test_staged_solve_gives_way():
+    """An FP64 solve over ragged boxes keeps phi and rhs on a box of its own.  That memory is given back
+    when the caller's next fab needs it, and the solve goes without it (the same bits) until there is
+    room again."""
+    n, box = (96, 80, 112), (48, 48, 48)
+    cells = n[0] * n[1] * n[2]
+
+    def solve(ctx, r, u):
+        mg.mg_fab_set_val(ctx, u, 0.0)
+        res = mg.mg_solve(ctx, r, u, mg.make_bc((0, 0, 0)), 1e-10, mg.make_options(fixed_vcycles=3))
+        return res.rel_resid, gu.fab_dense(ctx, u, n[::-1]).tobytes()
+
+    def fabs(ctx):
+        ba = mg.mg_box_array_create(ctx, (0, 0, 0), tuple(v - 1 for v in n), box)
+        r, u = mg.mg_fab_alloc(ctx, ba, 1, 0), mg.mg_fab_alloc(ctx, ba, 1, 1)
+        mg.mg_fab_set_val(ctx, r, 1.0)
+        return ba, r, u
+
+    ctx = mg.mg_init(0)
+    try:
+        _, r, u = fabs(ctx)
+        empty = mg.mg_pool_info(ctx)[1]
+        ref = solve(ctx, r, u)
+        full = mg.mg_pool_info(ctx)[1]
+        assert full - empty >= 2 * 8 * cells  # staged: phi and rhs again
+    finally:
+        mg.mg_finalize(ctx)
+    ctx = mg.mg_init(0, full + 8 * cells // 2)  # room for half a fab more
+    try:
+        ba, r, u = fabs(ctx)
+        assert solve(ctx, r, u) == ref and mg.mg_pool_info(ctx)[1] == full
+        other = mg.mg_fab_alloc(ctx, ba, 1, 0)  # takes it
+        assert mg.mg_pool_info(ctx)[1] < full
+        for _ in range(2):
+            assert solve(ctx, r, u) == ref and mg.mg_pool_info(ctx)[1] < full
+        mg.mg_fab_free(ctx, other)
+        assert solve(ctx, r, u) == ref and mg.mg_pool_info(ctx)[1] >= full
+    finally:
+        mg.mg_finalize(ctx)
