@@ -39,13 +39,12 @@ namespace gbmg {
 namespace {
 
 // The coarse side of a coarse/fine ghost: element offsets into the coarse phi fab (c[3q + p]:
-// tangential offsets p - 1 along the lower tangential dimension, q - 1 along the other); par bit
-// 0 / 1: the fine cell sits in the upper half of its parent along the lower / other tangential
-// dimension (weights at +1/4), else the lower half (-1/4).
+// tangential offsets p - 1 along the lower tangential dimension, q - 1 along the other); c[0] is
+// 4 times its offset plus, in bits 0 / 1, whether the fine cell sits in the upper half of its parent
+// along the lower / other tangential dimension (weights at +1/4), else the lower half (-1/4).  (With
+// the fine side and the kept value 104 bytes a ghost, as many as one entry of all took.)
 struct CFGhost {
   long long c[9];
-  int par;
-  int pad_;
 };
 
 // The fine side: element offsets into the fine phi fab (the ghost, the first and second fine
@@ -81,12 +80,13 @@ __global__ void __launch_bounds__(256) k_cf_coarse(const CFGhost* __restrict__ T
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const CFGhost& e = T[i];
-  const double* w0 = (e.par & 1) ? kWHi : kWLo;
-  const double* w1 = (e.par & 2) ? kWHi : kWLo;
+  const int par = (int)e.c[0] & 3;
+  const double* w0 = (par & 1) ? kWHi : kWLo;
+  const double* w1 = (par & 2) ? kWHi : kWLo;
   double c = 0.0;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    double cq = __dmul_rn(w0[0], coarse[e.c[3 * q]]);
+    double cq = __dmul_rn(w0[0], coarse[q == 0 ? e.c[0] >> 2 : e.c[3 * q]]);
     cq = __fma_rn(w0[1], coarse[e.c[3 * q + 1]], cq);
     cq = __fma_rn(w0[2], coarse[e.c[3 * q + 2]], cq);
     c = q == 0 ? __dmul_rn(w1[0], cq) : __fma_rn(w1[q], cq, c);
@@ -306,7 +306,7 @@ AmrPlan& get_plan(Ctx& c, int64_t rhs0, int64_t phi0, int64_t rhs1, int64_t phi1
             cc[t1] = P1 + qq - 1;
             e.c[3 * qq + pp] = oc.at(cc[0], cc[1], cc[2]);
           }
-        e.par = (i & 1) | ((j & 1) << 1);
+        e.c[0] = 4 * e.c[0] + ((i & 1) | ((j & 1) << 1));
         cf.push_back(e);
         cff.push_back(ef);
       }

@@ -103,3 +103,28 @@ def test_staged_solve_gives_way():
         assert solve(ctx, r, u) == ref and mg.mg_pool_info(ctx)[1] >= full
     finally:
         mg.mg_finalize(ctx)
+
+
+def test_amr_tables_per_ghost():
+    """A two-level plan's tables: 104 bytes a coarse/fine ghost (offsets of three fine and nine coarse
+    cells and the kept coarse value).  From two plans over one pair of levels, of which the second (other
+    options) builds its tables once more; the refluxing table takes 88 bytes a coarse face, and 0.9 MB
+    are allowed for the hierarchy and the box tables (at 8 bytes a ghost more, the excess is 0.8 MB)."""
+    ctx = mg.mg_init(0)
+    try:
+        n, m = 64, 128  # refined region: the whole domain but one coarse cell at every face
+        ba0 = mg.mg_box_array_create(ctx, (0, 0, 0), (n - 1,) * 3, (n,) * 3)
+        ba1 = mg.mg_box_array_create(ctx, (2, 2, 2), (m - 3,) * 3, (m,) * 3)
+        f = [mg.mg_fab_alloc(ctx, b, 1, g) for b, g in ((ba0, 0), (ba0, 1), (ba1, 0), (ba1, 1))]
+        mg.mg_fab_set_val(ctx, f[0], 1.0)
+        mg.mg_fab_set_val(ctx, f[2], 1.0)
+        used = mg.mg_pool_info(ctx)[1]
+        mg.mg_amr2_solve(ctx, *f, mg.make_bc((0, 0, 0)), 1e-10, mg.make_options(fixed_vcycles=1))
+        ghosts, c0, c1 = 6 * (m - 4) ** 2, n ** 3, (m - 4) ** 3
+        # work fabs r0, e0 (one ghost), r1; the hierarchy's levels below the finest
+        fabs = 8 * (c0 + (n + 2) * (n + 2) ** 2 + c1) + 8 * 2 * c0 / 7 * 1.2
+        # one-colour arrays of the finest coarse level
+        fabs += 8 * c0
+        assert mg.mg_pool_info(ctx)[1] - used <= fabs + 104 * ghosts + 88 * ghosts / 4 + 0.5e6
+    finally:
+        mg.mg_finalize(ctx)
