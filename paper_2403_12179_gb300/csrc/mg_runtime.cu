@@ -1217,28 +1217,32 @@ int mg_smooth(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double hh
     auto fr = c->get_fab(rhs);
     same_shape(*fp, *fr, "mg_smooth");
     if (fp->lay.g < 1) fail(MG_EINVAL, "phi needs at least one ghost cell");
-    if ((color & ~MG_SMOOTH_DIRECT_READS) == 0 || (color & ~MG_SMOOTH_DIRECT_READS) == 1) {
-      if (color & MG_SMOOTH_DIRECT_READS) {  // one half-sweep reading neighbouring boxes
-        int per[3];
-        const int code = bc_code(bc, per);
-        cudaStream_t s = S(stream);
-        double hv = default_h(*fp, hh);
-        const std::string op = "smooth_direct" + std::to_string(code);
-        const OpTable& t = op_table(*c, op.c_str(), {phi, rhs}, hv, [&] {
-          FaceReads faces = direct_neighbours(*fp, per);
-          if (!faces.ok())
-            fail(MG_EINVAL, "direct reads need boxes on a regular grid and even periodic extents");
-          OpTable tt = make_table(*c, fp->ba->ba, 0, hv, 0, [&](int b, DRow& R) {
-            R.v[0] = fp->view(b);
-            R.v[1] = fr->view(b);
-            faces.apply(b, R);
-          }, c->stream);
-          tt.direct = true;
-          return tt;
-        });
-        MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, color & 1, s, true, nullptr, t.width, false, t.ext));
-        return MG_OK;
-      }
+    cudaStream_t s = S(stream);
+    const double hv = default_h(*fp, hh);
+    // table of the forms that read neighbouring boxes, empty if the boxes do not allow it (kept too, so
+    // that they are not looked at again)
+    auto face_table = [&]() -> const OpTable& {
+      int per[3];
+      const std::string op = "smooth_direct" + std::to_string(bc_code(bc, per));
+      return op_table(*c, op.c_str(), {phi, rhs}, hv, [&] {
+        FaceReads faces = direct_neighbours(*fp, per);
+        if (!faces.ok()) return OpTable{};
+        OpTable tt = make_table(*c, fp->ba->ba, 0, hv, 0, [&](int b, DRow& R) {
+          R.v[0] = fp->view(b);
+          R.v[1] = fr->view(b);
+          faces.apply(b, R);
+        }, c->stream);
+        tt.direct = true;
+        return tt;
+      });
+    };
+    if (color == MG_SMOOTH_DIRECT_READS || color == (1 | MG_SMOOTH_DIRECT_READS)) {
+      // one half-sweep reading neighbouring boxes
+      const OpTable& t = face_table();
+      if (!t.direct)
+        fail(MG_EINVAL, "direct reads need boxes on a regular grid and even periodic extents");
+      MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, color & 1, s, true, nullptr, t.width, false, t.ext));
+      return MG_OK;
     }
     if (color < 0 || color > 2) fail(MG_EINVAL, "color must be 0, 1 or 2 (0 / 1 may add MG_SMOOTH_DIRECT_READS)");
     if (color == 2) {  // phi's ghosts, filled or read past: refused before anything is launched
@@ -1247,14 +1251,14 @@ int mg_smooth(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double hh
       std::string err;
       if (!fillable(fp->ba->ba, per, fp->lay.g, &err)) fail(MG_EINVAL, err);
     }
-    cudaStream_t s = S(stream);
-    double hv = default_h(*fp, hh);
-    const OpTable& t = op_table(*c, "smooth", {phi, rhs}, hv, [&] {
-      return make_table(*c, fp->ba->ba, 0, hv, 0, [&](int b, DRow& R) {
-        R.v[0] = fp->view(b);
-        R.v[1] = fr->view(b);
-      }, c->stream);
-    });
+    auto table = [&]() -> const OpTable& {  // of the forms that read ghost cells
+      return op_table(*c, "smooth", {phi, rhs}, hv, [&] {
+        return make_table(*c, fp->ba->ba, 0, hv, 0, [&](int b, DRow& R) {
+          R.v[0] = fp->view(b);
+          R.v[1] = fr->view(b);
+        }, c->stream);
+      });
+    };
     const bool fusable = color == 2 && fused_eligible(*fp, *fr);
     if (fusable && fp->dtype == DT_F32) {
       // boxes on a lattice: a sweep that reads the neighbouring boxes, into a scratch array, and back
@@ -1272,18 +1276,7 @@ int mg_smooth(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double hh
     // layout of the fused sweep, which leaves phi's ghosts stale, the black one too)
     const OpTable* td = nullptr;
     if (color == 2 && (fp->dtype == DT_F64 || !fusable)) {
-      int per[3];
-      const int code = bc_code(bc, per);
-      const OpTable& q = op_table(*c, ("smooth_any" + std::to_string(code)).c_str(), {phi, rhs}, hv, [&] {
-        FaceReads faces = direct_neighbours(*fp, per);
-        OpTable tt = make_table(*c, fp->ba->ba, 0, hv, 0, [&](int b, DRow& R) {
-          R.v[0] = fp->view(b);
-          R.v[1] = fr->view(b);
-          faces.apply(b, R);
-        }, c->stream);
-        tt.direct = faces.ok();
-        return tt;
-      });
+      const OpTable& q = face_table();
       if (q.direct) td = &q;
     }
     if (fusable && td) {
@@ -1308,16 +1301,16 @@ int mg_smooth(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double hh
       }
     }
     if (color < 2) {
+      const OpTable& t = table();
       MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, color, s, false, nullptr, t.width, false, t.ext));
-    } else {
-      for (int col = 0; col < 2; ++col) {
-        if (col == 0 && td) {
-          MG_CK(launch_rbgs_half(fp->dtype, td->rows(), td->nbox, td->nrows, 0, s, true, nullptr, td->width, false, td->ext));
-          continue;
-        }
-        launch_fill(*c, *fp, bc, s);
-        MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, col, s, false, nullptr, t.width, false, t.ext));
-      }
+      return MG_OK;
+    }
+    // one table for both colours (272 bytes a box): with face reads the black half-sweep finds in the
+    // neighbouring boxes what the fill before it, which leaves phi's ghosts as of then, has copied
+    const OpTable& t = td ? *td : table();
+    for (int col = 0; col < 2; ++col) {
+      if (col == 1 || !td) launch_fill(*c, *fp, bc, s);
+      MG_CK(launch_rbgs_half(fp->dtype, t.rows(), t.nbox, t.nrows, col, s, td && col == 0, nullptr, t.width, false, t.ext));
     }
     return MG_OK;
   });

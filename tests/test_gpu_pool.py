@@ -128,3 +128,23 @@ def test_amr_tables_per_ghost():
         assert mg.mg_pool_info(ctx)[1] - used <= fabs + 104 * ghosts + 88 * ghosts / 4 + 0.5e6
     finally:
         mg.mg_finalize(ctx)
+
+
+@pytest.mark.parametrize("box", [(4, 4, 4), (4, 4, 24)])
+@pytest.mark.parametrize("dt", [mg.MG_F64, mg.MG_F32])
+def test_whole_sweep_keeps_one_table(box, dt):
+    """mg_smooth with color 2 keeps one box table (272 bytes a box) besides the fill's tags, on a lattice
+    of boxes and off it."""
+    ctx = mg.mg_init(0)
+    try:
+        n = (32, 32, 40)
+        ba = mg.mg_box_array_create(ctx, (0, 0, 0), tuple(v - 1 for v in n), box)
+        nb = len(mg.mg_box_array_info(ctx, ba)[1])
+        f, r = mg.mg_fab_alloc(ctx, ba, 1, 1, dt), mg.mg_fab_alloc(ctx, ba, 1, 0, dt)
+        bc = mg.make_bc((0, 0, 0))
+        mg.mg_fill_boundary(ctx, f, bc)
+        used = mg.mg_pool_info(ctx)[1]
+        mg.mg_smooth(ctx, f, r, bc, 0.1, 2)
+        assert 0 < mg.mg_pool_info(ctx)[1] - used <= 272 * nb + 256
+    finally:
+        mg.mg_finalize(ctx)
