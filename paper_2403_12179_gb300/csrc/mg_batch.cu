@@ -71,7 +71,11 @@ struct SegB {
     const bool first = v.empty();
     ext.ok = (first || ext.ok) && t.ext.ok && nbox + t.nbox <= kMarchMaxBoxes;
     ext.even = (first || ext.even) && t.ext.even;
-    for (int d = 0; d < 3; ++d) ext.n[d] = std::max(ext.n[d], t.ext.n[d]);
+    for (int d = 0; d < 3; ++d) {
+      ext.n[d] = std::max(ext.n[d], t.ext.n[d]);
+      ext.march[d] += t.ext.march[d];
+      ext.rows[d] += t.ext.rows[d];
+    }
     direct = direct || t.direct;
     width = std::max(width, t.width);
     Seg s{};

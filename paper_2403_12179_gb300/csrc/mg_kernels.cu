@@ -1168,8 +1168,8 @@ cudaError_t launch_rbgs_half_l(int dt, const SegList& L, long long nrows, int co
   if (norms && (L.n != 1 || !direct)) return cudaErrorInvalidValue;
   if (pre && !norms) return cudaErrorInvalidValue;
   // FP64 boxes of even width march through their planes (mg_march.cu: 256^3 130 -> 88 us); the
-  // row kernel below is for the others and FP32
-  if (dt == DT_F64 && L.ext.ok && L.ext.even)
+  // row kernel below is for the others, small boxes and FP32
+  if (dt == DT_F64 && march_pays(L, MARCH_HALF, direct))
     return launch_half_march(L, norms ? (pre ? 2 : 1) : 0, color, norms, s);
   // a line of w cells holds w / 2 of one colour; two per lane (four on FP32 rows of 64 to
   // 127 cells)
@@ -1201,7 +1201,7 @@ cudaError_t launch_rbgs_half_l(int dt, const SegList& L, long long nrows, int co
 cudaError_t launch_residual_l(int dt, const SegList& L, long long nrows, unsigned long long* norms,
                               cudaStream_t s, bool direct, int color) {
   if (nrows <= 0) return cudaSuccess;
-  if (dt == DT_F64 && color < 0 && L.ext.ok)  // (256^3: 238 -> 182 us)
+  if (dt == DT_F64 && color < 0 && march_pays(L, MARCH_RESIDUAL, direct))  // (256^3: 238 -> 182 us)
     return launch_residual_march(L, norms, s);
   Grid g = row_grid(nrows, 16);
   GB_DISPATCH_D(dt, direct, k_residual, g.blocks, kThreads, 0, s, L, nrows, g.per, norms, color);
@@ -1227,7 +1227,7 @@ void prolong_add_g(int G, const Grid& g, cudaStream_t s, const SegList& L, long 
 cudaError_t launch_residual_restrict_l(int dt, const SegList& L, long long nrows, cudaStream_t s,
                                        bool direct, bool stored) {
   if (nrows <= 0) return cudaSuccess;
-  if (dt == DT_F64 && L.ext.ok && L.ext.even) return launch_restrict_march(L, stored, s);
+  if (dt == DT_F64 && march_pays(L, MARCH_RESTRICT, direct)) return launch_restrict_march(L, stored, s);
   // rows are coarse lines of width / 2 cells, one per lane
   const int G = group_lanes(L.width, 2, 8, 32);
   const Grid g = row_grid(nrows, row_blocks_per_sm(L.width), kWarps * (32 / G));
@@ -1390,7 +1390,7 @@ cudaError_t launch_rbgs_half_store(const DRow* rows, int nbox, long long nrows, 
                                    cudaStream_t s, int width, const BoxExtents& ext) {
   if (nrows <= 0) return cudaSuccess;
   const SegList L = one_seg(rows, nbox, 0, width, ext);
-  if (ext.ok && ext.even) return launch_half_march(L, 3, color, nullptr, s);
+  if (march_pays(L, MARCH_HALF, true)) return launch_half_march(L, 3, color, nullptr, s);
   const int G = group_lanes(L.width, 4, 8, 16);
   const Grid g = row_grid(nrows, row_blocks_per_sm(L.width), kWarps * (32 / G));
   rbgs_half_norm_g<double, 3>(G, g, s, L, nrows, color, nullptr);

@@ -116,10 +116,15 @@ __host__ __device__ inline int tag_chunk_rows(int ex, int ncomp, int esize = 8) 
 // (mg_march.cu); ok if every box's x extent is at most kMarchMaxX (and there are no more boxes
 // than a grid dimension holds), even if they are all even too.
 constexpr int kMarchMaxX = 256, kMarchMaxBoxes = 65535;
+// march and rows: the work of half-sweep, residual and residual + restriction in lanes, by the marching
+// kernels and by the row kernels (add_march_work), over the boxes, which march_pays compares.
+enum { MARCH_HALF = 0, MARCH_RESIDUAL = 1, MARCH_RESTRICT = 2 };
 struct BoxExtents {
   int n[3] = {0, 0, 0};
   bool ok = false, even = false;
+  float march[3] = {0, 0, 0}, rows[3] = {0, 0, 0};
 };
+void add_march_work(const int n[3], BoxExtents* e);
 // A launch may cover the box tables of several independent solves (batched and served
 // solves): each solve's table is one segment of the launch's row space.  norms and scales
 // of a row live at index slot + DRow::solve.
@@ -275,6 +280,8 @@ cudaError_t launch_restore_colour(int dt, const DRow* rows, int nbox, long long 
 cudaError_t launch_residual(int dt, const DRow* rows, int nbox, long long nrows,
                             unsigned long long* norms, cudaStream_t s, bool direct = false,
                             int color = -1, const BoxExtents& ext = {});
+// Whether an FP64 launch runs faster by the marching kernels (mg_march.cu) than by the row kernels.
+bool march_pays(const SegList& L, int op, bool direct);
 // The same (FP64, every cell) marching through planes (mg_march.cu); norms may be null.
 cudaError_t launch_residual_march(const SegList& L, unsigned long long* norms, cudaStream_t s);
 

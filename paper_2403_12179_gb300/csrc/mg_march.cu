@@ -524,6 +524,57 @@ bool use_int(const SegList& L) {
 
 }  // namespace
 
+// The marching kernels give a thread a pair of cells and a block whole rows of one box, so small boxes
+// leave lanes idle and blocks with one or two warps at work; the row kernels pack rows of many boxes
+// into a block, but leave lanes of narrow rows idle.  Counted per plane of a box: 32 lanes a warp at
+// work, twice for the residual (a thread takes both cells), against the lanes of the rows; blocks of
+// one or two warps hide less latency and count more (one: a half-sweep of rows of 16 cells and more
+// 1.3 times, restriction 1.6, residual 2.1; two: restriction and residual 1.15), the rows against
+// blocks of three or four 1.25 times.  Measured on GB300, row kernels / marching, us (the faster one is
+// taken): half-sweep of 64^3 in boxes of 4^3 9.2 / 14.3, 8 x 4 x 4 6.2 / 8.1, 8 x 2 x 64 6.2 / 12.6, 4 x 8 x 8 9.3 / 7.3, 8^3
+// 6.2 / 4.9; residual of 32^3 in 2^3 14.5 / 24.7, 128^3 in 32 x 2 x 128 37 / 64, 8^3 123 / 63; restriction of
+// 64^3 in 4^3 21 / 55, 128^3 in 8^3 67 / 82, 16^3 35 / 41, 8 x 16 x 8 67 / 49.
+void add_march_work(const int n[3], BoxExtents* e) {
+  auto lanes = [](int width, int cells, int lo, int hi) {  // of a row's group in the row kernels
+    int g = lo;
+    while (g < hi && g * cells < width) g *= 2;
+    return g;
+  };
+  const int pp = (n[0] + 1) / 2;
+  if (pp > kMarchThreads) return;
+  const int rb = kMarchThreads / pp;
+  auto warps = [&](int rows) { return rows / rb * ((pp * rb + 31) / 32) + (pp * (rows % rb) + 31) / 32; };
+  auto busy = [&](int rows) { return (pp * std::min(rows, rb) + 31) / 32; };  // warps of a block at work
+  auto up = [](int a, int b) { return (a + b - 1) / b * b; };
+  const float nz = (float)n[2];
+  const int one = busy(n[1]), two = busy(n[1] / 2);
+  e->march[MARCH_HALF] += nz * 32 * warps(n[1]) * (one == 1 && pp >= 8 ? 1.3f : 1.f);
+  e->rows[MARCH_HALF] += nz * n[1] * up(pp, lanes(n[0], 4, 4, 16)) * (one > 2 ? 1.25f : 1.f);
+  e->march[MARCH_RESIDUAL] += nz * 64 * warps(n[1]) * (one == 1 ? 2.1f : one == 2 ? 1.15f : 1.f);
+  e->rows[MARCH_RESIDUAL] += nz * n[1] * up(n[0], 32) * (one > 2 ? 1.25f : 1.f);
+  e->march[MARCH_RESTRICT] += nz * 32 * warps(n[1] / 2) * (two == 1 ? 1.6f : two == 2 ? 1.15f : 1.f);
+  e->rows[MARCH_RESTRICT] += nz * (n[1] / 2) * up(pp, lanes(n[0], 2, 8, 32)) * (two > 2 ? 1.25f : 1.f);
+}
+
+// Where the work is against them, the marching kernels still win while their blocks are few and short
+// enough to run at once (7 blocks an SM of the half-sweep, 4 of the restriction; rows that read their ghosts
+// start faster), and in the restriction with direct reads up to 1.4 times the work, whose row form spends more
+// on its neighbours' places: half-sweep with direct reads of 32^3 in 32 x 2 x 2 3.1 us, rows 4.6; 64^3 solve
+// in boxes of 32^3 with stages down to the bottom 1.09 ms, 1.29 without this line.  Solves, with the
+// marching kernels throughout / with this rule: 64^3 in 4^3 2.20 / 1.48 ms, 128^3 in 8^3 4.70 / 3.87, six of 64^3 in
+// 8^3 4.06 / 3.37, four of 128^3 in 16^3 8.72 / 8.21.
+bool march_pays(const SegList& L, int op, bool direct) {
+  const BoxExtents& e = L.ext;
+  if (!e.ok || (op != MARCH_RESIDUAL && !e.even)) return false;
+  if (e.march[op] <= e.rows[op]) return true;
+  if (op == MARCH_RESIDUAL) return false;
+  int zc;
+  const dim3 g = march_grid(L, &zc, op == MARCH_RESTRICT ? 2 : 1);
+  const long long blocks = (long long)g.x * g.y, sms = num_sms();
+  if (op == MARCH_HALF) return std::min(zc, e.n[2]) <= 4 && blocks <= (direct ? 7 : 2) * sms;
+  return blocks <= (direct ? 4 : 2) * sms || (direct && e.march[op] <= 1.4f * e.rows[op]);
+}
+
 cudaError_t launch_half_march(const SegList& L, int mode, int color, unsigned long long* norms,
                               cudaStream_t s) {
   int zc;
