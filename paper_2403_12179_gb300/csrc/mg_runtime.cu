@@ -366,6 +366,7 @@ void ensure_valid_rows(Ctx& c, FabObj& f) {
   append_rows(&rows, &n, f.ba->ba, 0, 1.0, 0, [&](int b, DRow& R) { R.v[0] = f.view(b); });
   f.valid_rows = c.upload(rows.data(), rows.size() * sizeof(DRow), c.stream);
   f.nrows = n;
+  for (const DRow& R : rows) f.width = std::max(f.width, R.n[0]);
   MG_CK(cudaStreamSynchronize(c.stream));
 }
 
@@ -407,7 +408,7 @@ void dense_upload(Ctx& c, FabObj& f, const void* host, cudaStream_t s) {
   DevBufP stage = c.alloc(bytes, s);
   MG_CK(cudaMemcpyAsync(stage->p, host, bytes, cudaMemcpyHostToDevice, s));
   MG_CK(launch_dense_copy(f.dtype, (const DRow*)f.valid_rows->p, (int)f.ba->ba.boxes.size(),
-                          f.nrows, stage->p, D.lo, n, f.lay.ncomp, 0, s, f.width()));
+                          f.nrows, stage->p, D.lo, n, f.lay.ncomp, 0, s, f.width));
   stage->reset(s);
 }
 
@@ -418,7 +419,7 @@ void dense_download(Ctx& c, FabObj& f, void* host, cudaStream_t s) {
   const size_t bytes = (size_t)D.npts() * f.lay.ncomp * f.esize();
   DevBufP stage = c.alloc(bytes, s);
   MG_CK(launch_dense_copy(f.dtype, (const DRow*)f.valid_rows->p, (int)f.ba->ba.boxes.size(),
-                          f.nrows, stage->p, D.lo, n, f.lay.ncomp, 1, s, f.width()));
+                          f.nrows, stage->p, D.lo, n, f.lay.ncomp, 1, s, f.width));
   MG_CK(cudaMemcpyAsync(host, stage->p, bytes, cudaMemcpyDeviceToHost, s));
   stage->reset(s);
 }
@@ -1124,7 +1125,7 @@ int mg_fab_copy_from_dense(mg_ctx_t h, mg_fab_t fab, const void* src, int src_on
     }
     MG_CK(launch_dense_copy(f->dtype, (const DRow*)f->valid_rows->p, (int)f->ba->ba.boxes.size(),
                             f->nrows, const_cast<void*>(dsrc), D.lo, n, f->lay.ncomp, 0, s,
-                            f->width()));
+                            f->width));
     if (stage) stage->reset(s);
     return MG_OK;
   });
@@ -1147,7 +1148,7 @@ int mg_fab_copy_to_dense(mg_ctx_t h, mg_fab_t fab, void* dst, int dst_on_host, v
       ddst = stage->p;
     }
     MG_CK(launch_dense_copy(f->dtype, (const DRow*)f->valid_rows->p, (int)f->ba->ba.boxes.size(),
-                            f->nrows, ddst, D.lo, n, f->lay.ncomp, 1, s, f->width()));
+                            f->nrows, ddst, D.lo, n, f->lay.ncomp, 1, s, f->width));
     if (dst_on_host) {
       MG_CK(cudaMemcpyAsync(dst, stage->p, bytes, cudaMemcpyDeviceToHost, s));
       stage->reset(s);

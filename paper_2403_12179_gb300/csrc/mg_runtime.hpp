@@ -121,11 +121,7 @@ struct FabObj {
   long long nrows = 0;
   std::shared_ptr<FabObj> partner;  // same-layout scratch for out-of-place sweeps
   std::shared_ptr<FabObj> plain;    // the same boxes without ghosts, for the same purpose
-  int width() const {               // widest box
-    int w = 0;
-    for (const Box& b : ba->ba.boxes) w = w > b.len(0) ? w : b.len(0);
-    return w;
-  }
+  int width = 0;                    // widest box (set with valid_rows)
   DView view(int b) const;
   int esize() const { return dtype == DT_F64 ? 8 : 4; }
   // whether the two fabs' storage shares bytes (one fab, or wrapped memory)
