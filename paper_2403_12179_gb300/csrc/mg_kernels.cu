@@ -1147,6 +1147,13 @@ int group_lanes(int width, int cells, int lo, int hi) {
   return g;
 }
 
+// More lanes a line for launches that would not give every SM a block otherwise (dense copy of 32^3 FP64
+// 2.0 us, 2.2 with 8 lanes a line).
+int spread_lanes(int G, int width, long long nrows) {
+  while (G < 32 && G < width && nrows * G < (long long)num_sms() * kThreads) G *= 2;
+  return G;
+}
+
 template <class T, bool DIRECT, int MODE = 0>
 void rbgs_half_g(int G, const Grid& g, cudaStream_t s, const SegList& L, long long nrows, int color,
                  unsigned long long* norms) {
@@ -1269,7 +1276,9 @@ cudaError_t launch_prolong_trilinear_l(int dt, const SegList& L, long long nrows
 
 cudaError_t launch_prolong_add_l(int dt, const SegList& L, long long nrows, cudaStream_t s) {
   if (nrows <= 0) return cudaSuccess;
-  const int G = group_lanes(L.width, dt == DT_F64 ? 2 : 4, 8, 32);  // cells per lane step
+  // cells per lane step; FP64: pairs, but up to 64^3 cells a lane a cell, more blocks (32^3 2.2 us, 2.8 with
+  // pairs; 64^3 in boxes of 16^3 3.4 and 3.8)
+  const int G = group_lanes(L.width, dt == DT_F64 ? (nrows * L.width <= 1ll << 18 ? 1 : 2) : 4, 8, 32);
   // FP64: the blocks that are resident (128^3 in boxes of 32^3: 12.7 us against 15.7 with four times as many)
   const Grid g = row_grid(nrows, dt == DT_F64 ? 8 : row_blocks_per_sm(L.width), kWarps * (32 / G));
   if (dt == DT_F64) prolong_add_g<double>(G, g, s, L, nrows);
@@ -1317,7 +1326,7 @@ cudaError_t launch_set_valid_l(int dt, const SegList& L, long long nrows, double
 cudaError_t launch_maxabs_l(int dt, const SegList& L, long long nrows, unsigned long long* norms,
                             cudaStream_t s) {
   if (nrows <= 0) return cudaSuccess;
-  const int G = group_lanes(L.width, kCopyCells, 8, 32);
+  const int G = spread_lanes(group_lanes(L.width, kCopyCells, 8, 32), L.width, nrows);
   const Grid g = row_grid(nrows, 8, kWarps * (32 / G));
   auto go = [&](auto k) { launch_k(k, g.blocks, kThreads, 0, s, L, nrows, g.per, norms); };
   if (dt == DT_F64) {
@@ -1401,7 +1410,8 @@ cudaError_t launch_rbgs_half_store(const DRow* rows, int nbox, long long nrows, 
 cudaError_t launch_restrict(int dt, const DRow* rows, int nbox, long long nrows, cudaStream_t s, int width) {
   if (nrows <= 0) return cudaSuccess;
   const int G = group_lanes(width, 2, 8, 32);  // rows are coarse lines of width / 2 cells
-  const Grid g = row_grid(nrows, 8, kWarps * (32 / G));
+  // (blocks an SM: FP64 256^3 in one box 37.2 us with 16, 41.2 with 8; FP32 192^3 in boxes of 96^3 8.0 and 7.4)
+  const Grid g = row_grid(nrows, dt == DT_F64 ? 16 : 8, kWarps * (32 / G));
   const SegList L = one_seg(rows, nbox, 0, width);
   auto go = [&](auto k) { launch_k(k, g.blocks, kThreads, 0, s, L, nrows, g.per); };
   if (dt == DT_F64) {
@@ -1475,7 +1485,7 @@ cudaError_t launch_dense_copy(int dt, const DRow* rows, int nbox, long long nrow
                               const int dom_lo[3], const int dom_n[3], int ncomp, int to_dense,
                               cudaStream_t s, int width) {
   if (nrows <= 0) return cudaSuccess;
-  const int G = group_lanes(width, kCopyCells, 8, 32);
+  const int G = spread_lanes(group_lanes(width, kCopyCells, 8, 32), width, nrows);
   const Grid g = row_grid(nrows, row_blocks_per_sm(width), kWarps * (32 / G));
   const SegList L = one_seg(rows, nbox, 0, width);
   int3 lo = make_int3(dom_lo[0], dom_lo[1], dom_lo[2]);
@@ -1496,7 +1506,7 @@ cudaError_t launch_dense_copy(int dt, const DRow* rows, int nbox, long long nrow
 
 cudaError_t launch_copy_valid(int dt, const DRow* rows, int nbox, long long nrows, cudaStream_t s, int width) {
   if (nrows <= 0) return cudaSuccess;
-  const int G = group_lanes(width, kCopyCells, 8, 32);
+  const int G = spread_lanes(group_lanes(width, kCopyCells, 8, 32), width, nrows);
   const Grid g = row_grid(nrows, row_blocks_per_sm(width), kWarps * (32 / G));
   const SegList L = one_seg(rows, nbox, 0, width);
   auto go = [&](auto k) { launch_k(k, g.blocks, kThreads, 0, s, L, nrows, g.per); };
