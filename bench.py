@@ -171,6 +171,7 @@ def whole_job_rate(world, steps, max_total_ms):
 KERNEL_SOURCES = {
     "rbgs_half_f64": ["mg_march.cu", "mg_isum.hpp", "mg_isum_dev.cuh", "mg_kernels.hpp"],
     "rbgs_fused_f32": ["mg_fused.cu", "mg_kernels.hpp", "mg_runtime.cu"],
+    "sweep_f32": ["mg_sweep.cu", "mg_sweep.hpp", "mg_kernels.hpp"],
     "copy_tags_f64": ["mg_kernels.cu", "mg_kernels.hpp", "mg_runtime.cu"],
 }
 
@@ -270,7 +271,7 @@ def run_ours(args, wl_name):
     assert all(r.status == 0 and r.rel_resid <= 1e-10 for r in results)
 
     # ---- dominant kernels on the fine level, timed alone on the solve stream
-    kt = kernel_timings(ctx, stream, ba, fp, fr, bc, h, cells, box)
+    kt = kernel_timings(ctx, stream, ba, fp, fr, bc, h, cells, box, mixed=prec == mg.MG_PREC_MIXED)
     if sweep_n:
         kt["rbgs_half_f64_in_solve"] = sweep_ms / sweep_n / 1e3
     fp64 = measure_fp64_peak(stream, local)
@@ -439,12 +440,33 @@ def measure_fp64_peak(stream, device_index, target_ms=40.0):
             "clocks": clocks}
 
 
-def kernel_timings(ctx, stream, ba, fp, fr, bc, h, cells, box, reps=40):
+def sweep_in_solve(ctx, stream, fr, fp, bc, vcycles=3):
+    """Duration (s) of one whole FP32 sweep of all levels as the mixed solve launches it (no ghost
+    cells, neighbouring boxes read directly): the difference of solves with four and two
+    pre-smoothing sweeps."""
+    from paper_2403_12179_gb300 import mg
+    inner = 2
+
+    def timed(nu1):
+        opt = mg.make_options(precision=mg.MG_PREC_MIXED, nu1=nu1, inner_cycles=inner, fixed_vcycles=vcycles)
+
+        def solve(_):
+            mg.mg_fab_set_val(ctx, fp, 0.0, True, stream)
+            mg.mg_solve(ctx, fr, fp, bc, 1e-10, opt)
+        return _time(stream, solve, 3)
+
+    return (timed(4) - timed(2)) / (2 * inner * vcycles)
+
+
+def kernel_timings(ctx, stream, ba, fp, fr, bc, h, cells, box, reps=40, mixed=False):
     """Average launch durations (s) of the fine-level kernels, each launched back to back
     on `stream` between two CUDA events: FP64 half-sweep, FP64 residual + norm, FP32 fused
-    sweep (out of place), FP32 half-sweep."""
+    sweep (out of place), FP32 half-sweep; of a mixed workload also a whole FP32 sweep of all
+    levels inside its solve."""
     from paper_2403_12179_gb300 import mg
     out = {}
+    if mixed:
+        out["sweep_f32_all_levels"] = sweep_in_solve(ctx, stream, fr, fp, bc)
     mg.mg_fill_boundary(ctx, fp, bc, stream)
     # the FP64 half-sweep as the solver runs it on regular box grids (neighbour boxes read
     # directly), and with ghost cells
@@ -496,9 +518,9 @@ def roofline(kt, wl_name, f64, fp64, in_solve_launches=0):
                           "dram_min_frac": round(12 * cells / kt["rbgs_half_f32"] / 1e9 / hbm, 4)},
     }
     extra["note"] = ("the FP64 kernels (half-sweep, residual) are bound by GB300's FP64 issue "
-                     "rate, measured by fp64_peak, and by the integer units, on which half of the "
-                     "warps make the six-addend sums (and all the multiplications by 1/6), bit for "
-                     "bit: fp64_frac counts every FP64 operation of the algorithm against the FP64 "
+                     "rate, measured by fp64_peak, and by the integer units, which make the six-addend "
+                     "sums of every second plane (half-sweep) or every second cell (residual) and all the "
+                     "multiplications by 1/6, bit for bit: fp64_frac counts every FP64 operation of the algorithm against the FP64 "
                      "rate alone, so it can exceed 1; at 100% of that rate a half-sweep moves about "
                      "42% of the HBM copy peak")
     if f64:
@@ -517,12 +539,17 @@ def roofline(kt, wl_name, f64, fp64, in_solve_launches=0):
                         "algorithmic_bytes_per_launch": 16 * cells},
                 "algorithmic_ops_per_launch": half_ops,
                 "traffic": roofline_traffic("rbgs_half_f64", wl_name), "kernels": extra}
-    t = kt["rbgs_fused_f32"]
-    ach = 12 * cells / t / 1e9
-    return {"kernel": "k_rbgs_fused<float> (full sweep, fine level, mg_smooth_fused)", "bound": "hbm",
+    t = kt["sweep_f32_all_levels"]
+    swept = 12 * cells * 8 / 7   # phi and rhs read, phi written, on all levels
+    ach = swept / t / 1e9
+    return {"kernel": "k_sweep_f32 (whole red + black sweep, FP32 levels of the mixed solve)", "bound": "hbm",
+            "measured": "a sweep of all levels inside the solve: the difference of solves with four and "
+                        "two pre-smoothing sweeps (CUDA events on the solve stream)",
+            "sweep_us": round(t * 1e6, 1),
             "achieved": round(ach, 1), "peak": hbm, "unit": "GB/s", "frac": round(ach / hbm, 4),
-            "peak_source": src, "algorithmic_bytes_per_launch": 12 * cells,
-            "traffic": roofline_traffic("rbgs_fused_f32", wl_name), "kernels": extra}
+            "peak_source": src, "algorithmic_bytes": round(swept),
+            "algorithmic_bytes_per_launch": 12 * cells,  # of the finest level's launch, as traffic
+            "traffic": roofline_traffic("sweep_f32", wl_name), "kernels": extra}
 
 
 def run_kernels_only(args, wl_name):
@@ -539,7 +566,7 @@ def run_kernels_only(args, wl_name):
     fp = mg.mg_fab_alloc(ctx, ba, 1, 2)
     mg.mg_fab_set_val(ctx, fr, 1.0, True, stream)
     kt = kernel_timings(ctx, stream, ba, fp, fr, mg.make_bc(wl["periodic"]), 1.0 / n, n ** 3, box,
-                        reps=args.steps)
+                        reps=args.steps, mixed=wl["precision"] == "mixed")
     mg.mg_finalize(ctx)
     print(json.dumps({"kernels_only": wl_name, "launch_s": kt}))
 
@@ -576,7 +603,8 @@ def sub_mixed512(args, steps=5, warmup=2):
     inner V-cycle, FP64 outer residual / correction / bottom) against the plain FP64 solve of
     the same problem, both timed with CUDA events on the solve stream (L2 flushed before each
     solve, outside the events); the difference of the two answers against the bound two
-    converged answers obey (P7); the FP32 smoother kernels at this size."""
+    converged answers obey (P7); the FP32 smoother kernels at this size (the whole sweep that the solve
+    runs, the TMA sweep and the half-sweep that other layouts take)."""
     import numpy as np
     import torch
     from paper_2403_12179_gb300 import mg
@@ -626,6 +654,8 @@ def sub_mixed512(args, steps=5, warmup=2):
                      "outer_iterations" if name == "mixed" else "vcycles": res[-1].vcycles,
                      "rel_resid": res[-1].rel_resid, "clocks": clocks}
         phis[name] = _fab_to_dense(ctx, fp, (n,) * 3, stream)
+        if name == "mixed":
+            t_w = sweep_in_solve(ctx, stream, fr, fp, bc)
         mg.mg_fab_free(ctx, fp, stream)
     diff = float((phis["mixed"] - phis["f64"]).abs().max())
     del phis
@@ -646,6 +676,10 @@ def sub_mixed512(args, steps=5, warmup=2):
     t_f = _time(stream, lambda k: mg.mg_smooth_fused(ctx, pair[k & 1], r32, pair[(k + 1) & 1], bc, h, stream), 20)
     t_h = _time(stream, lambda k: mg.mg_smooth(ctx, a32, r32, bc, h, (k & 1) | mg.MG_SMOOTH_DIRECT_READS, stream), 20)
     out["kernels"] = {
+        "sweep_f32_all_levels": {"sweep_us": round(t_w * 1e6, 1), "gbs": round(12 * cells * 8 / 7 / t_w / 1e9, 1),
+                                 "hbm_frac": round(12 * cells * 8 / 7 / t_w / 1e9 / hbm, 4),
+                                 "algorithmic_bytes_per_cell": 12,
+                                 "what": "one whole sweep of all FP32 levels inside the mixed solve"},
         "rbgs_fused_f32": {"launch_us": round(t_f * 1e6, 1), "gbs": round(12 * cells / t_f / 1e9, 1),
                            "hbm_frac": round(12 * cells / t_f / 1e9 / hbm, 4),
                            "algorithmic_bytes_per_cell": 12},

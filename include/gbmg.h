@@ -249,8 +249,15 @@ int mg_fill_boundary_unfused(mg_ctx_t ctx, mg_fab_t fab, const mg_bc* bc, void* 
  *   ghost cells, as the solver does; boxes must form a regular grid and periodic extents
  *   must be even (else MG_EINVAL: an odd periodic extent makes a cell's periodic image one of
  *   its own colour).
- * color 2: one full sweep, equal to fill, red, fill, black; with phi nghost >= 2 and rhs
- *   nghost >= 1 it runs as one fused kernel after one fill of each.
+ * color 2: one full sweep: phi's valid cells equal fill, red, fill, black; phi's ghost cells
+ *   are unspecified afterwards.  With phi nghost >= 2 and rhs nghost >= 1 rhs's ghosts are
+ *   filled, and on a regular box grid with even periodic extents FP32 fabs (boxes in whole
+ *   strips of 4 cells in x, an even y extent) are swept in one launch that reads neighbouring boxes, into
+ *   a scratch array kept with phi (4 bytes a cell), and copied back, and FP64 fabs take two
+ *   direct-read half-sweeps; on other boxes one fused kernel runs after a fill of each, into a
+ *   scratch copy kept with phi.  With fewer ghosts: two half-sweeps, the first with direct reads
+ *   where the boxes allow.  MG_EINVAL, with nothing changed, where phi's ghosts cannot be
+ *   filled (more layers than a Dirichlet dimension has cells).
  * Update: phi_c = (s - h^2 rhs_c) / 6, s = x- + x+ + y- + y+ + z- + z+ (in that order). */
 int mg_smooth(mg_ctx_t ctx, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double h, int color,
               void* stream);
@@ -288,7 +295,7 @@ int mg_prolong_add(mg_ctx_t ctx, mg_fab_t coarse, mg_fab_t fine, void* stream);
 int mg_prolong_add_trilinear(mg_ctx_t ctx, mg_fab_t coarse, mg_fab_t fine, void* stream);
 
 /* Exact bottom solve on a box array of at most 1024 cells: phi = M rhs with M from
- * mg_bottom_matrix (FP64 arithmetic for either fab type). */
+ * mg_bottom_matrix (FP64 arithmetic for either fab type).  phi may share memory with rhs. */
 int mg_bottom_solve(mg_ctx_t ctx, mg_fab_t rhs, mg_fab_t phi, const mg_bc* bc, double h,
                     void* stream);
 
@@ -330,7 +337,10 @@ int mg_residual_norm_noalloc(const int dom_lo[3], const int dom_hi[3], int nbox,
  * tol ||rhs||_inf (checked before each V-cycle), or after max_iter V-cycles
  * (MG_NOT_CONVERGED).  rhs == 0 gives phi = 0.  With fully periodic faces rhs must have
  * zero mean (to within tol).  The coarse levels are allocated on first use and cached per
- * (box array, bc, options) until mg_finalize.  Returns res->status. */
+ * (rhs, phi, bc, options) until one of the fabs is freed; where an allocation finds the pool full,
+ * solves that hold more than they need (phi and rhs again, on one box, for FP64 fabs over boxes not
+ * on a grid; the tables of the cluster's coarse launch) release it and go without, with the same results.
+ * Returns res->status. */
 int mg_solve(mg_ctx_t ctx, mg_fab_t rhs, mg_fab_t phi, const mg_bc* bc, double tol,
              const mg_options* opt, mg_result* res);
 

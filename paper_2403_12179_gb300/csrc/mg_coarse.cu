@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 512 : 1024, 1) k_coarse_cycle
   const int3 per = make_int3(J.periodic[0], J.periodic[1], J.periodic[2]);
   if (threadIdx.x < nl) L[threadIdx.x] = lev_of(J.lev[threadIdx.x], arena, rank, J.periodic[2] != 0);
   T* const res = arena + J.off_res;
-    const bool ints = sizeof(T) == 8 && ((threadIdx.x >> 7) & 1);
+  const bool ints = sizeof(T) == 8 && ((threadIdx.x >> 7) & 1);
   __syncthreads();
   // gather phi (the current guess) and rhs of level lc
   T* const gphi = (T*)J.phi;

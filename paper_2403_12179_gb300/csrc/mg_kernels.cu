@@ -669,8 +669,7 @@ __global__ void __launch_bounds__(kThreads) k_prolong_add(SegList L, long long n
     const T* c = line<T>(R.c[0], (y + oy) >> 1, (z + oz) >> 1);
     if constexpr (sizeof(T) == 4) {
       // FP32: four cells of a lane per step, all loads first (measured on GB300: 512
-      // batched problems 2242 -> 2345 solves/s; the FP64 form keeps one cell per step, as
-      // four made the 256^3 FP64 solve 3% slower)
+      // batched problems 2242 -> 2345 solves/s)
       for (int x = lane; x < n0; x += 4 * G) {
         T a[4], b[4];
 #pragma unroll
@@ -686,7 +685,7 @@ __global__ void __launch_bounds__(kThreads) k_prolong_add(SegList L, long long n
         }
       }
     } else if (!ox && !(n0 & 1) && !((uintptr_t)f & 15)) {
-      // FP64: a lane takes both children of a parent
+      // FP64: a lane takes both children of a parent (four cells a step made the 256^3 solve 3% slower)
       for (int x = 2 * lane; x < n0; x += 2 * G) {
         const double2 a = *(const double2*)(f + x);
         const T b = c[x >> 1];

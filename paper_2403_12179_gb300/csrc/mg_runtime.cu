@@ -1263,9 +1263,10 @@ int mg_smooth(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double hh
     };
     const bool fusable = color == 2 && fused_eligible(*fp, *fr);
     if (fusable && fp->dtype == DT_F32) {
-      // boxes on a lattice: a sweep that reads the neighbouring boxes, into a scratch array, and back
-      // (256^3, boxes of 64^3: 121 us a call, sweep 74, copy back 28, rhs fill 18, against 135 for two
-      // fills, the TMA sweep and a copy of the whole fab, and no autotuning on the first call: 92 ms)
+      // boxes on a lattice: a sweep that reads the neighbouring boxes, into a scratch array, and back (256^3,
+      // boxes of 64^3: sweep 74 us, copy back 28, rhs fill 18).  Against two fills, the TMA sweep and a copy
+      // of the whole fab, us a call: 64^3 in 32^3 17 -> 9.6, 192^3 in 64^3 64 -> 45, 256^3 in 64^3 115 -> 122 (from
+      // DRAM 129 -> 128), 384^3 in 64^3 463 -> 338; and no autotuning on the first call (92 ms)
       const SweepTable& st = sweep_table(*c, phi, *fp, rhs, *fr, bc, hv);
       if (st.ok) {
         launch_fill(*c, *fr, bc, s);
@@ -1275,7 +1276,9 @@ int mg_smooth(mg_ctx_t h, mg_fab_t phi, mg_fab_t rhs, const mg_bc* bc, double hh
       }
     }
     // the red half-sweep may read neighbouring boxes instead of ghost cells (and, in FP64 with the
-    // layout of the fused sweep, which leaves phi's ghosts stale, the black one too)
+    // layout of the fused sweep, which leaves phi's ghosts stale, the black one too).  Against a fill and
+    // ghost reads, FP32: 64^3 in 16^3 11.6 -> 9.1 us a sweep, 256^3 in 32^3 152 -> 137, in 64^3 106 -> 114 (from
+    // DRAM 118 -> 120), in 128^3 116 -> 113
     const OpTable* td = nullptr;
     if (color == 2 && (fp->dtype == DT_F64 || !fusable)) {
       const OpTable& q = face_table();
