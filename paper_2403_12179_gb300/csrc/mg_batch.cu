@@ -66,16 +66,15 @@ struct SegB {
   bool direct = false;  // some member's rows carry box-face reads
   int width = 0, nbox = 0;
   BoxExtents ext;
+  MarchWork work;
   void add(const OpTable& t, int slot) {
     if (!t.nrows) return;
     const bool first = v.empty();
     ext.ok = (first || ext.ok) && t.ext.ok && nbox + t.nbox <= kMarchMaxBoxes;
     ext.even = (first || ext.even) && t.ext.even;
-    for (int d = 0; d < 3; ++d) {
-      ext.n[d] = std::max(ext.n[d], t.ext.n[d]);
-      ext.march[d] += t.ext.march[d];
-      ext.rows[d] += t.ext.rows[d];
-    }
+    for (int d = 0; d < 3; ++d) ext.n[d] = std::max(ext.n[d], t.ext.n[d]);
+    work.add(t.work);
+    work.compare(&ext);
     direct = direct || t.direct;
     width = std::max(width, t.width);
     Seg s{};

@@ -116,15 +116,25 @@ __host__ __device__ inline int tag_chunk_rows(int ex, int ncomp, int esize = 8) 
 // (mg_march.cu); ok if every box's x extent is at most kMarchMaxX (and there are no more boxes
 // than a grid dimension holds), even if they are all even too.
 constexpr int kMarchMaxX = 256, kMarchMaxBoxes = 65535;
-// march and rows: the work of half-sweep, residual and residual + restriction in lanes, by the marching
-// kernels and by the row kernels (add_march_work), over the boxes, which march_pays compares.
+// work: how the marching kernels' work for half-sweep, residual and residual + restriction compares with
+// the row kernels' (MarchWork; 0: no more, 1: up to 1.4 times, 2: more), for march_pays.
 enum { MARCH_HALF = 0, MARCH_RESIDUAL = 1, MARCH_RESTRICT = 2 };
 struct BoxExtents {
   int n[3] = {0, 0, 0};
   bool ok = false, even = false;
-  float march[3] = {0, 0, 0}, rows[3] = {0, 0, 0};
+  char work[3] = {0, 0, 0};
 };
-void add_march_work(const int n[3], BoxExtents* e);
+// That work over the boxes of a launch, in lanes.
+struct MarchWork {
+  float march[3] = {0, 0, 0}, rows[3] = {0, 0, 0};
+  void add_box(const int n[3]);
+  void add(const MarchWork& o) {
+    for (int d = 0; d < 3; ++d) { march[d] += o.march[d]; rows[d] += o.rows[d]; }
+  }
+  void compare(BoxExtents* e) const {
+    for (int d = 0; d < 3; ++d) e->work[d] = march[d] <= rows[d] ? 0 : march[d] <= 1.4f * rows[d] ? 1 : 2;
+  }
+};
 // A launch may cover the box tables of several independent solves (batched and served
 // solves): each solve's table is one segment of the launch's row space.  norms and scales
 // of a row live at index slot + DRow::solve.

@@ -534,7 +534,7 @@ bool use_int(const SegList& L) {
 // taken): half-sweep of 64^3 in boxes of 4^3 9.2 / 14.3, 8 x 4 x 4 6.2 / 8.1, 8 x 2 x 64 6.2 / 12.6, 4 x 8 x 8 9.3 / 7.3, 8^3
 // 6.2 / 4.9; residual of 32^3 in 2^3 14.5 / 24.7, 128^3 in 32 x 2 x 128 37 / 64, 8^3 123 / 63; restriction of
 // 64^3 in 4^3 21 / 55, 128^3 in 8^3 67 / 82, 16^3 35 / 41, 8 x 16 x 8 67 / 49.
-void add_march_work(const int n[3], BoxExtents* e) {
+void MarchWork::add_box(const int n[3]) {
   auto lanes = [](int width, int cells, int lo, int hi) {  // of a row's group in the row kernels
     int g = lo;
     while (g < hi && g * cells < width) g *= 2;
@@ -548,12 +548,12 @@ void add_march_work(const int n[3], BoxExtents* e) {
   auto up = [](int a, int b) { return (a + b - 1) / b * b; };
   const float nz = (float)n[2];
   const int one = busy(n[1]), two = busy(n[1] / 2);
-  e->march[MARCH_HALF] += nz * 32 * warps(n[1]) * (one == 1 && pp >= 8 ? 1.3f : 1.f);
-  e->rows[MARCH_HALF] += nz * n[1] * up(pp, lanes(n[0], 4, 4, 16)) * (one > 2 ? 1.25f : 1.f);
-  e->march[MARCH_RESIDUAL] += nz * 64 * warps(n[1]) * (one == 1 ? 2.1f : one == 2 ? 1.15f : 1.f);
-  e->rows[MARCH_RESIDUAL] += nz * n[1] * up(n[0], 32) * (one > 2 ? 1.25f : 1.f);
-  e->march[MARCH_RESTRICT] += nz * 32 * warps(n[1] / 2) * (two == 1 ? 1.6f : two == 2 ? 1.15f : 1.f);
-  e->rows[MARCH_RESTRICT] += nz * (n[1] / 2) * up(pp, lanes(n[0], 2, 8, 32)) * (two > 2 ? 1.25f : 1.f);
+  march[MARCH_HALF] += nz * 32 * warps(n[1]) * (one == 1 && pp >= 8 ? 1.3f : 1.f);
+  rows[MARCH_HALF] += nz * n[1] * up(pp, lanes(n[0], 4, 4, 16)) * (one > 2 ? 1.25f : 1.f);
+  march[MARCH_RESIDUAL] += nz * 64 * warps(n[1]) * (one == 1 ? 2.1f : one == 2 ? 1.15f : 1.f);
+  rows[MARCH_RESIDUAL] += nz * n[1] * up(n[0], 32) * (one > 2 ? 1.25f : 1.f);
+  march[MARCH_RESTRICT] += nz * 32 * warps(n[1] / 2) * (two == 1 ? 1.6f : two == 2 ? 1.15f : 1.f);
+  rows[MARCH_RESTRICT] += nz * (n[1] / 2) * up(pp, lanes(n[0], 2, 8, 32)) * (two > 2 ? 1.25f : 1.f);
 }
 
 // Where the work is against them, the marching kernels still win while their blocks are few and short
@@ -566,13 +566,13 @@ void add_march_work(const int n[3], BoxExtents* e) {
 bool march_pays(const SegList& L, int op, bool direct) {
   const BoxExtents& e = L.ext;
   if (!e.ok || (op != MARCH_RESIDUAL && !e.even)) return false;
-  if (e.march[op] <= e.rows[op]) return true;
+  if (!e.work[op]) return true;
   if (op == MARCH_RESIDUAL) return false;
   int zc;
   const dim3 g = march_grid(L, &zc, op == MARCH_RESTRICT ? 2 : 1);
   const long long blocks = (long long)g.x * g.y, sms = num_sms();
   if (op == MARCH_HALF) return std::min(zc, e.n[2]) <= 4 && blocks <= (direct ? 7 : 2) * sms;
-  return blocks <= (direct ? 4 : 2) * sms || (direct && e.march[op] <= 1.4f * e.rows[op]);
+  return blocks <= (direct ? 4 : 2) * sms || (direct && e.work[op] == 1);
 }
 
 cudaError_t launch_half_march(const SegList& L, int mode, int color, unsigned long long* norms,

@@ -353,8 +353,9 @@ OpTable upload_table(Ctx& c, const std::vector<DRow>& rows, long long nrows, cud
     for (int d = 0; d < 3; ++d) t.ext.n[d] = std::max(t.ext.n[d], R.n[d]);
     t.ext.ok = t.ext.ok && R.n[0] <= kMarchMaxX;
     t.ext.even = t.ext.even && R.n[0] % 2 == 0;
-    add_march_work(R.n, &t.ext);
+    t.work.add_box(R.n);
   }
+  t.work.compare(&t.ext);
   if (!rows.empty()) t.d = c.upload(rows.data(), rows.size() * sizeof(DRow), s);
   return t;
 }

@@ -159,6 +159,7 @@ struct OpTable {
   bool direct = false;  // rows carry box-face reads (DRow::nbd / nbf)
   int width = 0;        // widest box x-extent of the rows
   BoxExtents ext;       // largest box extents
+  MarchWork work;       // of its rows
   const DRow* rows() const { return d ? (const DRow*)d->p : nullptr; }
 };
 
