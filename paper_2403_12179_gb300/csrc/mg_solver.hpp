@@ -108,8 +108,8 @@ struct Hierarchy {
 std::shared_ptr<Hierarchy> get_hierarchy(Ctx& c, FabObj& rhs, FabObj& phi, const mg_bc* bc, const SolveParams& p);
 // The tables that only a solve on its own launches from (whole sweeps, residual + restriction and coarse
 // cycle of one hierarchy), once per hierarchy, before its cycles are enqueued or captured: members of
-// batches go without (64^3 FP64 members: 74 KB each of 2.9 MB, and 0.4 of 4.1 ms for the first batch of
-// sixteen 32^3 mixed problems).
+// batches go without (64^3 FP64 members 3.59 -> 3.52 MB each; first batch of sixteen 32^3 mixed problems 4.0 ->
+// 3.4 ms).
 void prepare_alone(Ctx& c, Hierarchy& H);
 
 // One V-cycle for the hierarchy's problem from a zero guess: phi (the caller's level-0 fab,
